@@ -288,17 +288,38 @@ __device__ void lin_sweep_up(int K, const T *nh, const T *c1s, const T *ph, T *n
   }
 }
 
-// per-sample error e_s = |T - D|_p / |T|_p over the 36 components (FP64)
+// x^p and x^(1/p) for x >= 0.  The exponents 1 and 2 take no pow(): with 72
+// to 93 powers a sample on the FP64 pipe the error and seed kernels took 956
+// and 1540 us of a 6890 us training step (p = 1, K = 8, 65,536 samples).
+__device__ __forceinline__ double pow_p(double x, double p) {
+  return p == 1.0 ? x : (p == 2.0 ? x * x : pow(x, p));
+}
+__device__ __forceinline__ double root_p(double x, double p) {
+  return p == 1.0 ? x : (p == 2.0 ? sqrt(x) : pow(x, 1.0 / p));
+}
+
+// p-norms of T - D and of T over the 36 components (FP64)
 template <typename T>
-__device__ double lin_error(const double *Tg, const T *D, double p) {
+__device__ __forceinline__ void lin_norms(const double *Tg, const T *D, double p, double &nx, double &nt) {
   double num = 0.0, den = 0.0;
+#pragma unroll
   for (int i = 0; i < 6; ++i)
+#pragma unroll
     for (int j = 0; j < 6; ++j) {
-      const double x = Tg[6 * i + j] - double(sget(D, i, j)), y = Tg[6 * i + j];
-      num += pow(fabs(x), p);
-      den += pow(fabs(y), p);
+      const double y = Tg[6 * i + j];
+      num += pow_p(fabs(y - double(sget(D, i, j))), p);
+      den += pow_p(fabs(y), p);
     }
-  return pow(num, 1.0 / p) / pow(den, 1.0 / p);
+  nx = root_p(num, p);
+  nt = root_p(den, p);
+}
+
+// per-sample error e_s = |T - D|_p / |T|_p
+template <typename T>
+__device__ __forceinline__ double lin_error(const double *Tg, const T *D, double p) {
+  double nx, nt;
+  lin_norms(Tg, D, p, nx, nt);
+  return nx / nt;
 }
 
 template <typename T>
@@ -322,40 +343,70 @@ __global__ void k_lin_forward(int K, int64_t n, const double *C1, const double *
   }
 }
 
-// batch reduction of the errors: scal[0] = max e, scal[1] = (1/N) S^(1/q - 1)
-// with S = sum (e/max)^q, scal[2] = data term; also the penalty and J
-__global__ void k_lin_reduce(int K, int64_t n, const double *err, const double *v, double q, double penalty,
-                             double *scal, double *loss) {
-  __shared__ double red[1024];
+// Batch reduction of the errors, by the blocks that form them: block b leaves
+// its largest error m_b and S_b = sum (e / m_b)^q in part[2b], part[2b + 1];
+// the block that comes last (ticket) joins them in block order, so the result
+// does not depend on the order of arrival:
+//   scal[0] = m = max e, scal[1] = S^(1/q - 1) / n with S = sum (m_b / m)^q S_b,
+// and the loss (J, data term, penalty).  A block whose errors are all zero (or
+// NaN) has m_b = 0 and hands on their plain sum.  (One CTA over all errors, two
+// general powers a sample in a row, took 1815 us at 65,536 samples; the step
+// as a whole went from 6890 to 1837 us with this, the exact powers and the
+// parallel chain through the weights, and from 1637 to 173 us at 32 samples.)
+// All threads of all blocks call it; blockDim.x = kLvlThreads.
+constexpr int kLvlThreads = 128;
+__device__ __forceinline__ double block_max(double x, double *red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
+  x = red[0];
+  for (int w = 1; w < kLvlThreads / 32; ++w) x = fmax(x, red[w]);
+  return x;
+}
+__device__ __forceinline__ double block_sum(double x, double *red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
+  __syncthreads();
+  x = red[0];
+  for (int w = 1; w < kLvlThreads / 32; ++w) x += red[w];
+  return x;
+}
+__device__ void lin_reduce(int64_t n, double e, double q, double penalty, double *part, double *scal,
+                           double *loss) {
+  __shared__ double red[kLvlThreads / 32];
+  __shared__ bool last;
   const int t = threadIdx.x;
-  double m = 0.0;
-  for (int64_t s = t; s < n; s += blockDim.x) m = fmax(m, err[s]);
-  red[t] = m;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (t < o) red[t] = fmax(red[t], red[t + o]);
-    __syncthreads();
+  const double mb = block_max(e, red);
+  const double Sb = block_sum(mb > 0.0 ? pow(e / mb, q) : e, red);
+  if (t == 0) {
+    part[2 * blockIdx.x] = mb;
+    part[2 * blockIdx.x + 1] = Sb;
+    __threadfence();
+    last = atomicAdd(reinterpret_cast<unsigned *>(scal + 4), 1u) == gridDim.x - 1;
   }
-  m = red[0];
   __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double m = 0.0;
+  for (unsigned b = t; b < gridDim.x; b += kLvlThreads) m = fmax(m, part[2 * b]);
+  m = block_max(m, red);
   double acc = 0.0;
   if (m > 0.0)
-    for (int64_t s = t; s < n; s += blockDim.x) acc += pow(err[s] / m, q);
-  red[t] = acc;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (t < o) red[t] += red[t + o];
-    __syncthreads();
-  }
+    for (unsigned b = t; b < gridDim.x; b += kLvlThreads) {
+      const double mm = part[2 * b];
+      acc += mm > 0.0 ? pow(mm / m, q) * part[2 * b + 1] : part[2 * b + 1];
+    }
+  const double S = block_sum(acc, red);
   if (t == 0) {
-    const double S = red[0];
-    double wsum = 0.0;
-    for (int j = 0; j < (1 << K); ++j) wsum += v[j] > 0.0 ? v[j] : 0.0;
+    const double wsum = scal[5];
     const double data = m > 0.0 ? m * pow(S, 1.0 / q) / double(n) : 0.0;
     const double pen = penalty * (wsum - 1.0) * (wsum - 1.0);
     scal[0] = m;
     scal[1] = m > 0.0 ? pow(S, 1.0 / q - 1.0) / double(n) : 0.0;
-    scal[2] = data;
     loss[0] = data + pen;
     loss[1] = data;
     loss[2] = pen;
@@ -367,7 +418,6 @@ __global__ void k_lin_reduce(int K, int64_t n, const double *err, const double *
 // warp's loads of one component are contiguous); one launch per level and
 // direction, a 2-D grid of (sample blocks, nodes of the level), so every
 // block serves one node and reduces its gradient terms before one atomic add.
-constexpr int kLvlThreads = 128;
 
 template <typename T>
 __device__ __forceinline__ void lvl_load(const T *X, int p, int64_t n, int64_t s, T out[21]) {
@@ -387,22 +437,54 @@ __device__ __forceinline__ void phase_packed(const double *C, T out[21]) {
     for (int j = i; j < 6; ++j) out[sidx(i, j)] = T(0.5 * (C[6 * i + j] + C[6 * j + i]));
 }
 
-// normalised normals and c1 of every node in the laminate precision (one CTA)
+// Set-up of a training pass, one launch:
+//  block 0   the normalised normals and c1 of every node in the laminate precision;
+//  block 1   zeroes the gradient sums and the scalars (nz doubles from acc),
+//            and adds up the weights, in leaf order, into scal[5] (one thread;
+//            the additions run beside block 0's levels: in the chain through
+//            the weights they would stand alone);
+//  others    the phase stiffnesses of every sample, packed, in the laminate
+//            precision: PH[phase][21][sample] (converted once instead of by
+//            every bottom laminate).
+// (Three launches before, 11 us of kernels and two gaps more at 32 samples.)
+constexpr int kSetupThreads = 256;
 template <typename T>
-__global__ void k_lvl_const(int K, const double *normals, const double *v, T *nh, T *c1s) {
+__global__ void __launch_bounds__(kSetupThreads)
+    k_lvl_setup(int K, int64_t n, const double *normals, const double *v, const double *C1, const double *C2, T *nh,
+                T *c1s, T *PH, double *acc, int nz, double *scal) {
   __shared__ double Wt[2 * (1 << kLinMaxK)];
   const int N = (1 << K) - 1, L = 1 << K, t = threadIdx.x;
-  for (int pp = t; pp < N; pp += blockDim.x) {
+  if (blockIdx.x > 1) {
+    const int64_t s = int64_t(blockIdx.x - 2) * kSetupThreads + t;
+    if (s >= n) return;
+    T a[21], b[21];
+    phase_packed(C1 + 36 * s, a);
+    phase_packed(C2 + 36 * s, b);
+    lvl_store(PH, 0, n, s, a);
+    lvl_store(PH, 1, n, s, b);
+    return;
+  }
+  for (int j = t; j < L; j += kSetupThreads) Wt[j] = v[j] > 0.0 ? v[j] : 0.0;
+  if (blockIdx.x == 1) {
+    for (int i = t; i < nz; i += kSetupThreads) acc[i] = 0.0;
+    __syncthreads();
+    if (t == 0) {
+      double w = 0.0;
+      for (int j = 0; j < L; ++j) w += Wt[j];
+      scal[5] = w;
+    }
+    return;
+  }
+  for (int pp = t; pp < N; pp += kSetupThreads) {
     const double x = normals[3 * pp], y = normals[3 * pp + 1], z = normals[3 * pp + 2];
     const double il = 1.0 / sqrt(x * x + y * y + z * z);
     nh[3 * pp] = T(x * il);
     nh[3 * pp + 1] = T(y * il);
     nh[3 * pp + 2] = T(z * il);
   }
-  for (int j = t; j < L; j += blockDim.x) Wt[j] = v[j] > 0.0 ? v[j] : 0.0;
   __syncthreads();
   for (int k = K; k >= 1; --k) {
-    for (int i = t; i < (1 << (k - 1)); i += blockDim.x) {
+    for (int i = t; i < (1 << (k - 1)); i += kSetupThreads) {
       const int pp = (1 << K) - (1 << k) + i;
       const int pc = (1 << K) - (1 << (k + 1)) + 2 * i;
       const double a = k == K ? Wt[2 * i] : Wt[L + pc], b = k == K ? Wt[2 * i + 1] : Wt[L + pc + 1];
@@ -412,19 +494,6 @@ __global__ void k_lvl_const(int K, const double *normals, const double *v, T *nh
     }
     __syncthreads();
   }
-}
-
-// the phase stiffnesses of every sample, packed, in the laminate precision:
-// PH[phase][21][sample] (converted once instead of by every bottom laminate)
-template <typename T>
-__global__ void k_lvl_phases(int64_t n, const double *C1, const double *C2, T *PH) {
-  const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  T a[21], b[21];
-  phase_packed(C1 + 36 * s, a);
-  phase_packed(C2 + 36 * s, b);
-  lvl_store(PH, 0, n, s, a);
-  lvl_store(PH, 1, n, s, b);
 }
 
 template <typename T>
@@ -447,41 +516,51 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_fwd(int K, int k, int64_t n
   lvl_store(NS, pp, n, s, out);
 }
 
-// per-sample error from the root column
+// per-sample error from the root column, and the batch reduction
 template <typename T>
-__global__ void k_lvl_err(int K, int64_t n, const T *NS, const double *Ct, double p, double *err) {
-  const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  T D[21];
-  lvl_load(NS, (1 << K) - 2, n, s, D);
-  err[s] = lin_error<T>(Ct + 36 * s, D, p);
+__global__ void __launch_bounds__(kLvlThreads) k_lvl_err(int K, int64_t n, const T *NS, const double *Ct, double p,
+                                                         double q, double penalty, double *err, double *part,
+                                                         double *scal, double *loss) {
+  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
+  double e = 0.0;
+  if (s < n) {
+    T D[21];
+    lvl_load(NS, (1 << K) - 2, n, s, D);
+    e = lin_error<T>(Ct + 36 * s, D, p);
+    err[s] = e;
+  }
+  lin_reduce(n, e, q, penalty, part, scal, loss);
 }
 
 // dJ/dD at the root: (1/N) S^(1/q-1) (e_s/m)^(q-1) de_s/dD
 template <typename T>
-__global__ void k_lvl_seed(int K, int64_t n, const T *NS, const double *Ct, double p, double q, const double *err,
-                           const double *scal, T *GA) {
-  const int64_t s = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void lin_seed(const double *Tg, const T *D, double p, double q, double e,
+                                         const double *scal, T G[21]) {
+  const double m = scal[0];
+  const double coef = (m > 0.0 && e > 0.0) ? scal[1] * pow(e / m, q - 1.0) : 0.0;
+  double nx, nt;
+  lin_norms(Tg, D, p, nx, nt);
+  const double f = p == 1.0 ? 1.0 : pow(nx, 1.0 - p);
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = i; j < 6; ++j) {
+      const double x = Tg[6 * i + j] - double(sget(D, i, j));
+      const double sg = x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0);
+      const double xp = p == 1.0 ? 1.0 : (p == 2.0 ? fabs(x) : pow(fabs(x), p - 1.0));
+      const double de = nx > 0.0 ? -sg * xp * f / nt : 0.0;
+      G[sidx(i, j)] = T(coef * de);
+    }
+}
+template <typename T>
+__global__ void __launch_bounds__(kLvlThreads) k_lvl_seed(int K, int64_t n, const T *NS, const double *Ct, double p,
+                                                          double q, const double *err, const double *scal, T *GA) {
+  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
   if (s >= n) return;
   const int root = (1 << K) - 2;
   T D[21], G[21];
   lvl_load(NS, root, n, s, D);
-  const double m = scal[0], e = err[s];
-  const double coef = (m > 0.0 && e > 0.0) ? scal[1] * pow(e / m, q - 1.0) : 0.0;
-  const double *Tg = Ct + 36 * s;
-  double num = 0.0, den = 0.0;
-  for (int i = 0; i < 36; ++i) {
-    num += pow(fabs(Tg[i] - double(sget(D, i / 6, i % 6))), p);
-    den += pow(fabs(Tg[i]), p);
-  }
-  const double nx = pow(num, 1.0 / p), nt = pow(den, 1.0 / p);
-  for (int i = 0; i < 6; ++i)
-    for (int j = i; j < 6; ++j) {
-      const double x = Tg[6 * i + j] - double(sget(D, i, j));
-      const double sg = x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0);
-      const double de = nx > 0.0 ? -sg * pow(fabs(x), p - 1.0) * pow(nx, 1.0 - p) / nt : 0.0;
-      G[sidx(i, j)] = T(coef * de);
-    }
+  lin_seed(Ct + 36 * s, D, p, q, err[s], scal, G);
   lvl_store(GA, root, n, s, G);
 }
 
@@ -530,13 +609,17 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_bwd(int K, int k, int64_t n
   }
 }
 
-// the chain through the weights (c1 = W_1 / W, w = <v>_+, penalty) and the
-// normalisation of the normals; one thread
-__global__ void k_lin_finish(int K, const double *normals, const double *v, double penalty, const double *gnh,
-                             const double *gc1, double *grad_n, double *grad_v) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int N = (1 << K) - 1, L = 1 << K;
-  for (int pp = 0; pp < N; ++pp) {
+// The chain through the weights (c1 = W_1 / W, w = <v>_+, penalty) and the
+// normalisation of the normals: one CTA, the nodes of a level on its threads,
+// subtree weights and their adjoints in shared memory.  (One thread with both
+// in local memory took 928 us at K = 8.)
+__global__ void __launch_bounds__(1 << kLinMaxK)
+    k_lin_finish(int K, const double *normals, const double *v, double penalty, const double *gnh,
+                 const double *gc1, const double *scal, double *grad_n, double *grad_v) {
+  __shared__ double Wt[2 << kLinMaxK], gW[1 << kLinMaxK];  // weights: leaves [0, L), nodes [L, L + N)
+  const int N = (1 << K) - 1, L = 1 << K, t = threadIdx.x;
+  for (int j = t; j < L; j += blockDim.x) Wt[j] = v[j] > 0.0 ? v[j] : 0.0;
+  for (int pp = t; pp < N; pp += blockDim.x) {
     const double x = normals[3 * pp], y = normals[3 * pp + 1], z = normals[3 * pp + 2];
     const double len = sqrt(x * x + y * y + z * z);
     const double nh[3] = {x / len, y / len, z / len};
@@ -544,56 +627,33 @@ __global__ void k_lin_finish(int K, const double *normals, const double *v, doub
     const double gd = g[0] * nh[0] + g[1] * nh[1] + g[2] * nh[2];
     for (int c = 0; c < 3; ++c) grad_n[3 * pp + c] = (g[c] - gd * nh[c]) / len;
   }
-  // subtree weights of every node, bottom level first
-  double Wn[(1 << kLinMaxK) - 1];
-  double wsum = 0.0;
-  for (int j = 0; j < L; ++j) wsum += v[j] > 0.0 ? v[j] : 0.0;
-  for (int k = K; k >= 1; --k)
-    for (int i = 0; i < (1 << (k - 1)); ++i) {
-      const int pp = (1 << K) - (1 << k) + i;
-      double a, b;
-      if (k == K) {
-        a = v[2 * i] > 0.0 ? v[2 * i] : 0.0;
-        b = v[2 * i + 1] > 0.0 ? v[2 * i + 1] : 0.0;
-      } else {
-        const int pc = (1 << K) - (1 << (k + 1)) + 2 * i;
-        a = Wn[pc];
-        b = Wn[pc + 1];
-      }
-      Wn[pp] = a + b;
-    }
+  __syncthreads();
+  // children of node i of level k: slots ch, ch + 1 of Wt
+  auto child = [&](int k, int i) { return k == K ? 2 * i : L + (1 << K) - (1 << (k + 1)) + 2 * i; };
+  for (int k = K; k >= 1; --k) {
+    for (int i = t; i < (1 << (k - 1)); i += blockDim.x)
+      Wt[L + (1 << K) - (1 << k) + i] = Wt[child(k, i)] + Wt[child(k, i) + 1];
+    __syncthreads();
+  }
   // adjoints of the subtree weights, root first
-  double gW[(1 << kLinMaxK) - 1];
-  gW[N - 1] = 2.0 * penalty * (wsum - 1.0);
-  for (int k = 1; k <= K; ++k)
-    for (int i = 0; i < (1 << (k - 1)); ++i) {
-      const int pp = (1 << K) - (1 << k) + i;
-      const double W = Wn[pp];
-      double a, b;
-      if (k == K) {
-        a = v[2 * i] > 0.0 ? v[2 * i] : 0.0;
-        b = v[2 * i + 1] > 0.0 ? v[2 * i + 1] : 0.0;
-      } else {
-        const int pc = (1 << K) - (1 << (k + 1)) + 2 * i;
-        a = Wn[pc];
-        b = Wn[pc + 1];
-      }
+  if (t == 0) gW[N - 1] = 2.0 * penalty * (scal[5] - 1.0);
+  __syncthreads();
+  for (int k = 1; k <= K; ++k) {
+    for (int i = t; i < (1 << (k - 1)); i += blockDim.x) {
+      const int pp = (1 << K) - (1 << k) + i, ch = child(k, i);
+      const double W = Wt[L + pp], a = Wt[ch], b = Wt[ch + 1];
       const double dL = W > 0.0 ? gc1[pp] * b / (W * W) : 0.0;   // d c1 / d W_1 = W_2 / W^2
       const double dR = W > 0.0 ? -gc1[pp] * a / (W * W) : 0.0;  // d c1 / d W_2 = -W_1 / W^2
       if (k == K) {
-        grad_v[2 * i] = v[2 * i] > 0.0 ? gW[pp] + dL : 0.0;
-        grad_v[2 * i + 1] = v[2 * i + 1] > 0.0 ? gW[pp] + dR : 0.0;
+        grad_v[2 * i] = a > 0.0 ? gW[pp] + dL : 0.0;
+        grad_v[2 * i + 1] = b > 0.0 ? gW[pp] + dR : 0.0;
       } else {
-        const int pc = (1 << K) - (1 << (k + 1)) + 2 * i;
-        gW[pc] = gW[pp] + dL;
-        gW[pc + 1] = gW[pp] + dR;
+        gW[ch - L] = gW[pp] + dL;
+        gW[ch - L + 1] = gW[pp] + dR;
       }
     }
-}
-
-__global__ void k_lin_zero(double *x, int64_t n) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    x[i] = 0.0;
+    __syncthreads();
+  }
 }
 
 __global__ void k_amsgrad(int64_t n, double *x, const double *g, double *m, double *s, double *smax, double lr,
@@ -668,16 +728,17 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   if (nb > 2147483647u) return lin_fail("dmn_linear_loss_grad: batch too large");
   const int N = (1 << K) - 1;
   T *nh = consts, *c1s = consts + 3 * N;
-  k_lvl_const<T><<<1, 256, 0, st>>>(K, normals, v, nh, c1s);
-  k_lvl_phases<T><<<nb, kLvlThreads, 0, st>>>(n, C1, C2, PH);
+  const unsigned ns = unsigned((n + kSetupThreads - 1) / kSetupThreads);
+  k_lvl_setup<T><<<2 + ns, kSetupThreads, 0, st>>>(K, n, normals, v, C1, C2, nh, c1s, PH, gnh, 4 * N + 5, scal);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: set-up launch");
   for (int k = K; k >= 1; --k) {
     k_lvl_fwd<T><<<dim3(nb, 1u << (k - 1)), kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS);
     if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: forward level launch");
   }
-  k_lvl_err<T><<<nb, kLvlThreads, 0, st>>>(K, n, NS, Ct, p, err);
-  k_lin_reduce<<<1, 1024, 0, st>>>(K, n, err, v, q, penalty, scal, loss);
+  // the blocks' partial sums: in the adjoints' array, free until the seed, from an 8-byte boundary
+  double *part = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(GA) + 7) & ~uintptr_t(7));
+  k_lvl_err<T><<<nb, kLvlThreads, 0, st>>>(K, n, NS, Ct, p, q, penalty, err, part, scal, loss);
   k_lvl_seed<T><<<nb, kLvlThreads, 0, st>>>(K, n, NS, Ct, p, q, err, scal, GA);
   if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: loss launch");
   for (int k = 1; k <= K; ++k) {
@@ -722,9 +783,6 @@ extern "C" dmn_status dmn_linear_loss_grad(dmn_stream stream, int32_t K, int64_t
   const int N = (1 << K) - 1;
   double *err = d_work, *gnh = d_work + n_samples, *gc1 = gnh + 3 * N, *scal = gc1 + N;
   double *consts = scal + 8, *nodes = consts + 4 * N;
-  k_lin_zero<<<8, 256, 0, st>>>(gnh, 4 * N + 8);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: set-up launch");
   const int64_t cells = int64_t(21) * N * n_samples, ph = int64_t(42) * n_samples;
   dmn_status s;
   if (precision == DMN_LIN_FP64)
@@ -736,8 +794,9 @@ extern "C" dmn_status dmn_linear_loss_grad(dmn_stream stream, int32_t K, int64_t
                               d_loss, reinterpret_cast<float *>(consts), f, f + ph, f + ph + cells, gnh, gc1);
   }
   if (s != DMN_OK) return s;
-  k_lin_finish<<<1, 32, 0, st>>>(K, d_normals, d_v, penalty, gnh, gc1, d_grad_n, d_grad_v);
-  if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: finish launch");
+  k_lin_finish<<<1, 1 << kLinMaxK, 0, st>>>(K, d_normals, d_v, penalty, gnh, gc1, scal, d_grad_n, d_grad_v);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: finish launch");
   return DMN_OK;
 }
 
