@@ -60,9 +60,10 @@ dmn_status dmn_linear_forward(dmn_stream stream, int32_t K, int64_t n_samples, c
  *              DMN_LIN_FP64, floats for DMN_LIN_FP32), 2.8 GB at K = 8,
  *              65,536 samples, FP32
  * The gradient is exact for the forward computation (reverse mode through
- * every laminate).  Level-synchronous over the batch: set-up, K forward
- * launches, errors with the batch reduction, seed, K backward launches, the
- * chain through the weights (2K + 4 launches).
+ * every laminate).  Level-synchronous over the batch: set-up, the forward
+ * levels, errors with the batch reduction, seed, the backward levels, the
+ * chain through the weights; FP32 laminates take two levels a launch (K + 4
+ * launches for even K, K + 5 for odd), FP64 ones one (2K + 4).
  */
 dmn_status dmn_linear_loss_grad(dmn_stream stream, int32_t K, int64_t n_samples, const double *d_C1,
                                 const double *d_C2, const double *d_Ctarget, const double *d_normals,

@@ -652,6 +652,113 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_bwd(int K, int k, int64_t n
   }
 }
 
+// Two levels in one pass, FP32 laminates: a thread takes node j of level k and
+// its two children (level k + 1) of one sample, so that the children's
+// stiffnesses go to the parent, and the parent's adjoints to the children, in
+// registers.  LEAF: the children are bottom laminates (their children the
+// phases).  Of the 12 words of 21 a parent and its children move in two
+// launches (forward: 4 in, 2 in again, 3 out) the pass keeps 7; of the reverse
+// mode's 19 (9 + 2 x 5, no adjoints below the bottom) 15.  K = 8, 65,536
+// samples: forward 480 -> 500 us (its bottom pair spills at four CTAs per SM),
+// reverse 890 -> 745, the step 1714 -> 1493; 32 samples (half the launches):
+// 172 -> 155 us.
+template <bool LEAF, typename T>
+__global__ void __launch_bounds__(kLvlThreads, 4) k_lvl_fwd2(int K, int k, int64_t n, const T *PH, const T *nh,
+                                                          const T *c1s, T *NS) {
+  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
+  if (s >= n) return;
+  const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j, pc = (1 << K) - (1 << (k + 1)) + 2 * j;
+  const int pg = (1 << K) - (1 << (k + 2)) + 4 * j;  // grandchildren
+  T X[21], Y[21];
+  {
+    T CL[21], CR[21];
+    lvl_load(LEAF ? PH : NS, LEAF ? 0 : pg, n, s, CL);
+    lvl_load(LEAF ? PH : NS, LEAF ? 1 : pg + 1, n, s, CR);
+    const T nn[3] = {nh[3 * pc], nh[3 * pc + 1], nh[3 * pc + 2]};
+    lam_forward(CL, CR, nn, c1s[pc], X);
+    lvl_store(NS, pc, n, s, X);
+  }
+  {
+    T CL[21], CR[21];
+    lvl_load(LEAF ? PH : NS, LEAF ? 0 : pg + 2, n, s, CL);
+    lvl_load(LEAF ? PH : NS, LEAF ? 1 : pg + 3, n, s, CR);
+    const T nn[3] = {nh[3 * pc + 3], nh[3 * pc + 4], nh[3 * pc + 5]};
+    lam_forward(CL, CR, nn, c1s[pc + 1], Y);
+    lvl_store(NS, pc + 1, n, s, Y);
+  }
+  T out[21];
+  const T nn[3] = {nh[3 * pp], nh[3 * pp + 1], nh[3 * pp + 2]};
+  lam_forward(X, Y, nn, c1s[pp], out);
+  lvl_store(NS, pp, n, s, out);
+}
+
+template <bool LEAF, typename T>
+__global__ void __launch_bounds__(kLvlThreads, 3) k_lvl_bwd2(int K, int k, int64_t n, const T *PH, const T *nh,
+                                                          const T *c1s, const T *NS, T *GA, double *gnh,
+                                                          double *gc1) {
+  __shared__ T red[3][4][kLvlThreads / 32];
+  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
+  const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j, pc = (1 << K) - (1 << (k + 1)) + 2 * j;
+  const int pg = (1 << K) - (1 << (k + 2)) + 4 * j;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // sums of dJ/dn and dJ/dc1 over the warp's samples
+  auto warp_sums = [&](int node, const T gn[3], T g1) {
+    T r[4] = {gn[0], gn[1], gn[2], g1};
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) r[c] += __shfl_down_sync(0xffffffffu, r[c], o);
+    if (lane == 0)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) red[node][c][warp] = r[c];
+  };
+  T G[21], GR[21];
+  {
+    T gn[3] = {T(0), T(0), T(0)}, g1 = T(0);
+    if (s < n) {
+      T CL[21], CR[21], GL[21];
+      lvl_load(NS, pc, n, s, CL);
+      lvl_load(NS, pc + 1, n, s, CR);
+      lvl_load(GA, pp, n, s, G);
+      const T nn[3] = {nh[3 * pp], nh[3 * pp + 1], nh[3 * pp + 2]};
+      lam_backward<true>(CL, CR, nn, c1s[pp], G, GL, GR, gn, g1);
+#pragma unroll
+      for (int q = 0; q < 21; ++q) G[q] = GL[q];
+    }
+    warp_sums(0, gn, g1);
+  }
+#pragma unroll 1
+  for (int c = 0; c < 2; ++c) {
+    T gn[3] = {T(0), T(0), T(0)}, g1 = T(0);
+    if (s < n) {
+      T CL[21], CR[21];
+      lvl_load(LEAF ? PH : NS, LEAF ? 0 : pg + 2 * c, n, s, CL);
+      lvl_load(LEAF ? PH : NS, LEAF ? 1 : pg + 2 * c + 1, n, s, CR);
+      const int p = pc + c;
+      const T nn[3] = {nh[3 * p], nh[3 * p + 1], nh[3 * p + 2]};
+      if (LEAF) {
+        T *none = nullptr;
+        lam_backward<false>(CL, CR, nn, c1s[p], G, none, none, gn, g1);
+      } else {
+        T HL[21], HR[21];
+        lam_backward<true>(CL, CR, nn, c1s[p], G, HL, HR, gn, g1);
+        lvl_store(GA, pg + 2 * c, n, s, HL);
+        lvl_store(GA, pg + 2 * c + 1, n, s, HR);
+      }
+#pragma unroll
+      for (int q = 0; q < 21; ++q) G[q] = GR[q];
+    }
+    warp_sums(1 + c, gn, g1);
+  }
+  __syncthreads();
+  if (threadIdx.x < 12) {
+    const int node = threadIdx.x >> 2, c = threadIdx.x & 3, p = node == 0 ? pp : pc + node - 1;
+    T acc = T(0);
+    for (int w = 0; w < kLvlThreads / 32; ++w) acc += red[node][c][w];
+    atomicAdd(c < 3 ? gnh + 3 * p + c : gc1 + p, double(acc));
+  }
+}
+
 // The chain through the weights (c1 = W_1 / W, w = <v>_+, penalty) and the
 // normalisation of the normals: one CTA, the nodes of a level on its threads,
 // subtree weights and their adjoints in shared memory.  (One thread with both
@@ -773,21 +880,39 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   T *nh = consts, *c1s = consts + 3 * N;
   const unsigned ns = unsigned((n + kSetupThreads - 1) / kSetupThreads);
   k_lvl_setup<T><<<2 + ns, kSetupThreads, 0, st>>>(K, n, normals, v, C1, C2, nh, c1s, PH, gnh, 4 * N + 5, scal);
+  // FP32: pairs of levels from the bottom (FP64 laminates: 251 registers for one
+  // level, and bound by the FP64 pipe, so one level a launch)
+  int k = K;
+  if constexpr (sizeof(T) == 4)
+    for (; k >= 2; k -= 2) {
+      const dim3 grid(nb, 1u << (k - 2));
+      if (k == K) k_lvl_fwd2<true><<<grid, kLvlThreads, 0, st>>>(K, k - 1, n, PH, nh, c1s, NS);
+      else k_lvl_fwd2<false><<<grid, kLvlThreads, 0, st>>>(K, k - 1, n, PH, nh, c1s, NS);
+    }
+  for (; k >= 1; --k) k_lvl_fwd<T><<<dim3(nb, 1u << (k - 1)), kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: set-up launch");
-  for (int k = K; k >= 1; --k) {
-    k_lvl_fwd<T><<<dim3(nb, 1u << (k - 1)), kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS);
-    if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: forward level launch");
-  }
+  if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: forward level launch");
   // the blocks' partial sums: in the adjoints' array, free until the seed, from an 8-byte boundary
   double *part = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(GA) + 7) & ~uintptr_t(7));
   k_lvl_err<T><<<nb, kLvlThreads, 0, st>>>(K, n, NS, Ct, p, q, penalty, err, part, scal, loss);
   k_lvl_seed<T><<<nb, kLvlThreads, 0, st>>>(K, n, NS, Ct, p, q, err, scal, GA);
   if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: loss launch");
-  for (int k = 1; k <= K; ++k) {
-    k_lvl_bwd<T><<<dim3(nb, 1u << (k - 1)), kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: backward level launch");
+  // the same pairs, root first
+  k = 1;
+  if constexpr (sizeof(T) == 4) {
+    if (K & 1) {
+      k_lvl_bwd<T><<<dim3(nb, 1), kLvlThreads, 0, st>>>(K, 1, n, PH, nh, c1s, NS, GA, gnh, gc1);
+      k = 2;
+    }
+    for (; k < K; k += 2) {
+      const dim3 grid(nb, 1u << (k - 1));
+      if (k + 1 == K) k_lvl_bwd2<true><<<grid, kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
+      else k_lvl_bwd2<false><<<grid, kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
+    }
   }
+  for (; k <= K; ++k)
+    k_lvl_bwd<T><<<dim3(nb, 1u << (k - 1)), kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
+  if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: backward level launch");
   return DMN_OK;
 }
 
