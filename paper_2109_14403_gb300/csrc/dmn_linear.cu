@@ -218,31 +218,32 @@ __device__ __forceinline__ void lam_backward(const T *CL, const T *CR, const T n
   gn[0] = gB[0][0] + r * (gB[4][2] + gB[5][1]);
   gn[1] = gB[1][1] + r * (gB[3][2] + gB[5][0]);
   gn[2] = gB[2][2] + r * (gB[3][1] + gB[4][0]);
-  if (!kids) return;
-  T BQ[6][3];
+  if constexpr (kids) {
+    T BQ[6][3];
 #pragma unroll
-  for (int a = 0; a < 6; ++a)
+    for (int a = 0; a < 6; ++a)
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      const T col[3] = {Q[0][f], Q[1][f], Q[2][f]};
-      // BQ[4][1]: two rounded products, each of which another entry has too (Q
-      // is symmetric: r n2 Q[0][1] in BQ[3][0], r n0 Q[1][2] in BQ[5][2])
-      BQ[a][f] = a == 4 && f == 1 ? sum_rn(col[0], B[4][0], col[2], B[4][2]) : row_bt(col, B, a);
-    }
+      for (int f = 0; f < 3; ++f) {
+        const T col[3] = {Q[0][f], Q[1][f], Q[2][f]};
+        // BQ[4][1]: two rounded products, each of which another entry has too (Q
+        // is symmetric: r n2 Q[0][1] in BQ[3][0], r n0 Q[1][2] in BQ[5][2])
+        BQ[a][f] = a == 4 && f == 1 ? sum_rn(col[0], B[4][0], col[2], B[4][2]) : row_bt(col, B, a);
+      }
 #pragma unroll
-  for (int i = 0; i < 6; ++i)
+    for (int i = 0; i < 6; ++i)
 #pragma unroll
-    for (int j = i; j < 6; ++j) {
-      const int q = sidx(i, j);
-      T ab = row_bt(A[i], B, j);
+      for (int j = i; j < 6; ++j) {
+        const int q = sidx(i, j);
+        T ab = row_bt(A[i], B, j);
 #pragma unroll
-      for (int f = 0; f < 3; ++f)
-        if (bnz(i, f)) ab = mad(A[j][f], B[i][f], ab);
-      ab = T(0.5) * ab;
-      const T bqb = row_bt(BQ[i], B, j);
-      GL[q] = c1 * G[q] - T(2) * cc * ab + cc * c2 * bqb;
-      GR[q] = c2 * G[q] + T(2) * cc * ab + cc * c1 * bqb;
-    }
+        for (int f = 0; f < 3; ++f)
+          if (bnz(i, f)) ab = mad(A[j][f], B[i][f], ab);
+        ab = T(0.5) * ab;
+        const T bqb = row_bt(BQ[i], B, j);
+        GL[q] = c1 * G[q] - T(2) * cc * ab + cc * c2 * bqb;
+        GR[q] = c2 * G[q] + T(2) * cc * ab + cc * c1 * bqb;
+      }
+  }
 }
 
 // shared-memory carving of dmn_linear_forward (T words): normals 3N, c1 N,
@@ -329,44 +330,53 @@ __device__ void lin_sweep_up(int K, const T *nh, const T *c1s, const T *ph, T *n
   }
 }
 
-// x^p and x^(1/p) for x >= 0.  The exponents 1 and 2 take no pow(): with 72
-// to 93 powers a sample on the FP64 pipe the error and seed kernels took 956
-// and 1540 us of a 6890 us training step (p = 1, K = 8, 65,536 samples).
+// x^p and x^(1/p) for x >= 0, MODE 1: p = 1, 2: p = 2, 0: any p.  The first two
+// take no pow(): with 72 to 93 powers a sample on the FP64 pipe the error and
+// seed kernels took 956 and 1540 us of a 6890 us training step (p = 1, K = 8,
+// 65,536 samples).  The mode is a template argument of the sums: a test of p in
+// every term is an FP64 comparison each.
+__host__ __device__ inline int pow_mode(double p) { return p == 1.0 ? 1 : (p == 2.0 ? 2 : 0); }
+template <int MODE>
 __device__ __forceinline__ double pow_p(double x, double p) {
-  return p == 1.0 ? x : (p == 2.0 ? x * x : pow(x, p));
+  return MODE == 1 ? x : (MODE == 2 ? x * x : pow(x, p));
 }
+template <int MODE>
 __device__ __forceinline__ double root_p(double x, double p) {
-  return p == 1.0 ? x : (p == 2.0 ? sqrt(x) : pow(x, 1.0 / p));
+  return MODE == 1 ? x : (MODE == 2 ? sqrt(x) : pow(x, 1.0 / p));
 }
 
-// p-norms of T - D and of T over the 36 components (FP64)
-template <typename T>
-__device__ __forceinline__ void lin_norms(const double *Tg, const T *D, double p, double &nx, double &nt) {
-  double num = 0.0, den = 0.0;
-#pragma unroll
+// x^q for x >= 0; a small whole q by repeated squaring (within a few ulp).
+// One FP64 pow() is a serial chain of some 8 us here, and a 32-sample step had
+// six of them in a row.
+__device__ __forceinline__ double pow_q(double x, double q) {
+  if (!(q >= 0.0 && q <= 64.0) || q != floor(q)) return pow(x, q);
+  double r = 1.0;
+  for (int k = int(q); k; k >>= 1, x *= x)
+    if (k & 1) r *= x;
+  return r;
+}
+
+// |x|_p of the 36 components f(i, j), six partial sums
+template <int MODE, typename F>
+__device__ __forceinline__ double lin_norm(double p, F f) {
+  double col[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll(MODE ? 6 : 1)
   for (int i = 0; i < 6; ++i)
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      const double y = Tg[6 * i + j];
-      num += pow_p(fabs(y - double(sget(D, i, j))), p);
-      den += pow_p(fabs(y), p);
-    }
-  nx = root_p(num, p);
-  nt = root_p(den, p);
+    for (int j = 0; j < 6; ++j) col[j] += pow_p<MODE>(fabs(f(i, j)), p);
+  return root_p<MODE>(((col[0] + col[1]) + (col[2] + col[3])) + (col[4] + col[5]), p);
 }
 
-// per-sample error e_s = |T - D|_p / |T|_p
-template <typename T>
+// per-sample error e_s = |T - D|_p / |T|_p (FP64)
+template <int MODE, typename T>
 __device__ __forceinline__ double lin_error(const double *Tg, const T *D, double p) {
-  double nx, nt;
-  lin_norms(Tg, D, p, nx, nt);
-  return nx / nt;
+  const double nx = lin_norm<MODE>(p, [&](int i, int j) { return Tg[6 * i + j] - double(sget(D, i, j)); });
+  return nx / lin_norm<MODE>(p, [&](int i, int j) { return Tg[6 * i + j]; });
 }
 
 template <typename T>
 __global__ void k_lin_forward(int K, int64_t n, const double *C1, const double *C2, const double *normals,
-                              const double *v, const double *Ctarget, double p, double *Cbar,
-                              double *err) {
+                              const double *v, double *Cbar) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *sm = reinterpret_cast<T *>(smem_raw);
   const LinLayout L = lin_layout(K);
@@ -377,9 +387,7 @@ __global__ void k_lin_forward(int K, int64_t n, const double *C1, const double *
     __syncthreads();
     lin_sweep_up<T>(K, sm + L.nh, sm + L.c1, sm + L.ph, sm + L.ns);
     const T *D = sm + L.ns + 21 * root;
-    if (Cbar)
-      for (int q = threadIdx.x; q < 36; q += blockDim.x) Cbar[36 * s + q] = double(sget(D, q / 6, q % 6));
-    if (err && threadIdx.x == 0) err[s] = lin_error<T>(Ctarget + 36 * s, D, p);
+    for (int q = threadIdx.x; q < 36; q += blockDim.x) Cbar[36 * s + q] = double(sget(D, q / 6, q % 6));
     __syncthreads();
   }
 }
@@ -422,7 +430,7 @@ __device__ void lin_reduce(int64_t n, double e, double q, double penalty, double
   __shared__ bool last;
   const int t = threadIdx.x;
   const double mb = block_max(e, red);
-  const double Sb = block_sum(mb > 0.0 ? pow(e / mb, q) : e, red);
+  const double Sb = block_sum(mb > 0.0 ? pow_q(e / mb, q) : e, red);
   if (t == 0) {
     part[2 * blockIdx.x] = mb;
     part[2 * blockIdx.x + 1] = Sb;
@@ -439,15 +447,16 @@ __device__ void lin_reduce(int64_t n, double e, double q, double penalty, double
   if (m > 0.0)
     for (unsigned b = t; b < gridDim.x; b += kLvlThreads) {
       const double mm = part[2 * b];
-      acc += mm > 0.0 ? pow(mm / m, q) * part[2 * b + 1] : part[2 * b + 1];
+      acc += mm > 0.0 ? pow_q(mm / m, q) * part[2 * b + 1] : part[2 * b + 1];
     }
   const double S = block_sum(acc, red);
   if (t == 0) {
     const double wsum = scal[5];
-    const double data = m > 0.0 ? m * pow(S, 1.0 / q) / double(n) : 0.0;
+    const double root = m > 0.0 ? root_p<0>(S, q) / double(n) : 0.0;
+    const double data = m * root;
     const double pen = penalty * (wsum - 1.0) * (wsum - 1.0);
     scal[0] = m;
-    scal[1] = m > 0.0 ? pow(S, 1.0 / q - 1.0) / double(n) : 0.0;
+    scal[1] = m > 0.0 ? root / S : 0.0;
     loss[0] = data + pen;
     loss[1] = data;
     loss[2] = pen;
@@ -478,8 +487,30 @@ __device__ __forceinline__ void phase_packed(const double *C, T out[21]) {
     for (int j = i; j < 6; ++j) out[sidx(i, j)] = T(0.5 * (C[6 * i + j] + C[6 * j + i]));
 }
 
+// Slot of node pp's (level k) first child in an array of the leaves [0, L) and
+// the nodes [L, L + N); its second child follows
+__device__ __forceinline__ int child_slot(int K, int k, int pp) {
+  const int i = pp - ((1 << K) - (1 << k));
+  return k == K ? 2 * i : (2 << K) - (1 << (k + 1)) + 2 * i;
+}
+// level of node pp
+__device__ __forceinline__ int node_level(int K, int pp) { return 32 - __clz((1 << K) - pp - 1); }
+// the nodes' weights from the leaves' (slots as above); all threads of the
+// block, at least 2^(K-1) of them; a barrier before and after each level
+__device__ __forceinline__ void tree_weights(int K, int t, double *Wt) {
+  for (int k = K; k >= 1; --k) {
+    if (t < (1 << (k - 1))) {
+      const int pp = (1 << K) - (1 << k) + t, ch = child_slot(K, k, pp);
+      Wt[(1 << K) + pp] = Wt[ch] + Wt[ch + 1];
+    }
+    __syncthreads();
+  }
+}
+
 // Set-up of a training pass, one launch:
-//  block 0   the normalised normals and c1 of every node in the laminate precision;
+//  block 0   c1 of every node in the laminate precision (first half of the
+//            threads: the weights level by level, then all quotients at once)
+//            and the normalised normals (second half);
 //  block 1   zeroes the gradient sums and the scalars (nz doubles from acc),
 //            and adds up the weights, in leaf order, into scal[5] (one thread;
 //            the additions run beside block 0's levels: in the chain through
@@ -487,36 +518,38 @@ __device__ __forceinline__ void phase_packed(const double *C, T out[21]) {
 //  others    the phase stiffnesses of every sample, packed, in the laminate
 //            precision: PH[phase][21][sample] (converted once instead of by
 //            every bottom laminate).
-// (Three launches before, 11 us of kernels and two gaps more at 32 samples.)
-constexpr int kSetupThreads = 256;
+// Bound by the latency of FP64 division and square root: neither is in the
+// level loop.
+constexpr int kSetupThreads = 2 << kLinMaxK;
 template <typename T>
 __global__ void __launch_bounds__(kSetupThreads)
     k_lvl_setup(int K, int64_t n, const double *normals, const double *v, const double *C1, const double *C2, T *nh,
                 T *c1s, T *PH, double *acc, int nz, double *scal) {
   __shared__ double Wt[2 * (1 << kLinMaxK)];
   const int N = (1 << K) - 1, L = 1 << K, t = threadIdx.x;
+  constexpr int H = kSetupThreads / 2;
   if (blockIdx.x > 1) {
-    const int64_t s = int64_t(blockIdx.x - 2) * kSetupThreads + t;
-    if (s >= n) return;
-    T a[21], b[21];
-    phase_packed(C1 + 36 * s, a);
-    phase_packed(C2 + 36 * s, b);
-    lvl_store(PH, 0, n, s, a);
-    lvl_store(PH, 1, n, s, b);
+    const int64_t i = int64_t(blockIdx.x - 2) * H + (t & (H - 1)), ph = t / H;  // one phase a thread
+    if (i >= n) return;
+    T a[21];
+    phase_packed((ph ? C2 : C1) + 36 * i, a);
+    lvl_store(PH, int(ph), n, i, a);
     return;
   }
-  for (int j = t; j < L; j += kSetupThreads) Wt[j] = v[j] > 0.0 ? v[j] : 0.0;
+  if (t < L) Wt[t] = v[t] > 0.0 ? v[t] : 0.0;
   if (blockIdx.x == 1) {
     for (int i = t; i < nz; i += kSetupThreads) acc[i] = 0.0;
     __syncthreads();
     if (t == 0) {
       double w = 0.0;
+#pragma unroll 8
       for (int j = 0; j < L; ++j) w += Wt[j];
       scal[5] = w;
     }
     return;
   }
-  for (int pp = t; pp < N; pp += kSetupThreads) {
+  if (t >= H && t - H < N) {
+    const int pp = t - H;
     const double x = normals[3 * pp], y = normals[3 * pp + 1], z = normals[3 * pp + 2];
     const double il = 1.0 / sqrt(x * x + y * y + z * z);
     nh[3 * pp] = T(x * il);
@@ -524,16 +557,10 @@ __global__ void __launch_bounds__(kSetupThreads)
     nh[3 * pp + 2] = T(z * il);
   }
   __syncthreads();
-  for (int k = K; k >= 1; --k) {
-    for (int i = t; i < (1 << (k - 1)); i += kSetupThreads) {
-      const int pp = (1 << K) - (1 << k) + i;
-      const int pc = (1 << K) - (1 << (k + 1)) + 2 * i;
-      const double a = k == K ? Wt[2 * i] : Wt[L + pc], b = k == K ? Wt[2 * i + 1] : Wt[L + pc + 1];
-      const double W = a + b;
-      Wt[L + pp] = W;
-      c1s[pp] = T(W > 0.0 ? a / W : 0.5);
-    }
-    __syncthreads();
+  tree_weights(K, t, Wt);
+  if (t < N) {
+    const double a = Wt[child_slot(K, node_level(K, t), t)], W = Wt[L + t];
+    c1s[t] = T(W > 0.0 ? a / W : 0.5);
   }
 }
 
@@ -558,7 +585,7 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_fwd(int K, int k, int64_t n
 }
 
 // per-sample error from the root column, and the batch reduction
-template <typename T>
+template <int MODE, typename T>
 __global__ void __launch_bounds__(kLvlThreads) k_lvl_err(int K, int64_t n, const T *NS, const double *Ct, double p,
                                                          double q, double penalty, double *err, double *part,
                                                          double *scal, double *loss) {
@@ -567,33 +594,33 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_err(int K, int64_t n, const
   if (s < n) {
     T D[21];
     lvl_load(NS, (1 << K) - 2, n, s, D);
-    e = lin_error<T>(Ct + 36 * s, D, p);
+    e = lin_error<MODE>(Ct + 36 * s, D, p);
     err[s] = e;
   }
   lin_reduce(n, e, q, penalty, part, scal, loss);
 }
 
-// dJ/dD at the root: (1/N) S^(1/q-1) (e_s/m)^(q-1) de_s/dD
-template <typename T>
+// dJ/dD at the root: (1/N) S^(1/q-1) (e_s/m)^(q-1) de_s/dD, with |T - D|_p =
+// e_s |T|_p; for p = 1 every component's is +-1 / |T|_1
+template <int MODE, typename T>
 __device__ __forceinline__ void lin_seed(const double *Tg, const T *D, double p, double q, double e,
                                          const double *scal, T G[21]) {
   const double m = scal[0];
-  const double coef = (m > 0.0 && e > 0.0) ? scal[1] * pow(e / m, q - 1.0) : 0.0;
-  double nx, nt;
-  lin_norms(Tg, D, p, nx, nt);
-  const double f = p == 1.0 ? 1.0 : pow(nx, 1.0 - p);
+  const double coef = (m > 0.0 && e > 0.0) ? scal[1] * pow_q(e / m, q - 1.0) : 0.0;
+  const double nt = lin_norm<MODE>(p, [&](int i, int j) { return Tg[6 * i + j]; });
+  const double f = MODE == 1 ? 1.0 / nt : (MODE == 2 ? 1.0 / (e * nt) : pow(e * nt, 1.0 - p)) / nt;
 #pragma unroll
   for (int i = 0; i < 6; ++i)
 #pragma unroll
     for (int j = i; j < 6; ++j) {
       const double x = Tg[6 * i + j] - double(sget(D, i, j));
       const double sg = x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0);
-      const double xp = p == 1.0 ? 1.0 : (p == 2.0 ? fabs(x) : pow(fabs(x), p - 1.0));
-      const double de = nx > 0.0 ? -sg * xp * f / nt : 0.0;
+      const double xp = MODE == 1 ? 1.0 : (MODE == 2 ? fabs(x) : pow(fabs(x), p - 1.0));
+      const double de = e > 0.0 ? -sg * xp * f : 0.0;
       G[sidx(i, j)] = T(coef * de);
     }
 }
-template <typename T>
+template <int MODE, typename T>
 __global__ void __launch_bounds__(kLvlThreads) k_lvl_seed(int K, int64_t n, const T *NS, const double *Ct, double p,
                                                           double q, const double *err, const double *scal, T *GA) {
   const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
@@ -601,7 +628,7 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_seed(int K, int64_t n, cons
   const int root = (1 << K) - 2;
   T D[21], G[21];
   lvl_load(NS, root, n, s, D);
-  lin_seed(Ct + 36 * s, D, p, q, err[s], scal, G);
+  lin_seed<MODE>(Ct + 36 * s, D, p, q, err[s], scal, G);
   lvl_store(GA, root, n, s, G);
 }
 
@@ -659,11 +686,10 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_bwd(int K, int k, int64_t n
 // phases).  Of the 12 words of 21 a parent and its children move in two
 // launches (forward: 4 in, 2 in again, 3 out) the pass keeps 7; of the reverse
 // mode's 19 (9 + 2 x 5, no adjoints below the bottom) 15.  K = 8, 65,536
-// samples: forward 480 -> 500 us (its bottom pair spills at four CTAs per SM),
-// reverse 890 -> 745, the step 1714 -> 1493; 32 samples (half the launches):
-// 172 -> 155 us.
+// samples: the step 1714 -> 1493 us; 32 samples (half the launches): 172 ->
+// 155 us.
 template <bool LEAF, typename T>
-__global__ void __launch_bounds__(kLvlThreads, 4) k_lvl_fwd2(int K, int k, int64_t n, const T *PH, const T *nh,
+__global__ void __launch_bounds__(kLvlThreads, LEAF ? 3 : 4) k_lvl_fwd2(int K, int k, int64_t n, const T *PH, const T *nh,
                                                           const T *c1s, T *NS) {
   const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
   if (s >= n) return;
@@ -760,16 +786,20 @@ __global__ void __launch_bounds__(kLvlThreads, 3) k_lvl_bwd2(int K, int k, int64
 }
 
 // The chain through the weights (c1 = W_1 / W, w = <v>_+, penalty) and the
-// normalisation of the normals: one CTA, the nodes of a level on its threads,
-// subtree weights and their adjoints in shared memory.  (One thread with both
-// in local memory took 928 us at K = 8.)
-__global__ void __launch_bounds__(1 << kLinMaxK)
+// normalisation of the normals: one CTA.  Its second half takes the normals;
+// the first the weights level by level, then every node's two quotients at
+// once, then the adjoints of the subtree weights from the root down, so that
+// the level loops hold additions only.  (One thread with the weights in local
+// memory took 928 us at K = 8; divisions in the level loop, 19.)
+__global__ void __launch_bounds__(kSetupThreads)
     k_lin_finish(int K, const double *normals, const double *v, double penalty, const double *gnh,
                  const double *gc1, const double *scal, double *grad_n, double *grad_v) {
-  __shared__ double Wt[2 << kLinMaxK], gW[1 << kLinMaxK];  // weights: leaves [0, L), nodes [L, L + N)
+  __shared__ double Wt[2 << kLinMaxK], gW[2 << kLinMaxK];  // leaves [0, L), nodes [L, L + N)
   const int N = (1 << K) - 1, L = 1 << K, t = threadIdx.x;
-  for (int j = t; j < L; j += blockDim.x) Wt[j] = v[j] > 0.0 ? v[j] : 0.0;
-  for (int pp = t; pp < N; pp += blockDim.x) {
+  constexpr int H = kSetupThreads / 2;
+  if (t < L) Wt[t] = v[t] > 0.0 ? v[t] : 0.0;
+  if (t >= H && t - H < N) {
+    const int pp = t - H;
     const double x = normals[3 * pp], y = normals[3 * pp + 1], z = normals[3 * pp + 2];
     const double len = sqrt(x * x + y * y + z * z);
     const double nh[3] = {x / len, y / len, z / len};
@@ -778,32 +808,24 @@ __global__ void __launch_bounds__(1 << kLinMaxK)
     for (int c = 0; c < 3; ++c) grad_n[3 * pp + c] = (g[c] - gd * nh[c]) / len;
   }
   __syncthreads();
-  // children of node i of level k: slots ch, ch + 1 of Wt
-  auto child = [&](int k, int i) { return k == K ? 2 * i : L + (1 << K) - (1 << (k + 1)) + 2 * i; };
-  for (int k = K; k >= 1; --k) {
-    for (int i = t; i < (1 << (k - 1)); i += blockDim.x)
-      Wt[L + (1 << K) - (1 << k) + i] = Wt[child(k, i)] + Wt[child(k, i) + 1];
-    __syncthreads();
+  tree_weights(K, t, Wt);
+  if (t < N) {  // into the children's slots: what c1's derivative adds to the node's own adjoint
+    const int ch = child_slot(K, node_level(K, t), t);
+    const double W = Wt[L + t], a = Wt[ch], b = Wt[ch + 1], g = gc1[t];
+    gW[ch] = W > 0.0 ? g * b / (W * W) : 0.0;       // d c1 / d W_1 = W_2 / W^2
+    gW[ch + 1] = W > 0.0 ? -g * a / (W * W) : 0.0;  // d c1 / d W_2 = -W_1 / W^2
   }
-  // adjoints of the subtree weights, root first
-  if (t == 0) gW[N - 1] = 2.0 * penalty * (scal[5] - 1.0);
+  if (t == 0) gW[L + N - 1] = 2.0 * penalty * (scal[5] - 1.0);
   __syncthreads();
   for (int k = 1; k <= K; ++k) {
-    for (int i = t; i < (1 << (k - 1)); i += blockDim.x) {
-      const int pp = (1 << K) - (1 << k) + i, ch = child(k, i);
-      const double W = Wt[L + pp], a = Wt[ch], b = Wt[ch + 1];
-      const double dL = W > 0.0 ? gc1[pp] * b / (W * W) : 0.0;   // d c1 / d W_1 = W_2 / W^2
-      const double dR = W > 0.0 ? -gc1[pp] * a / (W * W) : 0.0;  // d c1 / d W_2 = -W_1 / W^2
-      if (k == K) {
-        grad_v[2 * i] = a > 0.0 ? gW[pp] + dL : 0.0;
-        grad_v[2 * i + 1] = b > 0.0 ? gW[pp] + dR : 0.0;
-      } else {
-        gW[ch - L] = gW[pp] + dL;
-        gW[ch - L + 1] = gW[pp] + dR;
-      }
+    if (t < (1 << (k - 1))) {
+      const int pp = (1 << K) - (1 << k) + t, ch = child_slot(K, k, pp);
+      gW[ch] = gW[L + pp] + gW[ch];
+      gW[ch + 1] = gW[L + pp] + gW[ch + 1];
     }
     __syncthreads();
   }
+  if (t < L) grad_v[t] = Wt[t] > 0.0 ? gW[t] : 0.0;
 }
 
 __global__ void k_amsgrad(int64_t n, double *x, const double *g, double *m, double *s, double *smax, double lr,
@@ -855,14 +877,13 @@ const char *lin_check(int32_t K, int64_t n, const double *C1, const double *C2, 
 
 template <typename T>
 dmn_status lin_forward(cudaStream_t st, int K, int64_t n, const double *C1, const double *C2,
-                       const double *normals, const double *v, const double *Ct, double p, double *Cbar,
-                       double *err) {
+                       const double *normals, const double *v, double *Cbar) {
   const size_t smem = sizeof(T) * lin_layout(K).words;
   const int threads = 1 << (K - 1);
   int grid = 0;
   cudaError_t e = lin_grid(k_lin_forward<T>, threads, smem, n, &grid);
   if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: launch configuration");
-  k_lin_forward<T><<<grid, threads, smem, st>>>(K, n, C1, C2, normals, v, Ct, p, Cbar, err);
+  k_lin_forward<T><<<grid, threads, smem, st>>>(K, n, C1, C2, normals, v, Cbar);
   if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: forward launch");
   return DMN_OK;
 }
@@ -878,7 +899,7 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   if (nb > 2147483647u) return lin_fail("dmn_linear_loss_grad: batch too large");
   const int N = (1 << K) - 1;
   T *nh = consts, *c1s = consts + 3 * N;
-  const unsigned ns = unsigned((n + kSetupThreads - 1) / kSetupThreads);
+  const unsigned ns = unsigned((n + kSetupThreads / 2 - 1) / (kSetupThreads / 2));
   k_lvl_setup<T><<<2 + ns, kSetupThreads, 0, st>>>(K, n, normals, v, C1, C2, nh, c1s, PH, gnh, 4 * N + 5, scal);
   // FP32: pairs of levels from the bottom (FP64 laminates: 251 registers for one
   // level, and bound by the FP64 pipe, so one level a launch)
@@ -894,8 +915,11 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: forward level launch");
   // the blocks' partial sums: in the adjoints' array, free until the seed, from an 8-byte boundary
   double *part = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(GA) + 7) & ~uintptr_t(7));
-  k_lvl_err<T><<<nb, kLvlThreads, 0, st>>>(K, n, NS, Ct, p, q, penalty, err, part, scal, loss);
-  k_lvl_seed<T><<<nb, kLvlThreads, 0, st>>>(K, n, NS, Ct, p, q, err, scal, GA);
+  const int mode = pow_mode(p);
+  (mode == 1 ? k_lvl_err<1, T> : mode == 2 ? k_lvl_err<2, T> : k_lvl_err<0, T>)<<<nb, kLvlThreads, 0, st>>>(
+      K, n, NS, Ct, p, q, penalty, err, part, scal, loss);
+  (mode == 1 ? k_lvl_seed<1, T> : mode == 2 ? k_lvl_seed<2, T> : k_lvl_seed<0, T>)<<<nb, kLvlThreads, 0, st>>>(
+      K, n, NS, Ct, p, q, err, scal, GA);
   if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: loss launch");
   // the same pairs, root first
   k = 1;
@@ -930,8 +954,8 @@ extern "C" dmn_status dmn_linear_forward(dmn_stream stream, int32_t K, int64_t n
   if (n_samples == 0) return DMN_OK;
   cudaStream_t st = (cudaStream_t)stream;
   return precision == DMN_LIN_FP64
-             ? lin_forward<double>(st, K, n_samples, d_C1, d_C2, d_normals, d_v, nullptr, 1.0, d_Cbar, nullptr)
-             : lin_forward<float>(st, K, n_samples, d_C1, d_C2, d_normals, d_v, nullptr, 1.0, d_Cbar, nullptr);
+             ? lin_forward<double>(st, K, n_samples, d_C1, d_C2, d_normals, d_v, d_Cbar)
+             : lin_forward<float>(st, K, n_samples, d_C1, d_C2, d_normals, d_v, d_Cbar);
 }
 
 extern "C" dmn_status dmn_linear_loss_grad(dmn_stream stream, int32_t K, int64_t n_samples, const double *d_C1,
@@ -962,7 +986,7 @@ extern "C" dmn_status dmn_linear_loss_grad(dmn_stream stream, int32_t K, int64_t
                               d_loss, reinterpret_cast<float *>(consts), f, f + ph, f + ph + cells, gnh, gc1);
   }
   if (s != DMN_OK) return s;
-  k_lin_finish<<<1, 1 << kLinMaxK, 0, st>>>(K, d_normals, d_v, penalty, gnh, gc1, scal, d_grad_n, d_grad_v);
+  k_lin_finish<<<1, kSetupThreads, 0, st>>>(K, d_normals, d_v, penalty, gnh, gc1, scal, d_grad_n, d_grad_v);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: finish launch");
   return DMN_OK;
