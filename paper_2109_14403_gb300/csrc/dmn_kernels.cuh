@@ -229,6 +229,12 @@ __device__ __forceinline__ void mat_point(MatPt<TF, HP> &o, HP theta, HP idt, TF
   if (LAW >= 2 && o.kind == 2) o.isy = hp_div(o.one, sy);
 }
 
+// A leaf's tangent by its parts: cP1 m m^T + cI I - cN N (x) N, m = (1,1,1,0,0,0)
+template <typename TF>
+struct LeafTan {
+  TF cP1, cI, cN, N[6];
+};
+
 // Leaf update at strain eps and the point's temperature (Sec. 4).  Stress,
 // coupling term D and dissipation X in HP; derivatives into the TF record.
 // zn = internal variables at t^n (eps_p Mandel 6, p; kind 2 also the leaf
@@ -243,11 +249,14 @@ __device__ __forceinline__ void mat_point(MatPt<TF, HP> &o, HP theta, HP idt, TF
 // 1/(3G + H) replaced by c m phi^(m-1) / (sigma_Y + c m phi^(m-1) (3G + H));
 // temperature-dependent moduli add theta (r'/r) sigma : (de - d eps_p) / dt
 // to D, de the leaf's strain increment.  With full = false the output-only
-// quantities (D, X and the record's tau, dd, gg) are left at zero.
-template <typename TF, typename HP, int LAW>
+// quantities (D, X and the record's tau, dd, gg) are left at zero.  PARTS
+// (FP64): the tangent goes to *tan by its parts, not into the record (whose ds
+// is not set either), and the plastic step takes one rsqrt in place of two
+// square roots and two divisions, each some 25 FP64 instructions.
+template <typename TF, typename HP, int LAW, bool PARTS = false>
 __device__ __forceinline__ void leaf_eval(const MatPt<TF, HP> &m, const HP eps[6], const HP *zn,
                                           HP trn, HP sig[6], HP &D, HP &X, Rec<TF> &R, HP *znew,
-                                          bool full = true) {
+                                          bool full = true, LeafTan<TF> *tan = nullptr) {
   const bool j2 = m.kind >= 1;
   const bool vp = LAW >= 2 && m.kind == 2;
   HP ee[6];
@@ -293,7 +302,13 @@ __device__ __forceinline__ void leaf_eval(const MatPt<TF, HP> &m, const HP eps[6
     const HP q2 = m.c15 * sn2;
     plastic = hp_gt(q2, yr * yr);
     if (plastic) {
-      const HP q = hp_sqrt(q2);  // q_tr = sqrt(3/2) |s_tr|
+      HP q, iq;  // q_tr = sqrt(3/2) |s_tr| (iq: PARTS only, 1 / q_tr)
+      if constexpr (PARTS) {
+        iq = rsqrt(q2);
+        q = q2 * iq;
+      } else {
+        q = hp_sqrt(q2);
+      }
       HP dp;
       TF kinv = m.iden_f, phif = TF(0);
       if (vp) {
@@ -336,7 +351,9 @@ __device__ __forceinline__ void leaf_eval(const MatPt<TF, HP> &m, const HP eps[6
       } else {
         dp = (q - yr) * m.iden;  // closed-form plastic multiplier
       }
-      const HP kap = hp_div(dp, q);  // dp / q_tr
+      HP kap;  // dp / q_tr
+      if constexpr (PARTS) kap = dp * iq;
+      else kap = hp_div(dp, q);
       const HP th1h = m.one - m.G3 * kap;
       const HP kz = m.c15 * kap;
 #pragma unroll
@@ -354,7 +371,9 @@ __device__ __forceinline__ void leaf_eval(const MatPt<TF, HP> &m, const HP eps[6
       const TF kapf = tf_of(kap, (TF *)nullptr), dpf = tf_of(dp, (TF *)nullptr);
       th1 = TF(1) - m.G3_f * kapf;
       thb = m.G3_f * kinv - m.G3_f * kapf;
-      const TF isn = TF(1) / sqrt(tf_of(sn2, (TF *)nullptr));
+      TF isn;  // 1 / |s_tr|
+      if constexpr (PARTS) isn = TF(1.2247448713915890491) * iq;
+      else isn = TF(1) / sqrt(tf_of(sn2, (TF *)nullptr));
 #pragma unroll
       for (int c = 0; c < 6; ++c) Nf[c] = tf_of(s[c], (TF *)nullptr) * isn;
       if (!full) {
@@ -384,21 +403,31 @@ __device__ __forceinline__ void leaf_eval(const MatPt<TF, HP> &m, const HP eps[6
     for (int c = 0; c < 6; ++c) sig[c] = c < 3 ? pk + s[c] : s[c];
   }
   // tangent C = 3K P1 + 2G th1 P2 - 2G thb N (x) N
-  const TF cP1 = m.Kb_f - m.G2_f * th1 / TF(3);  // coefficient of m m^T
+  TF cP1;  // coefficient of m m^T
+  if constexpr (PARTS) cP1 = m.Kb_f - m.G2_f * th1 * m.third;
+  else cP1 = m.Kb_f - m.G2_f * th1 / TF(3);
   const TF cI = m.G2_f * th1;
   const TF cN = m.G2_f * thb;
+  if constexpr (PARTS) {
+    tan->cP1 = cP1;
+    tan->cI = cI;
+    tan->cN = cN;
 #pragma unroll
-  for (int i = 0; i < 6; ++i)
+    for (int c = 0; c < 6; ++c) tan->N[c] = Nf[c];
+  } else {
 #pragma unroll
-    for (int j = i; j < 6; ++j)
-      R.C[sidx(i, j)] = (i < 3 && j < 3 ? cP1 : TF(0)) + (i == j ? cI : TF(0)) - cN * Nf[i] * Nf[j];
+    for (int i = 0; i < 6; ++i)
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    R.ds[c] = TF(0);
-    R.tau[c] = TF(0);
-    R.dd[c] = TF(0);
+      for (int j = i; j < 6; ++j)
+        R.C[sidx(i, j)] = (i < 3 && j < 3 ? cP1 : TF(0)) + (i == j ? cI : TF(0)) - cN * Nf[i] * Nf[j];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      R.ds[c] = TF(0);
+      R.tau[c] = TF(0);
+      R.dd[c] = TF(0);
+    }
+    R.gg = TF(0);
   }
-  R.gg = TF(0);
   if (!full) return;
   TF ta = -m.a3K_f;
   if (vp) ta += m.dKb_f * tf_of(tr, (TF *)nullptr);

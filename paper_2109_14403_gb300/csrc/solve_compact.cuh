@@ -197,6 +197,366 @@ __device__ __forceinline__ void combine_rows(const SolveParams &P, int p, int r,
   }
 }
 
+// ---- the condensation in FP64 (combine() of dmn_kernels.cuh with fewer
+// operations): with dC = C_L - C_R, U = dC B and c1 + c2 = 1,
+//   K = B^T C_R B + c2 B^T U,  C_hat = C_R + c1 dC - U (c1 c2 G),
+// and B's zeros left out.  About 400 FP64 instructions per node, against 500.
+
+// K^-1 of the symmetric K = (k00, k01, k02, k11, k12, k22)
+__device__ __forceinline__ void inv_sym3(const double k[6], double Ki[3][3]) {
+  const double a00 = k[3] * k[5] - k[4] * k[4], a01 = k[2] * k[4] - k[1] * k[5], a02 = k[1] * k[4] - k[2] * k[3];
+  const double a11 = k[0] * k[5] - k[2] * k[2], a12 = k[1] * k[2] - k[0] * k[4], a22 = k[0] * k[3] - k[1] * k[1];
+  const double id = 1.0 / (k[0] * a00 + k[1] * a01 + k[2] * a02);
+  Ki[0][0] = a00 * id;
+  Ki[0][1] = Ki[1][0] = a01 * id;
+  Ki[0][2] = Ki[2][0] = a02 * id;
+  Ki[1][1] = a11 * id;
+  Ki[1][2] = Ki[2][1] = a12 * id;
+  Ki[2][2] = a22 * id;
+}
+__device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
+  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
+}
+// What follows U and K for a whole node: G_p, h_p, the condensed vectors and
+// C_hat = base - U (c1 c2 G).  L: in the left child's vectors, out the node's;
+// C enters as the base.  bds = B^T (ds_L - ds_R) (0 for leaves).
+__device__ __forceinline__ void condense(Rec<double> &L, const Rec<double> &R, const double U[6][3],
+                                         const double k6[6], const NodeHP<double> &nd, const double rb[3],
+                                         bool leaves, double *gh, bool full) {
+  const double c1 = nd.c1, cc = nd.c1 * nd.c2;
+  double Ki[3][3], Gm[3][6];
+  inv_sym3(k6, Ki);
+#pragma unroll
+  for (int e = 0; e < 3; ++e)
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+      const double g = dot3(Ki[e], U[a]);
+      gh[6 * e + a] = g;
+      Gm[e][a] = cc * g;
+    }
+  // v <- c1 v_L + c2 v_R - c1 c2 U K^-1 (b + B^T (v_L - v_R)), the solve's
+  // right-hand side left in t, K^-1 t in h
+  auto vec = [&](double *v, const double *vr, const double *b, double t[3], double h[3], bool zero) {
+    double d[6];
+    if (!zero) {
+#pragma unroll
+      for (int c = 0; c < 6; ++c) d[c] = v[c] - vr[c];
+      btvec_hp(nd, d, t);
+    }
+#pragma unroll
+    for (int e = 0; e < 3; ++e) t[e] = zero ? b[e] : (b ? b[e] + t[e] : t[e]);
+    double hc[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      h[e] = dot3(Ki[e], t);
+      hc[e] = -cc * h[e];
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      double x = zero ? U[c][0] * hc[0] : fma(U[c][0], hc[0], fma(c1, d[c], vr[c]));
+      x = fma(U[c][1], hc[1], x);
+      v[c] = fma(U[c][2], hc[2], x);
+    }
+  };
+  double t[3], h[3];
+  vec(L.ds, R.ds, rb, t, h, leaves);
+#pragma unroll
+  for (int e = 0; e < 3; ++e) gh[18 + e] = h[e];
+  if (full) {
+    double ht[3];
+    vec(L.tau, R.tau, nullptr, t, ht, false);
+    vec(L.dd, R.dd, nullptr, t, h, false);
+    // g_hat = c1 g_L + c2 g_R - c1 c2 (B^T d_diff) . h_tau
+    L.gg = fma(c1, L.gg - R.gg, R.gg) - cc * dot3(t, ht);
+  }
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = i; j < 6; ++j) {
+      double x = L.C[sidx(i, j)];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) x = fma(-U[i][e], Gm[e][j], x);
+      L.C[sidx(i, j)] = x;
+    }
+}
+
+// node with children records L (in/out) and R; rb = B^T (S_L - S_R) / (w c1 c2)
+__device__ __forceinline__ void combine_d(Rec<double> &L, const Rec<double> &R, const NodeHP<double> &nd,
+                                          const double rb[3], double *gh, bool full) {
+#pragma unroll
+  for (int q = 0; q < 21; ++q) L.C[q] -= R.C[q];
+  double U[6][3], k6[6] = {};
+#pragma unroll
+  for (int a = 0; a < 6; ++a) {
+    double row[6], m[3];
+#pragma unroll
+    for (int b = 0; b < 6; ++b) row[b] = sget(L.C, a, b);
+    btvec_hp(nd, row, U[a]);
+#pragma unroll
+    for (int b = 0; b < 6; ++b) row[b] = sget(R.C, a, b);
+    btvec_hp(nd, row, m);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) m[f] = fma(nd.c2, U[a][f], m[f]);  // row a of M B
+    // K = B^T M B, upper triangle: rows of B as in bvec_hp
+    if (a == 0) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) k6[f] = nd.n[0] * m[f];
+    }
+    if (a == 1) {
+      k6[3] = nd.n[1] * m[1];
+      k6[4] = nd.n[1] * m[2];
+    }
+    if (a == 2) k6[5] = nd.n[2] * m[2];
+    if (a == 3) {
+      k6[3] = fma(nd.ns[2], m[1], k6[3]);
+      k6[4] = fma(nd.ns[2], m[2], k6[4]);
+      k6[5] = fma(nd.ns[1], m[2], k6[5]);
+    }
+    if (a == 4) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) k6[f] = fma(nd.ns[2], m[f], k6[f]);
+      k6[5] = fma(nd.ns[0], m[2], k6[5]);
+    }
+    if (a == 5) {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) k6[f] = fma(nd.ns[1], m[f], k6[f]);
+      k6[3] = fma(nd.ns[0], m[1], k6[3]);
+      k6[4] = fma(nd.ns[0], m[2], k6[4]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 21; ++q) L.C[q] = fma(nd.c1, L.C[q], R.C[q]);
+  condense(L, R, U, k6, nd, rb, false, gh, full);
+}
+
+// bottom laminate of two leaves with tangents cP1 m m^T + cI I - cN N N^T
+// (m = (1,1,1,0,0,0)): B^T m = n, B^T B = (I + n n^T) / 2, so K, U and the base
+// of C_hat need no 6x6 products.  L, R: the leaves' vectors (no ds).
+__device__ __forceinline__ void combine_leaves(Rec<double> &L, const Rec<double> &R, const LeafTan<double> &A,
+                                               const LeafTan<double> &B, const NodeHP<double> &nd,
+                                               const double rb[3], double *gh, bool full) {
+  const double c1 = nd.c1, c2 = nd.c2, dp = A.cP1 - B.cP1, di = A.cI - B.cI;
+  const double i2 = 0.5 * fma(c2, di, B.cI), al = fma(c2, dp, B.cP1) + i2;
+  const double *n = nd.n, *ns = nd.ns;
+  double k6[6], U[6][3];
+  {
+    const double an[3] = {al * n[0], al * n[1], al * n[2]};
+    k6[0] = fma(an[0], n[0], i2);
+    k6[1] = an[0] * n[1];
+    k6[2] = an[0] * n[2];
+    k6[3] = fma(an[1], n[1], i2);
+    k6[4] = an[1] * n[2];
+    k6[5] = fma(an[2], n[2], i2);
+  }
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    const double v = dp * n[f];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) U[a][f] = a == f ? fma(di, n[f], v) : v;
+  }
+  const double s0 = di * ns[0], s1 = di * ns[1], s2 = di * ns[2];
+  U[3][0] = 0.0, U[3][1] = s2, U[3][2] = s1;
+  U[4][0] = s2, U[4][1] = 0.0, U[4][2] = s0;
+  U[5][0] = s1, U[5][1] = s0, U[5][2] = 0.0;
+  const double pb = fma(c1, dp, B.cP1), ib = fma(c1, di, B.cI);
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = i; j < 6; ++j) L.C[sidx(i, j)] = i < 3 && j < 3 ? (i == j ? pb + ib : pb) : (i == j ? ib : 0.0);
+  // the rank-one part of a leaf: -w c N N^T in K (w = wk), sg c N N^T B in U,
+  // -w c N N^T in the base (w = wc); elastic leaves have none
+  auto rank1 = [&](const LeafTan<double> &X, double wk, double wc, double sg) {
+    if (X.cN == 0.0) return;
+    double t[3], v[3];
+    btvec_hp(nd, X.N, t);
+    const double ck = -wk * X.cN, cu = sg * X.cN, cb = -wc * X.cN;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const double k = ck * t[e];
+      v[e] = cu * t[e];
+#pragma unroll
+      for (int f = e; f < 3; ++f) k6[e * (5 - e) / 2 + f] = fma(k, t[f], k6[e * (5 - e) / 2 + f]);
+    }
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+      const double x = cb * X.N[a];
+#pragma unroll
+      for (int f = 0; f < 3; ++f) U[a][f] = fma(X.N[a], v[f], U[a][f]);
+#pragma unroll
+      for (int b = a; b < 6; ++b) L.C[sidx(a, b)] = fma(x, X.N[b], L.C[sidx(a, b)]);
+    }
+  };
+  rank1(A, c2, c1, -1.0);
+  rank1(B, c1, c2, 1.0);
+  condense(L, R, U, k6, nd, rb, true, gh, full);
+}
+
+// residual traction B^T (c2 S_L - c1 S_R), its square added to r2
+__device__ __forceinline__ void node_residual(const NodeHP<double> &nd, const double *sL, const double *sR,
+                                              double *sdst, double rv[3], double &r2) {
+  double dh[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    dh[c] = nd.c2 * sL[c] - nd.c1 * sR[c];
+    sdst[c] = sL[c] + sR[c];
+  }
+  btvec_hp(nd, dh, rv);
+  r2 += dot3(rv, rv);
+}
+
+// a node on one lane, children's records and sums in shared memory
+__device__ __forceinline__ void combine_node(const SolveParams &P, int p, const double *rcL, const double *rcR,
+                                             const double *sL, const double *sR, double *dst, double *sdst,
+                                             double *gh, double &r2, bool full) {
+  NodeHP<double> nd;
+  load_node(P, p, nd);
+  double n[3], c1, c2, iwcc, wcc, rv[3];
+  load_node_tf(P, p, n, c1, c2, iwcc, wcc);
+  node_residual(nd, sL, sR, sdst, rv, r2);
+#pragma unroll
+  for (int e = 0; e < 3; ++e) rv[e] *= iwcc;
+  Rec<double> L, R;
+  rec_get(L, rcL);
+  rec_get(R, rcR);
+  combine_d(L, R, nd, rv, gh, full);
+  rec_put(dst, L);
+}
+
+// A node on two lanes (2i, 2i + 1 of an aligned pair): lane h owns Mandel rows
+// 3h .. 3h + 2.  Sums over rows (K, the right-hand sides) are halves added by a
+// shuffle; of C_hat a lane forms its own 3 x 3 block's upper triangle and, of
+// the 3 x 3 block between the lanes, the pairs (own r, other o) with r <= o (both
+// form the diagonal).  About 300 FP64 instructions a lane.
+__device__ __forceinline__ void combine_half(const SolveParams &P, int p, int h, bool st, unsigned mask,
+                                             const double *rcL, const double *rcR, const double *sL,
+                                             const double *sR, double *dst, double *sdst, double *gh, double &r2,
+                                             bool full) {
+  NodeHP<double> nd;
+  load_node(P, p, nd);
+  double n_[3], c1, c2, iwcc, wcc;
+  load_node_tf(P, p, n_, c1, c2, iwcc, wcc);
+  const double cc = c1 * c2;
+  auto other = [&](double v) { return __shfl_xor_sync(mask, v, 1); };
+  // the lane's rows of B
+  double bo[3][3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int e = 0; e < 3; ++e) bo[r][e] = h ? (r == e ? 0.0 : nd.ns[3 - r - e]) : (r == e ? nd.n[r] : 0.0);
+  auto bt = [&](const double v[3], double t[3]) {  // B^T v, both lanes' rows
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const double x = bo[0][e] * v[0] + bo[1][e] * v[1] + bo[2][e] * v[2];
+      t[e] = x + other(x);
+    }
+  };
+  // packed index of (own r, own s) and of (own r, other o)
+  auto qo = [&](int r, int s) { return h ? sidx(3 + (r < s ? r : s), 3 + (r < s ? s : r)) : sidx(r < s ? r : s, r < s ? s : r); };
+  auto qx = [&](int r, int o) { return h ? sidx(o, 3 + r) : sidx(r, 3 + o); };
+  double U[3][3], k6[6] = {}, own[6], crs[6];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    double xr[6], dr[6], m[3];  // row 3h + r of C_R and of dC
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const int q0 = c < 3 ? sidx(r < c ? r : c, r < c ? c : r) : sidx(r, c);
+      const int q1 = c < 3 ? sidx(c, 3 + r) : sidx(3 + (r < c - 3 ? r : c - 3), 3 + (r < c - 3 ? c - 3 : r));
+      const int q = h ? q1 : q0;
+      xr[c] = rcR[q];
+      dr[c] = rcL[q] - xr[c];
+    }
+    btvec_hp(nd, dr, U[r]);
+    btvec_hp(nd, xr, m);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) m[f] = fma(c2, U[r][f], m[f]);
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+#pragma unroll
+      for (int f = e; f < 3; ++f) k6[e * (5 - e) / 2 + f] = fma(bo[r][e], m[f], k6[e * (5 - e) / 2 + f]);
+    // base of C_hat: C_R + c1 dC of the entries this lane forms
+#pragma unroll
+    for (int s = r; s < 3; ++s) {
+      const int i = r * (5 - r) / 2 + s;
+      own[i] = fma(c1, h ? dr[3 + s] : dr[s], h ? xr[3 + s] : xr[s]);
+      crs[i] = fma(c1, h ? dr[s] : dr[3 + s], h ? xr[s] : xr[3 + s]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 6; ++q) k6[q] += other(k6[q]);
+  double Ki[3][3], V[3][3], W[3][3];  // V[r][e]: column 3h + r of c1 c2 G; W: of the other lane's
+  inv_sym3(k6, Ki);
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const double g = dot3(Ki[e], U[r]);
+      if (st) gh[6 * e + 3 * h + r] = g;
+      V[r][e] = cc * g;
+      W[r][e] = other(V[r][e]);
+    }
+#pragma unroll
+  for (int r = 0; r < 3; ++r)
+#pragma unroll
+    for (int s = r; s < 3; ++s) {
+      const int i = r * (5 - r) / 2 + s;
+      const double x = own[i] - dot3(U[r], V[s]), y = crs[i] - dot3(U[r], W[s]);
+      if (st) dst[qo(r, s)] = x;
+      if (st && (h == 0 || r != s)) dst[qx(r, s)] = y;
+    }
+  // residual and condensed vectors, the lane's components
+  double rv[3];
+  {
+    double dh[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const double SL = sL[3 * h + r], SR = sR[3 * h + r];
+      dh[r] = c2 * SL - c1 * SR;
+      if (st) sdst[3 * h + r] = SL + SR;
+    }
+    bt(dh, rv);
+    if (st && h == 0) r2 += dot3(rv, rv);
+  }
+  auto vec = [&](int off, const double *b, double t[3], double hs[3]) {
+    double d[3], vr[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      vr[r] = rcR[off + 3 * h + r];
+      d[r] = rcL[off + 3 * h + r] - vr[r];
+    }
+    bt(d, t);
+    if (b) {
+#pragma unroll
+      for (int e = 0; e < 3; ++e) t[e] = fma(b[e], iwcc, t[e]);
+    }
+    double hc[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      hs[e] = dot3(Ki[e], t);
+      hc[e] = -cc * hs[e];
+    }
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      double x = fma(c1, d[r], vr[r]);
+#pragma unroll
+      for (int e = 0; e < 3; ++e) x = fma(U[r][e], hc[e], x);
+      if (st) dst[off + 3 * h + r] = x;
+    }
+  };
+  double t[3], hs[3];
+  vec(21, rv, t, hs);
+  if (st && h == 0) {
+#pragma unroll
+    for (int e = 0; e < 3; ++e) gh[18 + e] = hs[e];
+  }
+  if (full) {
+    double ht[3];
+    vec(27, nullptr, t, ht);
+    vec(33, nullptr, t, hs);
+    const double gR = rcR[39], gg = fma(c1, rcL[39] - gR, gR) - cc * dot3(t, ht);
+    if (st && h == 0) dst[39] = gg;
+  }
+}
+
 // The state block of a point is moved into shared memory by the bulk-copy
 // engine (cp.async.bulk, completion counted on an mbarrier): the jumps a into
 // a_s and, for the kinds that keep their internal variables as stored, z into
@@ -303,6 +663,17 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
   const unsigned mask = group_mask(G);
   const int W = group_width(G);
   const int lane = t & 31, warp = t >> 5, nwarp = (G + 31) >> 5;
+  // FP64 instances: an FP64 warp instruction takes 64 cycles of its
+  // sub-partition (19 of the SM with all four busy) whatever the number of
+  // active lanes (a probe of independent FMA chains), so their phases are laid
+  // out for few, full warps
+  constexpr bool D64 = sizeof(TF) == 8;
+  // this thread's bottom laminate.  FP64: the first half of the threads take
+  // the even ones, the second half the odd ones, so that the laminates of
+  // level K-1 find their left child in the registers of thread j < G/2 and
+  // fill whole warps (level K-1 below).  Mixed: in order (the packed level K-1
+  // cost it 2 to 4 %: one more barrier and more spills)
+  const int b = !D64 || K == 1 ? t : (t < G / 2 ? 2 * t : 2 * (t - G / 2) + 1);
   if (t == 0) {
     // a warp slot's sub-partition is slot mod 4 and a CTA's warps take
     // consecutive slots: rotate the leader by the CTA's slot group
@@ -351,14 +722,14 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
   const TF idt_f = TF(1.0 / P.dt);
   const TF tol = TF(P.tol), res_floor = TF(P.res_floor), gamma = TF(P.gamma);
 
-  const HP wL = hp_from(__ldg(P.leafw + 2 * t), tag), wR = hp_from(__ldg(P.leafw + 2 * t + 1), tag);
-  int zo0 = P.zoff[2 * t], zo1 = P.zoff[2 * t + 1];
+  const HP wL = hp_from(__ldg(P.leafw + 2 * b), tag), wR = hp_from(__ldg(P.leafw + 2 * b + 1), tag);
+  int zo0 = P.zoff[2 * b], zo1 = P.zoff[2 * b + 1];
   int zq0 = zo0 >= 0 ? zo0 - (8 + 3 * N) : -1, zq1 = zo1 >= 0 ? zo1 - (8 + 3 * N) : -1;
-  int hq0 = LAW == 3 ? P.hoff[2 * t] : zq0, hq1 = LAW == 3 ? P.hoff[2 * t + 1] : zq1;
-  int ph0 = P.phase[2 * t], ph1 = P.phase[2 * t + 1];
+  int hq0 = LAW == 3 ? P.hoff[2 * b] : zq0, hq1 = LAW == 3 ? P.hoff[2 * b + 1] : zq1;
+  int ph0 = P.phase[2 * b], ph1 = P.phase[2 * b + 1];
 
   // Strains of the bottom laminates by ancestor sums (eq. DMN kinematics):
-  // laminate t's strain is the root strain plus, for every ancestor p on its
+  // laminate b's strain is the root strain plus, for every ancestor p on its
   // path, +c2 B x_p (the path goes through child 1) or -c1 B x_p (child 2).
   // The two terms of every non-bottom node are formed at once, one node per
   // thread; after one barrier each thread adds its K-1 ancestors' terms root
@@ -366,7 +737,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
   //   SW_PLAIN: eK = eps_bar^{n+1} + sum of the B a terms
   //   SW_WARM:  a += da (da_s) on the way; eK as SW_PLAIN at the new a, and
   //             the trace of the strain at (eps_bar^n = tr_root, a^n) of
-  //             laminate t is returned (tr B a = a . n)
+  //             laminate b is returned (tr B a = a . n)
   //   SW_STEP:  eK += sum of the B da terms (the Newton increment in da_s),
   //             and a += da of the non-bottom nodes on the way
   // Ends with a barrier: eK is complete and the scratch region free again.
@@ -413,9 +784,9 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
 #pragma unroll
     for (int c = 0; c < 6; ++c) e[c] = mode == SW_STEP ? hp_zero(tag) : eb[c];
     for (int k = 1; k <= K - 1; ++k) {
-      const int p = (1 << K) - (1 << k) + (t >> (K - k));
+      const int p = (1 << K) - (1 << k) + (b >> (K - k));
       const HP *ent = anc + 14 * (p - G);
-      if ((t >> (K - k - 1)) & 1) {
+      if ((b >> (K - k - 1)) & 1) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) e[c] = e[c] - ent[6 + c];
         if (mode == SW_WARM) tr = tr - ent[13];
@@ -541,7 +912,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       __syncthreads();
 #pragma unroll 1
       for (int sd = 0; sd < 2; ++sd) {
-        const int j = 2 * t + sd, zo = sd ? zo1 : zo0, ph = sd ? ph1 : ph0, hq = sd ? hq1 : hq0;
+        const int zo = sd ? zo1 : zo0, ph = sd ? ph1 : ph0, hq = sd ? hq1 : hq0;
         if (zo < 0) continue;
         if (mp_s[ph].kind == 3) {
           pa_history<TF, HP>(mpa_s[ph], sin + zo, zn_s + hq);
@@ -549,7 +920,6 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
           const int nz = mp_s[ph].kind == 1 ? 7 : 13;
           for (int c = 0; c < nz; ++c) zn_s[hq + c] = hp_load(sin[zo + c], tag);
         }
-        (void)j;
       }
     }
     if (t == 0) {
@@ -572,14 +942,14 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       const HP tre =
           sweep(SW_WARM, hp_load(sin[0], tag) + hp_load(sin[1], tag) + hp_load(sin[2], tag));
       NodeHP<HP> nd;
-      load_node(P, t, nd);
-      const HP an[3] = {a_s[3 * t], a_s[3 * t + 1], a_s[3 * t + 2]};  // still a^n
+      load_node(P, b, nd);
+      const HP an[3] = {a_s[3 * b], a_s[3 * b + 1], a_s[3 * b + 2]};  // still a^n
       const HP trj = an[0] * nd.n[0] + an[1] * nd.n[1] + an[2] * nd.n[2];
       trn0 = tre + nd.c2 * trj;
       trn1 = tre - nd.c1 * trj;
 #pragma unroll
-      for (int r = 0; r < 3; ++r) a_s[3 * t + r] = hp_add_tf(an[r], da_s[3 * t + r]);
-      first = false;  // thread t alone uses a_s[3t..] until the next barrier
+      for (int r = 0; r < 3; ++r) a_s[3 * b + r] = hp_add_tf(an[r], da_s[3 * b + r]);
+      first = false;  // this thread alone uses a_s[3b..] until the next barrier
     } else {
       sweep(SW_PLAIN, hp_zero(tag));  // strains of the bottom laminates at a^n
     }
@@ -591,15 +961,15 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       // first pass of an iteration never gives the outputs: it skips their
       // terms (coupling term, dissipation, thermal tangents)
       const bool full = !ctrl->first;
-      // ---- R2: leaves and laminate t ----
+      // ---- R2: leaves and laminate b ----
       TF r2;
       HP S[6];
       {
         NodeHP<HP> nd;
-        load_node(P, t, nd);
+        load_node(P, b, nd);
         HP el[6], er[6];
         {
-          const HP av[3] = {a_s[3 * t], a_s[3 * t + 1], a_s[3 * t + 2]};
+          const HP av[3] = {a_s[3 * b], a_s[3 * b + 1], a_s[3 * b + 2]};
           HP J[6];
           bvec_hp(nd, av, J);
 #pragma unroll
@@ -616,14 +986,18 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
         }
         HP sl[6], sr[6], DL, DR, XL, XR;
         Rec<TF> rr;
+        // FP64: the leaves' tangents by their parts (an isotropic one minus a
+        // rank-one term), not as 21 components
+        constexpr bool PARTS = D64 && LAW < 3;
+        LeafTan<TF> tl, tr;
         if (LAW == 3 && mp_s[ph0].kind == 3)
           leaf_pa66<TF, HP>(mp_s[ph0], mpa_s[ph0], el, zn0, trn0, sl, DL, XL, rec, zw0);
         else
-          leaf_eval<TF, HP, LAW>(mp_s[ph0], el, zn0, trn0, sl, DL, XL, rec, zw0, full);
+          leaf_eval<TF, HP, LAW, PARTS>(mp_s[ph0], el, zn0, trn0, sl, DL, XL, rec, zw0, full, &tl);
         if (LAW == 3 && mp_s[ph1].kind == 3)
           leaf_pa66<TF, HP>(mp_s[ph1], mpa_s[ph1], er, zn1, trn1, sr, DR, XR, rr, zw1);
         else
-          leaf_eval<TF, HP, LAW>(mp_s[ph1], er, zn1, trn1, sr, DR, XR, rr, zw1, full);
+          leaf_eval<TF, HP, LAW, PARTS>(mp_s[ph1], er, zn1, trn1, sr, DR, XR, rr, zw1, full, &tr);
         if (full) {
           Dsum = wL * DL + wR * DR;
           Xsum = wL * XL + wR * XR;
@@ -637,22 +1011,41 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
         HP rbh[3];
         btvec_hp(nd, dsh, rbh);  // B^T (sigma_L - sigma_R) = r_t / (w c1 c2)
         TF n[3], c1, c2, iwcc, wcc;
-        load_node_tf(P, t, n, c1, c2, iwcc, wcc);
+        load_node_tf(P, b, n, c1, c2, iwcc, wcc);
         const TF rbv[3] = {tf_of(rbh[0], (TF *)nullptr), tf_of(rbh[1], (TF *)nullptr),
                            tf_of(rbh[2], (TF *)nullptr)};
         r2 = wcc * wcc * (rbv[0] * rbv[0] + rbv[1] * rbv[1] + rbv[2] * rbv[2]);
-        combine<TF>(rec, rr, n, c1, c2, rbv, gh_s + 21 * t, full);
+        if constexpr (PARTS) combine_leaves(rec, rr, tl, tr, nd, rbv, gh_s + 21 * b, full);
+        else if constexpr (D64) combine_d(rec, rr, nd, rbv, gh_s + 21 * b, full);
+        else combine<TF>(rec, rr, n, c1, c2, rbv, gh_s + 21 * b, full);
         if (K == 1) put_root(rec, S);
       }
-      // ---- level K-1: neighbouring lanes (2j, 2j+1) ----
+      // ---- level K-1.  FP64: node j on thread j < G/2, which formed its left
+      //      child; the right child's record comes through shared memory, in
+      //      the slot that then takes the node's own.  Mixed: neighbouring
+      //      lanes (2j, 2j+1) ----
       if (K >= 2) {
         Rec<TF> other;
-        rec_shfl_down(other, rec, 1, mask, W);
         HP So[6];
+        if constexpr (D64) {
+          if (t >= G / 2) {
+            rec_put(recX + RS * (t - G / 2), rec);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) So[c] = hp_shfl_down(mask, S[c], 1, W);
-        if ((t & 1) == 0) {
-          const int j = t >> 1;
+            for (int c = 0; c < 6; ++c) Sx[6 * (t - G / 2) + c] = S[c];
+          }
+          __syncthreads();
+        } else {
+          rec_shfl_down(other, rec, 1, mask, W);
+#pragma unroll
+          for (int c = 0; c < 6; ++c) So[c] = hp_shfl_down(mask, S[c], 1, W);
+        }
+        if (D64 ? t < G / 2 : (t & 1) == 0) {
+          const int j = D64 ? t : t >> 1;
+          if constexpr (D64) {
+            rec_get(other, recX + RS * j);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) So[c] = Sx[6 * j + c];
+          }
           const int p = (1 << K) - (1 << (K - 1)) + j;
           NodeHP<HP> nd;
           load_node(P, p, nd);
@@ -670,7 +1063,8 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
                             tf_of(rh[2], (TF *)nullptr)};
           r2 += rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
           const TF rbv[3] = {rv[0] * iwcc, rv[1] * iwcc, rv[2] * iwcc};
-          combine<TF>(rec, other, n, c1, c2, rbv, gh_s + 21 * p, full);
+          if constexpr (D64) combine_d(rec, other, nd, rbv, gh_s + 21 * p, full);
+          else combine<TF>(rec, other, n, c1, c2, rbv, gh_s + 21 * p, full);
           if (K >= 3) {
             rec_put(recX + RS * j, rec);
 #pragma unroll
@@ -688,10 +1082,14 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       //      move to the reduction barrier.  A CTA of fewer than 8 threads
       //      (K = 3) condenses its root on one thread. ----
       if (G >= 8) {
+        // lanes per node.  FP64: as many as keep the warps full: one on levels of
+        // 64 and more nodes, two (combine_half) on 8 to 32, eight below
+        // (K = 8: 9.9 k -> about 5.8 k FP64 warp instructions per pass)
+        auto lanes_of = [&](int k) { return !D64 || k <= 3 ? 8 : (k <= 6 ? 2 : 1); };
         for (int k = K - 2; k >= 1; --k) {
-          const int ntask = 8 << (k - 1);
+          const int lpn = lanes_of(k), ntask = lpn << (k - 1);
           const bool wide = ntask > 32 && G > 32;
-          const bool prod_wide = k + 1 == K - 1 ? G > 32 : (2 * ntask > 32 && G > 32);
+          const bool prod_wide = k + 1 == K - 1 ? G > 32 : ((lanes_of(k + 1) << k) > 32 && G > 32);
           if (prod_wide) __syncthreads();
           if (!wide) {  // this level and the ones above: warp L alone
             if (warp != L) break;
@@ -704,7 +1102,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
             if (qb + (q0 & ~31) >= ntask) break;  // the whole warp is past the level
             const int q = qb + q0;
             const bool st = q < ntask;            // else a copy of the last node, not stored
-            const int j = st ? q >> 3 : cnt - 1;
+            const int j = st ? q / lpn : cnt - 1;
             const int p = (1 << K) - (1 << k) + j;
             // children: slots 2j, 2j + 1 of level k + 1's buffer (debug build: checked)
             const int cap = ((K - 1 - (k + 1)) & 1) ? sc_.GY : sc_.GX;
@@ -718,6 +1116,16 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
               const int js = DMN_IDX(j, ((K - 1 - k) & 1) ? sc_.GY : sc_.GX);
               dst = recbuf(k) + RS * js;
               sd = sbuf(k) + 6 * js;
+            }
+            if constexpr (D64) {
+              if (lpn == 1) {
+                combine_node(P, p, rc, rc + RS, sc, sc + 6, dst, sd, gh_s + 21 * p, r2, full);
+                continue;
+              }
+              if (lpn == 2) {
+                combine_half(P, p, q & 1, st, mask, rc, rc + RS, sc, sc + 6, dst, sd, gh_s + 21 * p, r2, full);
+                continue;
+              }
             }
             combine_rows<TF, HP>(P, p, q & 7, st, mask, rc, rc + RS, sc, sc + 6, dst, sd, gh_s + 21 * p, r2,
                                  full, k == 1);
@@ -749,7 +1157,8 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
                             tf_of(rh[2], (TF *)nullptr)};
           r2 += rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
           const TF rbv[3] = {rv[0] * iwcc, rv[1] * iwcc, rv[2] * iwcc};
-          combine<TF>(rec, other, n, c1, c2, rbv, gh_s + 21 * p, full);
+          if constexpr (D64) combine_d(rec, other, nd, rbv, gh_s + 21 * p, full);
+          else combine<TF>(rec, other, n, c1, c2, rbv, gh_s + 21 * p, full);
           put_root(rec, S);
         }
       }
