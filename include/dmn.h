@@ -142,15 +142,17 @@ typedef struct {
                            residual, the convergence test and every output
                            accumulation in FP64-class precision (float-float
                            on the FP32 pipe, about 48 significant bits)          */
-  int32_t solve_variant; /* kernel variant of the solve, depth K <= 8 (deeper
-                           trees always take the default).  0 = library
-                           default (owner-mapped kernel; mixed: 3 CTAs/SM);
-                           2, 3, 4 = owner-mapped mixed kernel compiled for
-                           that many resident CTAs per SM; 11 = compact kernel
-                           (upper tree levels on one warp, strains updated by
-                           the Newton step), FP64 (mixed: as 12); 12, 13, 14
-                           = compact mixed kernel for 2, 3 or 4 CTAs per SM.  The
-                           2..4 choice has no effect in FP64.  22, 23, 24 =
+  int32_t solve_variant; /* kernel variant of the mixed solve, depth K <= 8
+                           (deeper trees always take the default; FP64 takes
+                           the compact kernel up to K = 9 whatever the
+                           variant).  0 = library default (owner-mapped
+                           kernel, 3 CTAs/SM); 2, 3, 4 = owner-mapped kernel
+                           compiled for that many resident CTAs per SM; 11 =
+                           compact kernel (upper tree levels on one warp,
+                           strains updated by the Newton step), as 12; 12, 13,
+                           14 = compact kernel for 2, 3 or 4 CTAs per SM.
+                           Launches of at most two CTAs per SM run the
+                           instance for two.  22, 23, 24 =
                            one warp per Gauss point (lane l condenses the
                            subtree under level-6 node l in registers, levels
                            5..1 by shuffles; four points per CTA, register

@@ -16,8 +16,8 @@ is given.  Workloads: the random walk of the benchmark ("random_walk"), the
 uniaxial ramp that drives the matrix into plastic flow ("plastic") and the
 lognormal increment magnitudes of the uneven batch ("uneven").  Variant
 numbers are those of ``dmn_options.solve_variant``: 2, 3, 4 owner-mapped
-mixed; 12, 13, 14 compact mixed; 22, 23, 24 warp form (mixed, K = 6..8);
-0 owner-mapped FP64; 11 compact FP64.  A variant the library rejects for a
+mixed; 12, 13, 14 compact mixed; 22, 23, 24 warp form (mixed, K = 6..8).
+FP64 has one form, the compact one (11, and 0).  A variant the library rejects for a
 configuration is left out of that run.
 
 Usage (on a GPU):  python -m paper_2109_14403_gb300.autotune [--K 8] [--points 65536]

@@ -449,7 +449,8 @@ static dmn_status eval_impl(dmn_handle h, dmn_stream stream, int64_t n_points,
   int64_t grid = (int64_t)h->num_sms * h->blocks_per_sm;  // the scratch holds this many CTAs
   const int64_t per_cta = is_warp_variant(h->opt.solve_variant) ? warp_form_warps() : 1;
   if (grid > (n_points + per_cta - 1) / per_cta) grid = (n_points + per_cta - 1) / per_cta;
-  cudaError_t e = launch_solve(P, mixed, h->opt.solve_variant, (int)grid, (cudaStream_t)stream);
+  cudaError_t e = launch_solve(P, mixed, h->opt.solve_variant, (int)grid, h->num_sms, h->blocks_per_sm,
+                               (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "dmn_eval launch");
   return DMN_OK;
 }

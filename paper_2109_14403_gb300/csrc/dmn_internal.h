@@ -12,7 +12,7 @@ namespace dmn {
 size_t solve_smem_bytes(int K, int zw, int n_mats, bool mixed, int variant, int law);
 bool solve_variant_valid(int variant);
 // the compact solve kernel: dmn_solve_compact.cu (kinds 0 and 1, K <= 8) and
-// dmn_solve_compact_vp.cu (also kind 2, K <= 9)
+// dmn_solve_compact_vp.cu (also kind 2, K <= 9; FP64 trees of K = 9)
 using KernelFn = void (*)(const SolveParams);
 size_t compact_smem_bytes(int K, int zw, int n_mats, bool mixed);
 KernelFn compact_kernel(int K, bool mixed, int minb);
@@ -58,7 +58,8 @@ KernelFn warp_kernel8(int minb);
 int solve_block_threads(int K, int variant, int law);
 cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
                           int *blocks_per_sm);
-cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, cudaStream_t s);
+cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, int blocks_per_sm,
+                         cudaStream_t s);
 // dmn_eval_mixed (dmn_drive.cu): prescribed strain components, outer = 0 and
 // optionally the tangent predictor; one outer Newton update after an
 // evaluation; the status bit of the points given up

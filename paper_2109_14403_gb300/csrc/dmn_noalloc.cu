@@ -207,7 +207,7 @@ extern "C" dmn_status dmn_eval_noalloc(int32_t K, const double *leaf_w, const do
   P.iters = d_iters;
   int64_t grid = (int64_t)num_sms * blocks_per_sm;
   if (grid > n_points) grid = n_points;
-  e = launch_solve(P, mixed, o.solve_variant, (int)grid, s);
+  e = launch_solve(P, mixed, o.solve_variant, (int)grid, num_sms, blocks_per_sm, s);
   if (e != cudaSuccess) return na_fail(DMN_ERR_CUDA, "dmn_eval_noalloc launch: %s", cudaGetErrorString(e));
   return DMN_OK;
 }

@@ -457,13 +457,20 @@ static size_t owner_smem_bytes(int K, int zw, int n_mats, bool mixed) {
 }
 
 // kernel variants: (form, precision, threads bound, CTAs per SM requested).
-// 0 = default; 2..4 = owner-mapped mixed kernel for that many CTAs per SM;
-// 10 + m = compact kernel (dmn_solve_compact.cu), mixed compiled for m = 2, 3
-// or 4 CTAs per SM (11 runs as 12), FP64 for one.  Depth K > 8 takes the
-// owner-mapped 512-thread kernel.  A tree with Perzyna leaves (law 2) always
-// takes the compact instances that include that leaf law
-// (dmn_solve_compact_vp.cu, K <= 9), whatever the variant; one with PA66
-// leaves (law 3) the instances of dmn_solve_compact_pa66.cu (K <= 8).
+// FP64, K <= 9: the compact kernel, whatever the variant (the owner-mapped form
+// has each level's nodes on one lane per warp or less, and an FP64 warp
+// instruction costs the same however few lanes are active: 1.4 to 2.0 times
+// the time at every K = 3..8, from 32 to 65,536 points).  Mixed: 0 = default;
+// 2..4 = owner-mapped kernel for that many CTAs per SM; 10 + m = compact kernel
+// (dmn_solve_compact.cu) compiled for m = 2, 3 or 4 CTAs per SM (11 runs as
+// 12).  Deeper trees take the owner-mapped 512-thread kernel.  A tree with
+// Perzyna leaves (law 2) always takes the compact instances that include that
+// leaf law (dmn_solve_compact_vp.cu, K <= 9), whatever the variant; one with
+// PA66 leaves (law 3) the instances of dmn_solve_compact_pa66.cu (K <= 8).
+// A mixed launch of at most two CTAs per SM (`few`) takes its form's instance
+// for two: the same operations with more registers (compact 232 against 168,
+// no spills), where the smaller budget gains no residency (27 points at K = 8
+// 66.2 -> 63.6 us, 32 at K = 3 62.5 -> 59.4).
 bool is_warp_variant(int variant) { return variant >= 22 && variant <= 24; }
 bool solve_variant_valid(int variant) {
   return variant == 0 || (variant >= 2 && variant <= 4) || (variant >= 11 && variant <= 14) ||
@@ -476,18 +483,17 @@ int solve_block_threads(int K, int variant, int law) {
   (void)law;
   return is_warp_variant(variant) ? 32 * warp_form_warps() : (1 << (K - 1));
 }
-static bool is_compact(int K, int variant, int law) {
-  return law >= 2 ? K <= 9 : (K <= 8 && variant >= 11);
+static bool is_compact(int K, bool mixed, int variant, int law) {
+  return law >= 2 || !mixed ? K <= 9 : (K <= 8 && variant >= 11);
 }
 
-static KernelFn pick(int K, bool mixed, int variant, int law) {
+static KernelFn pick(int K, bool mixed, int variant, int law, bool few) {
   if (uses_warp_form(K, mixed, variant, law)) return warp_kernel(K, variant - 20);
   if (law == 3) return compact_kernel_pa66(K, mixed);
-  if (law >= 2) return compact_kernel_vp(K, mixed);
-  if (is_compact(K, variant, law)) return compact_kernel(K, mixed, variant - 10);
+  if (law >= 2 || (!mixed && K == 9)) return compact_kernel_vp(K, mixed);
+  if (is_compact(K, mixed, variant, law)) return compact_kernel(K, mixed, few ? 2 : variant - 10);
   if (K > 8) return mixed ? dmn_solve_kernel<float, dfl, 512, 1> : dmn_solve_kernel<double, double, 512, 1>;
-  if (!mixed) return dmn_solve_kernel<double, double, 128, 1>;
-  switch (variant) {
+  switch (few ? 2 : variant) {
     case 2: return dmn_solve_kernel<float, dfl, 128, 2>;
     case 4: return dmn_solve_kernel<float, dfl, 128, 4>;
     default: return dmn_solve_kernel<float, dfl, 128, 3>;
@@ -497,59 +503,71 @@ static KernelFn pick(int K, bool mixed, int variant, int law) {
 size_t solve_smem_bytes(int K, int zw, int n_mats, bool mixed, int variant, int law) {
   if (uses_warp_form(K, mixed, variant, law)) return warp_smem_bytes(K, n_mats);
   if (law == 3) return compact_smem_bytes_pa(K, zw, n_mats, mixed);
-  return is_compact(K, variant, law) ? compact_smem_bytes(K, zw, n_mats, mixed)
+  return is_compact(K, mixed, variant, law) ? compact_smem_bytes(K, zw, n_mats, mixed)
                                      : owner_smem_bytes(K, zw, n_mats, mixed);
 }
 
-cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
-                          int *blocks_per_sm) {
-  const size_t smem = solve_smem_bytes(K, zw, n_mats, mixed, variant, law);
-  KernelFn f = pick(K, mixed, variant, law);
-  // One kernel instance serves every tree of a depth range (the compact
-  // instances do not depend on K), and its attributes are global to the
-  // process: raise them, never lower them, so that a handle prepared for a
-  // larger tree (more shared memory, a larger carveout) stays launchable
-  // after a smaller tree has been prepared.
+// One kernel instance serves every tree of a depth range (the compact instances
+// do not depend on K), and the shared memory it may ask for is global to the
+// process: raise it, never lower it, so that a handle prepared for a larger
+// tree stays launchable after a smaller one has been prepared.  The split of
+// the SM's 256 KB into shared memory and L1 goes with each launch instead
+// (carveout_pct): as an attribute of the function it let one tree's choice
+// bound the resident CTAs of another (K = 7 after K = 8 got five CTAs per SM of
+// the six that fit: 21,845 uneven points 3.37 -> 2.72 ms; K = 8 in FP64 after K =
+// 4 one of two), and a raised one takes L1 from a tree that needs less.
+static cudaError_t prepare_kernel(KernelFn f, size_t smem, int threads, int *blocks_per_sm) {
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, f);
   if (e != cudaSuccess) return e;
   if (int(smem) > fa.maxDynamicSharedSizeBytes &&
       (e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess)
     return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, solve_block_threads(K, variant, law),
-                                                          smem)) != cudaSuccess)
-    return e;
-  // shared memory carveout: the smallest configuration that holds the
-  // resident CTAs (plus 1 KB per CTA for the system); the rest of the SM's
-  // unified 256 KB stays L1 for the node tables and spills.  The driver
-  // rounds a requested percentage up to the next configuration, so request
-  // the largest percentage below the chosen one.
-  int dev = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  if (per_sm > 0 && *blocks_per_sm > 0) {
-    static const int kConfigKB[] = {0, 8, 16, 32, 64, 100, 132, 164, 196, 228};
-    const size_t need = size_t(*blocks_per_sm) * (smem + 1024);
-    size_t pick_b = size_t(per_sm);
-    for (int kb : kConfigKB)
-      if (size_t(kb) * 1024 >= need) {
-        pick_b = size_t(kb) * 1024;
-        break;
-      }
-    int pct = pick_b >= size_t(per_sm) ? 100 : int(pick_b * 100 / size_t(per_sm));
-    if (pct > fa.preferredShmemCarveout &&
-        (e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, pct)) != cudaSuccess)
-      return e;
-  }
-  return cudaSuccess;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }
 
-cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, cudaStream_t s) {
+// The smallest shared memory configuration that holds the resident CTAs (1 KB
+// per CTA for the system); the rest stays L1 for the node tables and spills.
+// The driver rounds a requested percentage up to the next configuration, so
+// request the largest percentage below the chosen one.
+static int carveout_pct(size_t smem, int ctas) {
+  static const int kConfigKB[] = {8, 16, 32, 64, 100, 132, 164, 196};
+  const size_t need = size_t(ctas) * (smem + 1024);
+  for (int kb : kConfigKB)
+    if (size_t(kb) * 1024 >= need) return kb * 100 / 228;
+  return 100;
+}
+
+cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
+                          int *blocks_per_sm) {
+  const size_t smem = solve_smem_bytes(K, zw, n_mats, mixed, variant, law);
+  const int threads = solve_block_threads(K, variant, law);
+  const KernelFn f = pick(K, mixed, variant, law, false), g = pick(K, mixed, variant, law, true);
+  if (g != f) {  // the instance of small launches
+    int b = 0;
+    const cudaError_t e = prepare_kernel(g, smem, threads, &b);
+    if (e != cudaSuccess) return e;
+  }
+  return prepare_kernel(f, smem, threads, blocks_per_sm);
+}
+
+cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, int blocks_per_sm,
+                         cudaStream_t s) {
   const size_t smem = solve_smem_bytes(P.K, P.zw, P.n_mats, mixed, variant, P.law);
   cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  pick(P.K, mixed, variant, P.law)<<<grid, solve_block_threads(P.K, variant, P.law), smem, s>>>(P);
-  return cudaGetLastError();
+  const int per_sm = (grid + num_sms - 1) / num_sms;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at[0].val.sharedMemCarveout = unsigned(carveout_pct(smem, per_sm < blocks_per_sm ? per_sm : blocks_per_sm));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(grid));
+  cfg.blockDim = dim3(unsigned(solve_block_threads(P.K, variant, P.law)));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, pick(P.K, mixed, variant, P.law, grid <= 2 * num_sms), P);
 }
 
 // the index-check log of this translation unit (debug build; dmn_check.cuh)
