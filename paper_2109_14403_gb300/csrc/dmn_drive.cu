@@ -7,76 +7,101 @@
 namespace dmn {
 namespace {
 
-// LU with partial pivoting on an m x m system (m <= 7), in place; false when
-// a pivot vanishes
-__device__ bool small_solve(double A[7][7], double b[7], int m) {
-  for (int k = 0; k < m; ++k) {
-    int piv = k;
-    double best = fabs(A[k][k]);
-    for (int r = k + 1; r < m; ++r)
-      if (fabs(A[r][k]) > best) {
-        best = fabs(A[r][k]);
-        piv = r;
-      }
-    if (!(best > 0.0)) return false;
-    if (piv != k) {
-      for (int c = 0; c < m; ++c) {
-        const double t = A[k][c];
-        A[k][c] = A[piv][c];
-        A[piv][c] = t;
-      }
-      const double t = b[k];
-      b[k] = b[piv];
-      b[piv] = t;
-    }
-    for (int r = k + 1; r < m; ++r) {
-      const double f = A[r][k] / A[k][k];
-      for (int c = k; c < m; ++c) A[r][c] -= f * A[k][c];
-      b[r] -= f * b[k];
-    }
+constexpr int kUpdThreads = 32, kWorkThreads = 128;
+
+// LU with partial pivoting on a 7 x 7 system, in registers (every index is a
+// constant after unrolling; rows are exchanged by selects); false when a pivot
+// vanishes.  Pivots by the leading 32 bits of the magnitudes (integer
+// comparisons; an FP64 instruction takes 64 cycles of a warp here), one
+// reciprocal per column: about 300 FP64 instructions a point.  (With the
+// system in local memory and a division per row the 4,096-point predictor took
+// 44 us.)
+template <int k>
+__device__ __forceinline__ void lu_column(double A[7][7], double b[7], double inv[7], bool &ok) {
+  unsigned best = unsigned(__double2hiint(A[k][k])) & 0x7fffffffu;
+  int piv = k;
+#pragma unroll
+  for (int r = k + 1; r < 7; ++r) {
+    const unsigned m = unsigned(__double2hiint(A[r][k])) & 0x7fffffffu;
+    piv = m > best ? r : piv;
+    best = m > best ? m : best;
   }
-  for (int k = m - 1; k >= 0; --k) {
-    double s = b[k];
-    for (int c = k + 1; c < m; ++c) s -= A[k][c] * b[c];
-    b[k] = s / A[k][k];
+#pragma unroll
+  for (int r = k + 1; r < 7; ++r) {
+    const bool sw = piv == r;
+#pragma unroll
+    for (int c = k; c < 7; ++c) {
+      const double x = A[k][c], y = A[r][c];
+      A[k][c] = sw ? y : x;
+      A[r][c] = sw ? x : y;
+    }
+    const double x = b[k], y = b[r];
+    b[k] = sw ? y : x;
+    b[r] = sw ? x : y;
   }
-  return true;
+  ok = ok && best != 0u;
+  inv[k] = 1.0 / A[k][k];
+#pragma unroll
+  for (int r = k + 1; r < 7; ++r) {
+    const double f = A[r][k] * inv[k];
+#pragma unroll
+    for (int c = k + 1; c < 7; ++c) A[r][c] = fma(-f, A[k][c], A[r][c]);
+    b[r] = fma(-f, b[k], b[r]);
+  }
+}
+__device__ __forceinline__ bool solve7(double A[7][7], double b[7]) {
+  double inv[7];
+  bool ok = true;
+  lu_column<0>(A, b, inv, ok);
+  lu_column<1>(A, b, inv, ok);
+  lu_column<2>(A, b, inv, ok);
+  lu_column<3>(A, b, inv, ok);
+  lu_column<4>(A, b, inv, ok);
+  lu_column<5>(A, b, inv, ok);
+  lu_column<6>(A, b, inv, ok);
+#pragma unroll
+  for (int k = 6; k >= 0; --k) {
+#pragma unroll
+    for (int c = 6; c > 0; --c)
+      if (c > k) b[k] = fma(-A[k][c], b[c], b[k]);
+    b[k] *= inv[k];
+  }
+  return ok;
 }
 
-// Unknowns of a point under mask m: the stress-prescribed components (bits
-// 0..5) in order, then theta when adiabatic (bit 6); returns their number.
-__device__ int unknowns(unsigned m, int unk[7]) {
-  int nu = 0;
-  for (int c = 0; c < 6; ++c)
-    if ((m >> c) & 1u) unk[nu++] = c;
-  if ((m >> 6) & 1u) unk[nu++] = 6;
-  return nu;
-}
-
-// One Newton step on the unknowns: r holds the residuals (stress rows, then
-// the heat balance c (theta - theta^n)/dt - D_bar), o the outputs whose
-// tangents form the Jacobian.  Adds the step to deps / theta; false when the
-// system is singular (nothing changed).
-__device__ bool newton_step(const int unk[7], int nu, const double *o, double c_heat, double dt,
-                            const double r[7], double *deps, double *theta) {
+// One Newton step on a point's unknowns under mask m: the stress-prescribed
+// strain increments (bits 0..5) and theta when adiabatic (bit 6); the others'
+// rows and columns are the identity's.  r holds the residuals of the unknowns'
+// equations (stress rows, then the heat balance c (theta - theta^n)/dt -
+// D_bar), o the outputs whose tangents form the Jacobian.  Adds the step to
+// deps / theta; false when the system is singular (nothing changed).
+__device__ __forceinline__ bool newton_step(unsigned m, const double *o, double c_heat, double dt,
+                                            const double r[7], double *deps, double *theta) {
   double A[7][7], b[7];
-  for (int a = 0; a < nu; ++a) {
-    for (int q = 0; q < nu; ++q) {
-      const int ra = unk[a], cq = unk[q];
-      double v;
-      if (ra < 6) v = cq < 6 ? o[6 + 6 * ra + cq] : o[42 + ra];  // d sigma / d eps, d sigma / d theta
-      else v = cq < 6 ? -o[49 + cq] : c_heat / dt - o[55];       // heat balance
+#pragma unroll
+  for (int a = 0; a < 7; ++a) {
+    const bool ua = (m >> a) & 1u;
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      const bool u = ua && ((m >> q) & 1u);
+      double v = a == q ? 1.0 : 0.0;
+      if (u) {
+        if (a < 6) v = q < 6 ? o[6 + 6 * a + q] : o[42 + a];  // d sigma / d eps, d sigma / d theta
+        else v = q < 6 ? -o[49 + q] : c_heat / dt - o[55];    // heat balance
+      }
       A[a][q] = v;
     }
-    b[a] = -r[a];
+    b[a] = ua ? -r[a] : 0.0;
   }
-  if (!small_solve(A, b, nu)) return false;
-  for (int a = 0; a < nu; ++a)
-    if (!isfinite(b[a])) return false;
-  for (int a = 0; a < nu; ++a) {
-    if (unk[a] < 6) deps[unk[a]] += b[a];
-    else *theta += b[a];
-  }
+  if (!solve7(A, b)) return false;
+  bool fin = true;
+#pragma unroll
+  for (int a = 0; a < 7; ++a) fin = fin && isfinite(b[a]);
+  if (!fin) return false;
+#pragma unroll
+  for (int a = 0; a < 6; ++a)
+    if ((m >> a) & 1u) deps[a] += b[a];
+  if ((m >> 6) & 1u) *theta += b[6];
   return true;
 }
 
@@ -86,7 +111,7 @@ __device__ bool newton_step(const int unk[7], int nu, const double *o, double c_
 //   sigma ~ sigma^n + C deps + C_theta (theta - theta^n),
 //   D ~ D_eps . deps + D_theta (theta - theta^n),
 // for the prescribed stresses and the heat balance.
-__global__ void k_mixed_prepare(int64_t n, int sw, const uint8_t *mask, const double *target,
+__global__ void __launch_bounds__(kUpdThreads) k_mixed_prepare(int64_t n, int sw, const uint8_t *mask, const double *target,
                                 double *deps, double *theta, double dt, double c_heat,
                                 const double *sin, const double *out, int predict, int32_t *outer) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
@@ -97,28 +122,30 @@ __global__ void k_mixed_prepare(int64_t n, int sw, const uint8_t *mask, const do
     for (int c = 0; c < 6; ++c)
       if (!((m >> c) & 1u)) e[c] = tg[c];
     outer[i] = 0;
-    int unk[7];
-    const int nu = unknowns(m, unk);
-    if (!predict || nu == 0) continue;
+    if (!predict || (m & 0x7fu) == 0u) continue;
     const double *o = out + i * 57;
     const double thn = sin[i * sw + 6];
     const bool adiabatic = (m >> 6) & 1u;
     double x[6], th = adiabatic ? thn : theta[i];
     for (int c = 0; c < 6; ++c) x[c] = ((m >> c) & 1u) ? 0.0 : tg[c];
     double r[7];
-    for (int a = 0; a < nu; ++a) {
-      const int c = unk[a];
-      double v;
+#pragma unroll
+    for (int c = 0; c < 7; ++c) {
+      double v = 0.0;
       if (c < 6) {
-        v = o[c] - tg[c] + o[42 + c] * (th - thn);
-        for (int q = 0; q < 6; ++q) v += o[6 + 6 * c + q] * x[q];
-      } else {
+        if ((m >> c) & 1u) {
+          v = o[c] - tg[c] + o[42 + c] * (th - thn);
+#pragma unroll
+          for (int q = 0; q < 6; ++q) v += o[6 + 6 * c + q] * x[q];
+        }
+      } else if (adiabatic) {
         v = (c_heat / dt - o[55]) * (th - thn);
+#pragma unroll
         for (int q = 0; q < 6; ++q) v -= o[49 + q] * x[q];
       }
-      r[a] = v;
+      r[c] = v;
     }
-    if (newton_step(unk, nu, o, c_heat, dt, r, x, &th)) {
+    if (newton_step(m, o, c_heat, dt, r, x, &th)) {
       for (int c = 0; c < 6; ++c) e[c] = x[c];
       theta[i] = th;
     }
@@ -128,18 +155,15 @@ __global__ void k_mixed_prepare(int64_t n, int sw, const uint8_t *mask, const do
 // Residuals of the prescribed stresses and of the heat balance at the last
 // evaluation; a point that meets them is done (outer = +evaluations), one that
 // cannot go on is given up (outer = -evaluations), any other takes one Newton
-// step on (unknown deps components, theta) and is counted in *open.  Also
-// writes the next evaluation's warm-start increment (its a - a^n).
-__global__ void k_mixed_update(int64_t n, int sw, int n3, const uint8_t *mask, const double *target,
-                               double *deps, double *theta, double dt, double c_heat, double tol,
-                               const double *sin, const double *sout, const double *out,
-                               const int32_t *status, int32_t *outer, int it, int last, float *work,
-                               unsigned long long *open) {
+// step on (unknown deps components, theta) and is counted in *open.  One point
+// a thread: a serial FP64 chain, in CTAs of one warp so that a small batch
+// spreads over the SMs.
+__global__ void __launch_bounds__(kUpdThreads)
+    k_mixed_update(int64_t n, int sw, const uint8_t *mask, const double *target, double *deps, double *theta,
+                   double dt, double c_heat, double tol, const double *sin, const double *out,
+                   const int32_t *status, int32_t *outer, int it, int last, unsigned long long *open) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n;
        i += int64_t(gridDim.x) * blockDim.x) {
-    if (work)
-      for (int j = 0; j < n3; ++j)
-        work[i * n3 + j] = float(sout[i * sw + 8 + j] - sin[i * sw + 8 + j]);
     if (outer[i] != 0) continue;  // settled in an earlier evaluation
     const unsigned m = mask[i];
     const double *o = out + i * 57;
@@ -149,18 +173,18 @@ __global__ void k_mixed_update(int64_t n, int sw, int n3, const uint8_t *mask, c
     }
     double smax = 1.0;
     for (int c = 0; c < 6; ++c) smax = fmax(smax, fabs(o[c]));
-    int unk[7];
-    const int nu = unknowns(m, unk);
     double r[7];
     bool ok = true;
-    for (int a = 0; a < nu; ++a) {
-      const int c = unk[a];
+#pragma unroll
+    for (int c = 0; c < 7; ++c) {
+      r[c] = 0.0;
+      if (!((m >> c) & 1u)) continue;
       if (c < 6) {
-        r[a] = o[c] - target[i * 6 + c];
-        if (!(fabs(r[a]) <= tol * smax)) ok = false;
+        r[c] = o[c] - target[i * 6 + c];
+        if (!(fabs(r[c]) <= tol * smax)) ok = false;
       } else {
-        r[a] = c_heat * (theta[i] - sin[i * sw + 6]) / dt - o[48];
-        if (!(fabs(r[a]) <= tol * c_heat / dt)) ok = false;
+        r[c] = c_heat * (theta[i] - sin[i * sw + 6]) / dt - o[48];
+        if (!(fabs(r[c]) <= tol * c_heat / dt)) ok = false;
       }
     }
     if (ok) {
@@ -171,11 +195,28 @@ __global__ void k_mixed_update(int64_t n, int sw, int n3, const uint8_t *mask, c
       outer[i] = -(it + 1);
       continue;
     }
-    if (!newton_step(unk, nu, o, c_heat, dt, r, deps + i * 6, theta + i)) {
+    if (!newton_step(m, o, c_heat, dt, r, deps + i * 6, theta + i)) {
       outer[i] = -(it + 1);
       continue;
     }
     atomicAdd(open, 1ull);
+  }
+}
+
+// The next evaluation's warm-start increment a - a^n of the points still open
+// (the solve skips the others), one warp a point, lanes along the jumps: bound
+// by its 20 bytes per jump.  (Inside k_mixed_update a thread walked its own
+// point's 765 jumps: 360 us at K = 8, 4,096 points, most of them settled.)
+__global__ void __launch_bounds__(kWorkThreads)
+    k_mixed_work(int64_t n, int sw, int n3, const double *sin, const double *sout, const int32_t *outer,
+                 float *work) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarp = (int64_t(gridDim.x) * kWorkThreads) >> 5;
+  for (int64_t i = (blockIdx.x * int64_t(kWorkThreads) + threadIdx.x) >> 5; i < n; i += nwarp) {
+    if (outer[i] != 0) continue;
+    const double *a = sin + i * sw + 8, *b = sout + i * sw + 8;
+#pragma unroll 4
+    for (int j = lane; j < n3; j += 32) work[i * n3 + j] = float(b[j] - a[j]);
   }
 }
 
@@ -189,8 +230,8 @@ __global__ void k_mixed_finish(int64_t n, int32_t *status, int32_t *outer) {
     }
 }
 
-int blocks_for(int64_t n) {
-  int64_t b = (n + 127) / 128;
+int blocks_for(int64_t n, int threads = 128) {
+  int64_t b = (n + threads - 1) / threads;
   return int(b > 65535 ? 65535 : (b < 1 ? 1 : b));
 }
 
@@ -200,7 +241,7 @@ cudaError_t mixed_prepare(cudaStream_t s, int64_t n, int sw, const uint8_t *mask
                           const double *target, double *deps, double *theta, double dt,
                           double c_heat, const double *sin, const double *out, bool predict,
                           int32_t *outer) {
-  k_mixed_prepare<<<blocks_for(n), 128, 0, s>>>(n, sw, mask, target, deps, theta, dt, c_heat, sin,
+  k_mixed_prepare<<<blocks_for(n, kUpdThreads), kUpdThreads, 0, s>>>(n, sw, mask, target, deps, theta, dt, c_heat, sin,
                                                 out, predict ? 1 : 0, outer);
   return cudaGetLastError();
 }
@@ -210,9 +251,11 @@ cudaError_t mixed_update(cudaStream_t s, int64_t n, int sw, int n3, const uint8_
                          double tol, const double *sin, const double *sout, const double *out,
                          const int32_t *status, int32_t *outer, int it, bool last, float *work,
                          unsigned long long *open) {
-  k_mixed_update<<<blocks_for(n), 128, 0, s>>>(n, sw, n3, mask, target, deps, theta, dt, c_heat, tol,
-                                               sin, sout, out, status, outer, it, last ? 1 : 0, work,
-                                               open);
+  k_mixed_update<<<blocks_for(n, kUpdThreads), kUpdThreads, 0, s>>>(n, sw, mask, target, deps, theta, dt, c_heat,
+                                                                    tol, sin, out, status, outer, it, last ? 1 : 0,
+                                                                    open);
+  if (work)
+    k_mixed_work<<<blocks_for(n * 32, kWorkThreads), kWorkThreads, 0, s>>>(n, sw, n3, sin, sout, outer, work);
   return cudaGetLastError();
 }
 
