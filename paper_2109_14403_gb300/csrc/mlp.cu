@@ -50,36 +50,75 @@ bool make_map(CUtensorMap *map, const void *ptr, uint64_t rows, uint64_t cols, u
 int g_gemm_configured_dev = -1;
 int g_gemm_sms = 0;
 
-// C = A . B^T with the fused epilogue ep; A [M x K], B [N x K] bf16.  N a
-// multiple of 256: the persistent wide form (one CTA per SM), else the tile
-// form.
-cudaError_t gemm(cudaStream_t s, const void *A, const void *B, int M, int N, int K, EpiArgs ep) {
-  if (M % BM || N % BN || K % BK || M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
-  if (M / BM > 65535 || N / BN > 65535) return cudaErrorInvalidValue;  // grid limits
-  if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) return cudaErrorInvalidValue;
+cudaError_t gemm_setup() {
   cudaError_t e = get_encode();
   if (e != cudaSuccess) return e;
   int dev = 0;
-  cudaGetDevice(&dev);
-  if (g_gemm_configured_dev != dev) {
-    e = cudaFuncSetAttribute(gemm_bf16_tn, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(gemm_bf16_tn_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, WGEMM_SMEM);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_gemm_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    g_gemm_configured_dev = dev;
-  }
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (g_gemm_configured_dev == dev) return cudaSuccess;
+  const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  e = cudaFuncSetAttribute(gemm_bf16_tile<false, false, BN, STAGES>, smem, GEMM_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tile<false, true, BN, STAGES>, smem, GEMM_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_bf16_wgrad, smem, tile_smem(WG_BN, WG_ST));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tn_wide, smem, WGEMM_SMEM);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_gemm_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) g_gemm_configured_dev = dev;
+  return e;
+}
+bool gemm_args_ok(const void *A, const void *B, int M, int N, int K) {
+  return M % BM == 0 && N % BN == 0 && K % BK == 0 && M > 0 && N > 0 && K > 0 && M / BM <= 65535 &&
+         N / BN <= 65535 &&  // grid limits
+         !((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15);
+}
+
+// C = A . B^T with the fused epilogue ep; A [M x K], B [N x K] bf16; rows of A
+// from a_rows on read as zero.  N a multiple of 256 and a 128 x 256 tile for
+// every SM: the persistent wide form (one CTA per SM), else (and with z_out or
+// the loss, the training step's) the tile form, whose 128 x 128 tiles spread a
+// product over twice the SMs (4,096 rows, a hidden layer: 18 -> 12 us).
+cudaError_t gemm(cudaStream_t s, const void *A, const void *B, int M, int N, int K, EpiArgs ep, int64_t a_rows) {
+  if (!gemm_args_ok(A, B, M, N, K)) return cudaErrorInvalidValue;
+  cudaError_t e = gemm_setup();
+  if (e != cudaSuccess) return e;
   CUtensorMap ma, mb;
-  if (N % WBN == 0) {
-    if (!make_map(&ma, A, M, K) || !make_map(&mb, B, N, K, WBN)) return cudaErrorInvalidValue;
+  if (!make_map(&ma, A, a_rows, K)) return cudaErrorInvalidValue;
+  if (N % WBN == 0 && (M / BM) * (N / WBN) >= g_gemm_sms && !ep.z_out && ep.mode != EPI_LOSS) {
+    CUtensorMap mh = ma;  // unused unless the activation leaves by TMA
+    if (!make_map(&mb, B, N, K, WBN) || (ep.mode == EPI_BIAS_SILU && !make_map(&mh, ep.h_out, M, N, 32)))
+      return cudaErrorInvalidValue;
     const int tiles = (M / BM) * (N / WBN);
-    gemm_bf16_tn_wide<<<tiles < g_gemm_sms ? tiles : g_gemm_sms, 64 + 32 * WEPI, WGEMM_SMEM, s>>>(ma, mb, M, N,
+    gemm_bf16_tn_wide<<<tiles < g_gemm_sms ? tiles : g_gemm_sms, 64 + 32 * WEPI, WGEMM_SMEM, s>>>(ma, mb, mh, M, N,
                                                                                               K, ep);
     return cudaGetLastError();
   }
-  if (!make_map(&ma, A, M, K) || !make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
-  gemm_bf16_tn<<<dim3(N / BN, M / BM), 128, GEMM_SMEM, s>>>(ma, mb, K, ep);
+  if (!make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
+  gemm_bf16_tile<false, false, BN, STAGES><<<dim3(N / BN, M / BM), 128, GEMM_SMEM, s>>>(ma, mb, K, ep);
   return cudaGetLastError();
+}
+// input gradient: C [M x N] = A . B, A [M x K], B [K x N] as stored
+cudaError_t gemm_dgrad(cudaStream_t s, const void *A, const void *B, int M, int N, int K, EpiArgs ep) {
+  if (!gemm_args_ok(A, B, M, N, K)) return cudaErrorInvalidValue;
+  cudaError_t e = gemm_setup();
+  if (e != cudaSuccess) return e;
+  CUtensorMap ma, mb;
+  if (!make_map(&ma, A, M, K) || !make_map(&mb, B, K, N, BK)) return cudaErrorInvalidValue;
+  gemm_bf16_tile<false, true, BN, STAGES><<<dim3(N / BN, M / BM), 128, GEMM_SMEM, s>>>(ma, mb, K, ep);
+  return cudaGetLastError();
+}
+// adds layer l's weight gradient to a launch: C [M x N] (fp32) = A^T . B, A [K x
+// M], B [K x N] (rows from b_rows on read as zero)
+bool wgrad_add(WgradArgs &W, const void *A, const void *B, int M, int N, int K, float *C, int64_t b_rows) {
+  const int l = W.layers;
+  if (l >= kMaxLayers || !gemm_args_ok(A, B, M, N, K) || !make_map(&W.a[l], A, K, M, BK) ||
+      !make_map(&W.b[l], B, b_rows, N, BK))
+    return false;
+  W.nx[l] = N / WG_BN;
+  W.ldc[l] = N;
+  W.out[l] = C;
+  W.blk0[l + 1] = W.blk0[l] + W.nx[l] * (M / BM);
+  W.layers = l + 1;
+  return true;
 }
 
 int64_t rup(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
@@ -94,17 +133,16 @@ unsigned blocks_for(int64_t n, int t = 256) {
 // the network input converts 768 words per row.  Magnitudes outside the
 // normal float range (and NaN) take the FP64 conversion; zero and double
 // subnormals give a signed zero.
+// (the conversion as a call: otherwise every lane issues it under a false
+// predicate, which kept the FP64 pipe 55 % busy)
+__device__ __noinline__ float f32_rn_call(double d) { return __double2float_rn(d); }
 __device__ __forceinline__ float f32_rn(double d) {
-  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(d));
-  const unsigned E = unsigned(b >> 52) & 0x7ffu;
-  const unsigned sign = unsigned(b >> 32) & 0x80000000u;
-  if (E == 0u) return __uint_as_float(sign);
-  if (E < 897u || E > 1150u) return __double2float_rn(d);
-  const unsigned long long mant = b & ((1ull << 52) - 1);
-  unsigned r = sign | ((E - 896u) << 23) | unsigned(mant >> 29);
-  const unsigned rem = unsigned(mant & ((1ull << 29) - 1)), half = 1u << 28;
-  if (rem > half || (rem == half && (r & 1u))) r += 1u;  // a carry moves into the exponent
-  return __uint_as_float(r);
+  const unsigned hi = unsigned(__double2hiint(d)), lo = unsigned(__double2loint(d));
+  const unsigned t = hi & 0x7fffffffu, sign = hi & 0x80000000u;
+  if (t - (897u << 20) >= (254u << 20)) return t < (1u << 20) ? __uint_as_float(sign) : f32_rn_call(d);
+  unsigned r = __funnelshift_l(lo, t - (896u << 20), 3);        // exponent and 23 bits, truncated
+  r += (lo & 0x1fffffffu) + (r & 1u) > 0x10000000u ? 1u : 0u;  // to nearest, ties to even; a carry moves into the exponent
+  return __uint_as_float(sign | r);
 }
 
 // feature c of a row: deps (6), theta^{n+1}, theta^{n+1} - theta^n,
@@ -133,10 +171,14 @@ __global__ void k_features(int64_t n, int n3, int sw, const double *deps, const 
 
 // features of k_features, normalised and rounded to bf16 in one pass: one
 // warp per row, each lane two adjacent columns per step (one bf16x2 store;
-// ld = kin is a multiple of 128, so the pairs stay 4-byte aligned)
-__global__ void k_features_norm(int64_t n, int n3, int sw, int ld, const double *deps,
-                                const double *theta, const double *sin, const double *sprev,
-                                const float *mean, const float *inv, bf16 *x) {
+// ld = kin is a multiple of 128, so the pairs stay 4-byte aligned).  Bound by the
+// two states' jumps it reads (12 KB a row at K = 8).  VEC: a lane's pair of jumps
+// as one 16-byte load, four steps in flight (states 16-byte aligned, an even
+// number of words); else word by word.
+template <bool VEC>
+__global__ void __launch_bounds__(256)
+    k_features_norm(int64_t n, int n3, int sw, int ld, const double *deps, const double *theta, const double *sin,
+                    const double *sprev, const float *mean, const float *inv, bf16 *x) {
   const int nin = 8 + n3 + kExtraFeatures;
   const int lane = threadIdx.x & 31;
   const int64_t nwarp = (int64_t(gridDim.x) * blockDim.x) >> 5;
@@ -144,18 +186,46 @@ __global__ void k_features_norm(int64_t n, int n3, int sw, int ld, const double 
     const double *a = sin + r * sw;
     const double *ap = sprev ? sprev + r * sw : nullptr;
     __nv_bfloat162 *xr = reinterpret_cast<__nv_bfloat162 *>(x + r * ld);
-    for (int c0 = 2 * lane; c0 < ld; c0 += 64) {
-      float v[2];
+    auto put = [&](int c0, float f0, float f1) {  // features of columns c0, c0 + 1
+      float v0 = 0.0f, v1 = 0.0f;
+      if (c0 < nin) v0 = (f0 - __ldg(mean + c0)) * __ldg(inv + c0);
+      if (c0 + 1 < nin) v1 = (f1 - __ldg(mean + c0 + 1)) * __ldg(inv + c0 + 1);
+      xr[c0 >> 1] = __floats2bfloat162_rn(v0, v1);
+    };
+    if (VEC && ap) {
+      constexpr int U = 4;
+      for (int c0 = 2 * lane; c0 < ld; c0 += 64 * U) {
+        double2 q[U], p[U];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int c = c0 + u;
-        v[u] = 0.0f;
-        if (c < nin) {
-          const float f = feature(c, n3, deps + r * 6, theta[r], a, ap);
-          v[u] = (f - mean[c]) * inv[c];
+        for (int u = 0; u < U; ++u) {
+          const int c = c0 + 64 * u;
+          const bool in = c >= 8 && c + 1 < sw && c < nin;  // c + 1 == nin: the word after the jumps
+          q[u] = in ? __ldcs(reinterpret_cast<const double2 *>(a + c)) : make_double2(0.0, 0.0);
+          p[u] = in ? __ldcs(reinterpret_cast<const double2 *>(ap + c)) : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int c = c0 + 64 * u;
+          if (c >= ld) break;
+          if (c < 8 || c + 1 >= sw) {  // the load's features; a state that ends with the jumps
+            float f[2];
+#pragma unroll
+            for (int w = 0; w < 2; ++w)
+              f[w] = c + w < nin ? feature(c + w, n3, deps + r * 6, theta[r], a, ap) : 0.0f;
+            put(c, f[0], f[1]);
+          } else {
+            put(c, f32_rn(q[u].x) - f32_rn(p[u].x), f32_rn(q[u].y) - f32_rn(p[u].y));
+          }
         }
       }
-      xr[c0 >> 1] = __floats2bfloat162_rn(v[0], v[1]);
+    } else {
+      for (int c0 = 2 * lane; c0 < ld; c0 += 64) {
+        float f[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          f[u] = c0 + u < nin ? feature(c0 + u, n3, deps + r * 6, theta[r], a, ap) : 0.0f;
+        put(c0, f[0], f[1]);
+      }
     }
   }
 }
@@ -231,70 +301,104 @@ __global__ void k_norm_t(int64_t n, int nout, int ld, const float *tgt, const fl
   }
 }
 
-// dst[c][r] = src[r][c] for a rows x cols bf16 matrix (32 x 32 tiles)
-__global__ void k_transpose(int rows, int cols, const bf16 *src, bf16 *dst) {
-  __shared__ bf16 tile[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int r = r0 + j, c = c0 + threadIdx.x;
-    if (r < rows && c < cols) tile[j][threadIdx.x] = src[size_t(r) * cols + c];
+// Bias gradients of every layer in one launch: the column sums of dZ_l [npad x
+// C_l], 64 columns a CTA, 32 warps over the rows; the last block adds up the
+// loss (the warps' sums of squares, FP64, fixed order).
+struct ColsumArgs {
+  int layers, npad, nloss, blk0[kMaxLayers + 1];  // first block of each layer
+  const bf16 *dz[kMaxLayers];
+  float *db[kMaxLayers];
+  int cols[kMaxLayers];
+  const float *loss_part;
+  float *loss, lscale;
+};
+__global__ void __launch_bounds__(1024) k_colsum(const ColsumArgs A) {
+  __shared__ float2 red[32][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (int(blockIdx.x) == A.blk0[A.layers]) {
+    __shared__ double rl[32];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < A.nloss; i += 1024) s += double(A.loss_part[i]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) rl[warp] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 32; ++w) s += rl[w];
+      *A.loss = float(s * double(A.lscale));
+    }
+    return;
   }
+  int l = 0;
+  while (int(blockIdx.x) >= A.blk0[l + 1]) ++l;
+  const int c = (int(blockIdx.x) - A.blk0[l]) * 64 + 2 * lane, C = A.cols[l];
+  const bf16 *p = A.dz[l] + c;
+  float2 s = {0.0f, 0.0f};
+#pragma unroll 32
+  for (int r = warp; r < A.npad; r += 32) {
+    const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p + size_t(r) * C));
+    s.x += v.x;
+    s.y += v.y;
+  }
+  red[warp][lane] = s;
   __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int c = c0 + j, r = r0 + threadIdx.x;
-    if (r < rows && c < cols) dst[size_t(c) * rows + r] = tile[threadIdx.x][j];
+  // pairwise over the warps (the tree of a warp's shuffle reduction)
+  for (int o = 16; o > 0; o >>= 1) {
+    if (warp < o) {
+      red[warp][lane].x += red[warp + o][lane].x;
+      red[warp][lane].y += red[warp + o][lane].y;
+    }
+    __syncthreads();
   }
-}
-
-// MSE on normalised targets: dY = 2 (y - t) / (n n_out) on valid rows and
-// columns, 0 elsewhere; bf16 copy and (through a 32 x 32 shared tile) a
-// transposed copy; loss sum.  Block (32, 8) per tile of 32 rows x 32 columns.
-__global__ void k_loss(int n, int npad, int nout, int ld, const float *y, const float *t, bf16 *dz,
-                       bf16 *dzt, float *loss, float scale) {
-  __shared__ bf16 tile[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  float part = 0.0f;
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int r = r0 + j, c = c0 + threadIdx.x;
-    const size_t i = size_t(r) * ld + c;
-    const float d = (r < n && c < nout) ? y[i] - t[i] : 0.0f;
-    part += d * d;
-    const bf16 g = __float2bfloat16(2.0f * d * scale);
-    dz[i] = g;
-    tile[j][threadIdx.x] = g;
-  }
-  __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += 8)
-    dzt[size_t(c0 + j) * npad + r0 + threadIdx.x] = tile[threadIdx.x][j];
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-  if (threadIdx.x == 0 && loss) atomicAdd(loss, part * scale);
-}
-
-// db[i] = sum_j dzt[i][j] (one warp per row)
-__global__ void k_rowsum(int rows, int cols, const bf16 *dzt, float *db) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  float s = 0.0f;
-  for (int j = lane; j < cols; j += 32) s += __bfloat162float(dzt[size_t(row) * cols + j]);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  if (lane == 0) db[row] = s;
+  if (warp == 0) *reinterpret_cast<float2 *>(A.db[l] + c) = red[0][lane];
 }
 
 // AMSGrad with bias correction (Reddi, Kale, Kumar 2018; the maximum of the
 // second-moment estimates replaces it in the step size)
-__global__ void k_amsgrad(int64_t count, float *w, const float *g, float *m, float *v, float *vmax,
-                          float lr, float b1, float b2, float eps, float bc1, float bc2) {
+struct AmsArgs {
+  float lr, b1, b2, eps, bc1, bc2;
+};
+__device__ __forceinline__ void amsgrad_elem(float &w, float gi, float &m, float &v, float &vmax, const AmsArgs &a) {
+  const float mi = a.b1 * m + (1.0f - a.b1) * gi;
+  const float vi = a.b2 * v + (1.0f - a.b2) * gi * gi;
+  const float vm = fmaxf(vmax, vi);
+  m = mi;
+  v = vi;
+  vmax = vm;
+  w -= a.lr * (mi / a.bc1) / (sqrtf(vm / a.bc2) + a.eps);
+}
+__global__ void k_amsgrad(int64_t count, float *w, const float *g, float *m, float *v, float *vmax, AmsArgs a) {
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < count;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    const float vm = fmaxf(vmax[i], vi);
-    m[i] = mi;
-    v[i] = vi;
-    vmax[i] = vm;
-    w[i] -= lr * (mi / bc1) / (sqrtf(vm / bc2) + eps);
+       i += int64_t(gridDim.x) * blockDim.x)
+    amsgrad_elem(w[i], g[i], m[i], v[i], vmax[i], a);
+}
+// The same for the network's parameters, four a thread, with the bf16 weights
+// of the next pass (every layer's count and offset are multiples of four)
+struct PackArgs {
+  int layers;
+  int64_t ow[kMaxLayers], ob[kMaxLayers];  // weights of layer l: [ow, ob)
+  bf16 *w[kMaxLayers];
+};
+__global__ void __launch_bounds__(256)
+    k_amsgrad_pack(int64_t count4, float4 *w, const float4 *g, float4 *m, float4 *v, float4 *vmax, AmsArgs a,
+                   const PackArgs P) {
+  const int64_t i = blockIdx.x * int64_t(256) + threadIdx.x;
+  if (i >= count4) return;
+  const float4 gi = g[i];
+  float4 wi = w[i], mi = m[i], vi = v[i], xi = vmax[i];
+  amsgrad_elem(wi.x, gi.x, mi.x, vi.x, xi.x, a);
+  amsgrad_elem(wi.y, gi.y, mi.y, vi.y, xi.y, a);
+  amsgrad_elem(wi.z, gi.z, mi.z, vi.z, xi.z, a);
+  amsgrad_elem(wi.w, gi.w, mi.w, vi.w, xi.w, a);
+  w[i] = wi;
+  m[i] = mi;
+  v[i] = vi;
+  vmax[i] = xi;
+  int l = 0;
+  while (l + 1 < P.layers && 4 * i >= P.ow[l + 1]) ++l;
+  if (4 * i < P.ob[l]) {
+    __nv_bfloat162 *o = reinterpret_cast<__nv_bfloat162 *>(P.w[l] + (4 * i - P.ow[l]));
+    o[0] = __floats2bfloat162_rn(wi.x, wi.y);
+    o[1] = __floats2bfloat162_rn(wi.z, wi.w);
   }
 }
 
@@ -304,23 +408,14 @@ constexpr float kBeta1 = 0.9f, kBeta2 = 0.999f, kEps = 1e-8f;
 // One AMSGrad step at iteration step >= 1.  The bias corrections 1 - b^t are
 // formed in FP64 from the FP32 betas and rounded once: in FP32, 1 - powf(b2, t)
 // for b2 near 1 would lose about 5 of its 24 bits to cancellation.
-cudaError_t amsgrad(cudaStream_t s, int64_t n, float *w, const float *g, float *m, float *v, float *vmax,
-                    float lr, float b1, float b2, float eps, int64_t step) {
-  const float bc1 = float(1.0 - pow(double(b1), double(step)));
-  const float bc2 = float(1.0 - pow(double(b2), double(step)));
-  k_amsgrad<<<blocks_for(n), 256, 0, s>>>(n, w, g, m, v, vmax, lr, b1, b2, eps, bc1, bc2);
-  return cudaGetLastError();
+AmsArgs ams_args(float lr, float b1, float b2, float eps, int64_t step) {
+  return {lr, b1, b2, eps, float(1.0 - pow(double(b1), double(step))), float(1.0 - pow(double(b2), double(step)))};
 }
 
-// bf16 weights and their transpose from the fp32 master copy
-__global__ void k_pack(int rows, int cols, const float *w32, bf16 *w, bf16 *wt) {
-  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < int64_t(rows) * cols;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    const int r = int(i / cols), c = int(i - int64_t(r) * cols);
-    const bf16 b = __float2bfloat16(w32[i]);
-    w[i] = b;
-    wt[size_t(c) * rows + r] = b;
-  }
+// bf16 weights from the fp32 master copy
+__global__ void k_pack(int64_t n, const float *w32, bf16 *w) {
+  for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    w[i] = __float2bfloat16(w32[i]);
 }
 
 uint64_t splitmix(uint64_t &s) {
@@ -339,11 +434,11 @@ struct dmn_mlp_s {
   std::vector<int64_t> ow, ob;
   int64_t nparam;
   float *params, *grads, *m, *v, *vmax;
-  std::vector<bf16 *> w, wt;
+  std::vector<bf16 *> w;
   float *fmean, *finv, *tmean, *tstd, *tinv;
-  bf16 *x, *xt;
-  std::vector<bf16 *> z, h, ht, dz, dzt;
-  float *y, *t;
+  bf16 *x;
+  std::vector<bf16 *> z, h, dz;
+  float *t, *lpart;
   double *acc;
   int *err;
   int step;
@@ -366,15 +461,12 @@ dmn_status cuda_fail(cudaError_t e, const char *what) {
 void free_mlp(dmn_mlp p) {
   if (!p) return;
   void *bufs[] = {p->params, p->grads, p->m, p->v, p->vmax, p->fmean, p->finv, p->tmean, p->tstd,
-                  p->tinv, p->x, p->xt, p->y, p->t, p->acc, p->err};
+                  p->tinv, p->x, p->t, p->lpart, p->acc, p->err};
   for (void *b : bufs) cudaFree(b);
   for (auto *b : p->w) cudaFree(b);
-  for (auto *b : p->wt) cudaFree(b);
   for (auto *b : p->z) cudaFree(b);
   for (auto *b : p->h) cudaFree(b);
-  for (auto *b : p->ht) cudaFree(b);
   for (auto *b : p->dz) cudaFree(b);
-  for (auto *b : p->dzt) cudaFree(b);
   delete p;
 }
 template <typename T>
@@ -383,51 +475,57 @@ cudaError_t dalloc(T **p, size_t count) {
 }
 cudaError_t pack_all(dmn_mlp p, cudaStream_t s) {
   for (int l = 0; l < p->L; ++l) {
-    k_pack<<<blocks_for(int64_t(p->dout[l]) * p->din[l]), 256, 0, s>>>(
-        p->dout[l], p->din[l], p->params + p->ow[l], p->w[l], p->wt[l]);
+    const int64_t n = int64_t(p->dout[l]) * p->din[l];
+    k_pack<<<blocks_for(n), 256, 0, s>>>(n, p->params + p->ow[l], p->w[l]);
   }
   return cudaGetLastError();
 }
-// copy a batch into the padded workspace (rows n..npad zeroed)
-cudaError_t stage_x(dmn_mlp p, cudaStream_t s, int64_t n, int64_t npad, const void *x) {
-  const size_t row = sizeof(bf16) * p->kin;
-  cudaError_t e = cudaMemcpyAsync(p->x, x, row * n, cudaMemcpyDeviceToDevice, s);
-  if (e == cudaSuccess && npad > n) e = cudaMemsetAsync(p->x + n * p->kin, 0, row * (npad - n), s);
-  return e;
+// the batch's rows, copied into the workspace only if TMA cannot read them
+// where they are (16-byte alignment); rows from n on are read as zero
+cudaError_t stage_x(dmn_mlp p, cudaStream_t s, int64_t n, const void *x, const bf16 **in) {
+  *in = static_cast<const bf16 *>(x);
+  if (!(reinterpret_cast<uintptr_t>(x) & 15)) return cudaSuccess;
+  *in = p->x;
+  return cudaMemcpyAsync(p->x, x, sizeof(bf16) * p->kin * n, cudaMemcpyDeviceToDevice, s);
 }
-// forward pass; train = keep pre-activations and transposed activations
-cudaError_t forward(dmn_mlp p, cudaStream_t s, int64_t n, int64_t npad, bool train, float *da,
+// forward pass; t: training, the loss against these targets into dz of the last
+// layer (and pre-activations kept), else the prediction into da
+cudaError_t forward(dmn_mlp p, cudaStream_t s, int64_t n, int64_t npad, const float *t, float *da,
                     const bf16 *x_in) {
   cudaError_t e = cudaSuccess;
   const bf16 *in = x_in;
+  int64_t rows = n;
   for (int l = 0; l < p->L; ++l) {
     EpiArgs ep;
     memset(&ep, 0, sizeof(ep));
     ep.err = p->err;
     ep.bias = p->params + p->ob[l];
     ep.ldc = p->dout[l];
-    ep.ldt = int(npad);
     if (l < p->L - 1) {
       ep.mode = EPI_BIAS_SILU;
-      ep.z_out = train ? p->z[l] : nullptr;  // pre-activations only for the backward pass
+      ep.z_out = t ? p->z[l] : nullptr;  // pre-activations only for the backward pass
       ep.h_out = p->h[l];
-      ep.t_out = train ? p->ht[l] : nullptr;
     } else {
-      ep.mode = EPI_BIAS_F32;
-      if (train) {
-        ep.f_out = p->y;
+      ep.m_valid = int(n);
+      ep.n_valid = p->n3;
+      if (t) {
+        ep.mode = EPI_LOSS;
+        ep.target = t;
+        ep.gscale = 1.0f / (float(n) * float(p->n3));
+        ep.loss_part = p->lpart;
+        ep.h_out = p->dz[l];
       } else {
+        ep.mode = EPI_BIAS_F32;
         ep.f_out = da;
         ep.scale = p->tstd;
         ep.shift = p->tmean;
-        ep.m_valid = int(n);
-        ep.n_valid = p->n3;
         ep.ld_f = p->n3;
       }
     }
-    e = gemm(s, in, p->w[l], int(npad), p->dout[l], p->din[l], ep);
+    e = gemm(s, in, p->w[l], int(npad), p->dout[l], p->din[l], ep, rows);
     if (e != cudaSuccess) return e;
     if (l < p->L - 1) in = p->h[l];
+    rows = npad;
   }
   return e;
 }
@@ -468,34 +566,29 @@ extern "C" dmn_status dmn_mlp_create(dmn_mlp *out, int32_t K, int32_t hidden, in
   p->step = 0;
   p->params = p->grads = p->m = p->v = p->vmax = nullptr;
   p->fmean = p->finv = p->tmean = p->tstd = p->tinv = nullptr;
-  p->x = p->xt = nullptr;
-  p->y = p->t = nullptr;
+  p->x = nullptr;
+  p->t = p->lpart = nullptr;
   p->acc = nullptr;
   p->err = nullptr;
   p->w.assign(p->L, nullptr);
-  p->wt.assign(p->L, nullptr);
   p->z.assign(p->nh, nullptr);
   p->h.assign(p->nh, nullptr);
-  p->ht.assign(p->nh, nullptr);
   p->dz.assign(p->L, nullptr);
-  p->dzt.assign(p->L, nullptr);
   const int64_t B = p->bmax;
   bool ok = dalloc(&p->params, p->nparam) == cudaSuccess && dalloc(&p->grads, p->nparam) == cudaSuccess &&
             dalloc(&p->m, p->nparam) == cudaSuccess && dalloc(&p->v, p->nparam) == cudaSuccess &&
             dalloc(&p->vmax, p->nparam) == cudaSuccess && dalloc(&p->fmean, p->kin) == cudaSuccess &&
             dalloc(&p->finv, p->kin) == cudaSuccess && dalloc(&p->tmean, p->nout_pad) == cudaSuccess &&
             dalloc(&p->tstd, p->nout_pad) == cudaSuccess && dalloc(&p->tinv, p->nout_pad) == cudaSuccess &&
-            dalloc(&p->x, B * p->kin) == cudaSuccess && dalloc(&p->xt, B * p->kin) == cudaSuccess &&
-            dalloc(&p->y, B * p->nout_pad) == cudaSuccess && dalloc(&p->t, B * p->nout_pad) == cudaSuccess &&
+            dalloc(&p->x, B * p->kin) == cudaSuccess && dalloc(&p->t, B * p->nout_pad) == cudaSuccess &&
+            dalloc(&p->lpart, (B / BM) * (p->nout_pad / BN) * 4) == cudaSuccess &&
             dalloc(&p->acc, 2 * int64_t(p->kin > p->nout_pad ? p->kin : p->nout_pad)) == cudaSuccess &&
             dalloc(&p->err, 1) == cudaSuccess;
   for (int l = 0; ok && l < p->L; ++l)
     ok = dalloc(&p->w[l], int64_t(p->din[l]) * p->dout[l]) == cudaSuccess &&
-         dalloc(&p->wt[l], int64_t(p->din[l]) * p->dout[l]) == cudaSuccess &&
-         dalloc(&p->dz[l], B * p->dout[l]) == cudaSuccess && dalloc(&p->dzt[l], B * p->dout[l]) == cudaSuccess;
+         dalloc(&p->dz[l], B * p->dout[l]) == cudaSuccess;
   for (int l = 0; ok && l < p->nh; ++l)
-    ok = dalloc(&p->z[l], B * hidden) == cudaSuccess && dalloc(&p->h[l], B * hidden) == cudaSuccess &&
-         dalloc(&p->ht[l], B * hidden) == cudaSuccess;
+    ok = dalloc(&p->z[l], B * hidden) == cudaSuccess && dalloc(&p->h[l], B * hidden) == cudaSuccess;
   if (!ok) {
     free_mlp(p);
     return fail(DMN_ERR_OOM, "dmn_mlp_create: device allocation failed");
@@ -573,7 +666,9 @@ extern "C" dmn_status dmn_mlp_input(dmn_mlp m, dmn_stream stream, int64_t n, con
   if (!m || n < 0 || !d_deps || !d_theta || !d_state_in || !d_x_bf16 || state_words < 8 + m->n3)
     return fail(DMN_ERR_ARG, "dmn_mlp_input: invalid argument");
   if (n == 0) return DMN_OK;
-  k_features_norm<<<blocks_for(n * 32), 256, 0, (cudaStream_t)stream>>>(
+  const bool vec = ((reinterpret_cast<uintptr_t>(d_state_in) | reinterpret_cast<uintptr_t>(d_state_prev)) & 15) == 0 &&
+                   (state_words & 1) == 0;
+  (vec ? k_features_norm<true> : k_features_norm<false>)<<<blocks_for(n * 32), 256, 0, (cudaStream_t)stream>>>(
       n, m->n3, int(state_words), m->kin, d_deps, d_theta, d_state_in, d_state_prev, m->fmean,
       m->finv, static_cast<bf16 *>(d_x_bf16));
   cudaError_t e = cudaGetLastError();
@@ -642,48 +737,59 @@ extern "C" dmn_status dmn_mlp_train_step(dmn_mlp m, dmn_stream stream, int64_t n
     return fail(DMN_ERR_ARG, "dmn_mlp_train_step: invalid argument");
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t npad = rup(n, 128);
-  cudaError_t e = stage_x(m, s, n, npad, d_x_bf16);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(m->t, d_t, sizeof(float) * m->nout_pad * n, cudaMemcpyDeviceToDevice, s);
-  if (e == cudaSuccess && d_loss) e = cudaMemsetAsync(d_loss, 0, sizeof(float), s);
-  if (e != cudaSuccess) return cuda_fail(e, "dmn_mlp_train_step staging");
-  k_transpose<<<dim3((m->kin + 31) / 32, unsigned((npad + 31) / 32)), dim3(32, 8), 0, s>>>(
-      int(npad), m->kin, m->x, m->xt);
-  if ((e = forward(m, s, n, npad, true, nullptr, m->x)) != cudaSuccess) return cuda_fail(e, "forward");
-  const int Lo = m->L - 1;
-  k_loss<<<dim3(m->nout_pad / 32, unsigned(npad / 32)), dim3(32, 8), 0, s>>>(
-      int(n), int(npad), m->n3, m->nout_pad, m->y, m->t, m->dz[Lo], m->dzt[Lo], d_loss,
-      1.0f / (float(n) * float(m->n3)));
-  for (int l = Lo; l >= 0; --l) {
-    // weight gradient dW_l = dZ_l^T . input_l  (reduction over the batch)
-    EpiArgs ep;
-    memset(&ep, 0, sizeof(ep));
-    ep.err = m->err;
-    ep.mode = EPI_F32;
-    ep.f_out = m->grads + m->ow[l];
-    ep.ldc = m->din[l];
-    const bf16 *inT = l == 0 ? m->xt : m->ht[l - 1];
-    if ((e = gemm(s, m->dzt[l], inT, m->dout[l], m->din[l], int(npad), ep)) != cudaSuccess)
-      return cuda_fail(e, "wgrad");
-    k_rowsum<<<(m->dout[l] + 7) / 8, 256, 0, s>>>(m->dout[l], int(npad), m->dzt[l], m->grads + m->ob[l]);
-    if (l > 0) {  // input gradient through W_l and silu' of the layer below
-      EpiArgs ed;
-      memset(&ed, 0, sizeof(ed));
-      ed.err = m->err;
-      ed.mode = EPI_DSILU;
-      ed.z_in = m->z[l - 1];
-      ed.h_out = m->dz[l - 1];
-      ed.t_out = m->dzt[l - 1];
-      ed.ldc = m->H;
-      ed.ldt = int(npad);
-      if ((e = gemm(s, m->dz[l], m->wt[l], int(npad), m->din[l], m->dout[l], ed)) != cudaSuccess)
-        return cuda_fail(e, "dgrad");
-    }
+  const bf16 *x = nullptr;
+  const float *t = d_t;
+  cudaError_t e = stage_x(m, s, n, d_x_bf16, &x);
+  if (e == cudaSuccess && (reinterpret_cast<uintptr_t>(d_t) & 15)) {
+    t = m->t;
+    e = cudaMemcpyAsync(m->t, d_t, sizeof(float) * m->nout_pad * n, cudaMemcpyDeviceToDevice, s);
   }
+  if (e != cudaSuccess) return cuda_fail(e, "dmn_mlp_train_step staging");
+  if ((e = forward(m, s, n, npad, t, nullptr, x)) != cudaSuccess) return cuda_fail(e, "forward");
+  for (int l = m->L - 1; l > 0; --l) {  // input gradient through W_l and silu' of the layer below
+    EpiArgs ed;
+    memset(&ed, 0, sizeof(ed));
+    ed.err = m->err;
+    ed.mode = EPI_DSILU;
+    ed.z_in = m->z[l - 1];
+    ed.h_out = m->dz[l - 1];
+    ed.ldc = m->H;
+    if ((e = gemm_dgrad(s, m->dz[l], m->w[l], int(npad), m->din[l], m->dout[l], ed)) != cudaSuccess)
+      return cuda_fail(e, "dgrad");
+  }
+  WgradArgs wg = {};  // weight gradients dW_l = dZ_l^T . input_l (reduction over the batch)
+  wg.err = m->err;
+  for (int l = 0; l < m->L; ++l)
+    if (!wgrad_add(wg, m->dz[l], l == 0 ? x : m->h[l - 1], m->dout[l], m->din[l], int(npad), m->grads + m->ow[l],
+                   l == 0 ? n : npad))
+      return cuda_fail(cudaErrorInvalidValue, "wgrad");
+  gemm_bf16_wgrad<<<wg.blk0[m->L], 128, tile_smem(WG_BN, WG_ST), s>>>(wg, int(npad));
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "wgrad");
+  ColsumArgs C = {};
+  PackArgs P = {};
+  C.layers = P.layers = m->L;
+  C.npad = int(npad);
+  for (int l = 0; l < m->L; ++l) {
+    C.dz[l] = m->dz[l];
+    C.db[l] = m->grads + m->ob[l];
+    C.cols[l] = m->dout[l];
+    C.blk0[l + 1] = C.blk0[l] + m->dout[l] / 64;
+    P.ow[l] = m->ow[l];
+    P.ob[l] = m->ob[l];
+    P.w[l] = m->w[l];
+  }
+  C.nloss = int(npad / BM) * (m->nout_pad / BN) * 4;
+  C.loss_part = m->lpart;
+  C.loss = d_loss;
+  C.lscale = 1.0f / (float(n) * float(m->n3));
+  k_colsum<<<C.blk0[m->L] + (d_loss ? 1 : 0), 1024, 0, s>>>(C);
   m->step += 1;
-  if ((e = amsgrad(s, m->nparam, m->params, m->grads, m->m, m->v, m->vmax, lr, kBeta1, kBeta2, kEps,
-                   m->step)) != cudaSuccess)
-    return cuda_fail(e, "amsgrad");
-  if ((e = pack_all(m, s)) != cudaSuccess) return cuda_fail(e, "pack");
+  const int64_t n4 = m->nparam / 4;
+  k_amsgrad_pack<<<unsigned((n4 + 255) / 256), 256, 0, s>>>(
+      n4, reinterpret_cast<float4 *>(m->params), reinterpret_cast<const float4 *>(m->grads),
+      reinterpret_cast<float4 *>(m->m), reinterpret_cast<float4 *>(m->v), reinterpret_cast<float4 *>(m->vmax),
+      ams_args(lr, kBeta1, kBeta2, kEps, m->step), P);
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dmn_mlp_train_step");
   return DMN_OK;
 }
 
@@ -697,7 +803,9 @@ extern "C" dmn_status dmn_mlp_amsgrad(dmn_stream stream, int64_t n, float *d_w, 
   if (!(beta1 >= 0.0f && beta1 < 1.0f) || !(beta2 >= 0.0f && beta2 < 1.0f) || !(eps > 0.0f) ||
       !isfinite(lr))
     return fail(DMN_ERR_ARG, "dmn_mlp_amsgrad: 0 <= beta < 1, eps > 0 required");
-  cudaError_t e = amsgrad((cudaStream_t)stream, n, d_w, d_g, d_m, d_v, d_vmax, lr, beta1, beta2, eps, step);
+  k_amsgrad<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(n, d_w, d_g, d_m, d_v, d_vmax,
+                                                             ams_args(lr, beta1, beta2, eps, step));
+  const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? DMN_OK : cuda_fail(e, "dmn_mlp_amsgrad");
 }
 
@@ -718,13 +826,9 @@ extern "C" dmn_status dmn_mlp_predict(dmn_mlp m, dmn_stream stream, int64_t n, c
   if (n == 0) return DMN_OK;
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t npad = rup(n, 128);
-  cudaError_t e = cudaSuccess;
-  const bf16 *xin = static_cast<const bf16 *>(d_x_bf16);
-  if (npad != n || (reinterpret_cast<uintptr_t>(d_x_bf16) & 15)) {  // pad into the workspace
-    e = stage_x(m, s, n, npad, d_x_bf16);
-    xin = m->x;
-  }
-  if (e == cudaSuccess) e = forward(m, s, n, npad, false, d_da, xin);
+  const bf16 *x = nullptr;
+  cudaError_t e = stage_x(m, s, n, d_x_bf16, &x);
+  if (e == cudaSuccess) e = forward(m, s, n, npad, nullptr, d_da, x);
   return e == cudaSuccess ? DMN_OK : cuda_fail(e, "dmn_mlp_predict");
 }
 
@@ -771,6 +875,6 @@ extern "C" dmn_status dmn_gemm_bf16_tn(dmn_stream stream, int32_t M, int32_t N, 
   ep.mode = EPI_F32;
   ep.f_out = d_c;
   ep.ldc = N;
-  cudaError_t e = gemm((cudaStream_t)stream, d_a, d_b, M, N, K, ep);
+  cudaError_t e = gemm((cudaStream_t)stream, d_a, d_b, M, N, K, ep, M);
   return e == cudaSuccess ? DMN_OK : cuda_fail(e, "dmn_gemm_bf16_tn");
 }
