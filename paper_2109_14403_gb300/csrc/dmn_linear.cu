@@ -26,6 +26,7 @@
 
 #include "../../include/dmn_linear.h"
 #include "dmn_internal.h"
+#include "pdl.cuh"
 
 namespace dmn {
 namespace {
@@ -356,6 +357,19 @@ __device__ __forceinline__ double pow_q(double x, double q) {
   return r;
 }
 
+// S^(1/q): a small whole q from the FP32 root by two Newton steps (relative
+// error 1e-6 -> 5e-12 -> rounding), a fifth of the FP64 pow()'s chain
+__device__ __forceinline__ double root_q(double S, double q) {
+  if (!(q >= 1.0 && q <= 64.0) || q != floor(q) || !(S > 1e-30 && S < 1e30)) return pow(S, 1.0 / q);
+  double x = double(powf(float(S), float(1.0 / q)));
+#pragma unroll 1
+  for (int k = 0; k < 2; ++k) {
+    const double y = pow_q(x, q - 1.0);
+    x -= (x * y - S) / (q * y);
+  }
+  return x;
+}
+
 // |x|_p of the 36 components f(i, j), six partial sums
 template <int MODE, typename F>
 __device__ __forceinline__ double lin_norm(double p, F f) {
@@ -367,11 +381,29 @@ __device__ __forceinline__ double lin_norm(double p, F f) {
   return root_p<MODE>(((col[0] + col[1]) + (col[2] + col[3])) + (col[4] + col[5]), p);
 }
 
-// per-sample error e_s = |T - D|_p / |T|_p (FP64)
-template <int MODE, typename T>
-__device__ __forceinline__ double lin_error(const double *Tg, const T *D, double p) {
-  const double nx = lin_norm<MODE>(p, [&](int i, int j) { return Tg[6 * i + j] - double(sget(D, i, j)); });
-  return nx / lin_norm<MODE>(p, [&](int i, int j) { return Tg[6 * i + j]; });
+// The error and seed kernels take a sample on LP = 1 thread, or on eight lanes,
+// one row of the six each, where the batch is too small to fill the SMs (an
+// FP64 instruction holds a warp's sub-partition for 64 cycles, so what counts
+// there is the length of a lane's chain, not the number of lanes).
+template <int LP>
+__device__ __forceinline__ double lane_sum(double x) {
+#pragma unroll
+  for (int o = LP / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+// p-norm over the 36 components f(i, j) of a sample, row i on lane i
+template <int MODE, int LP, typename F>
+__device__ __forceinline__ double sample_norm(double p, int row, F f) {
+  if (LP == 1) return lin_norm<MODE>(p, f);
+  double a = 0.0, b = 0.0;
+  if (row < 6) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      a += pow_p<MODE>(fabs(f(row, j)), p);
+      b += pow_p<MODE>(fabs(f(row, j + 3)), p);
+    }
+  }
+  return root_p<MODE>(lane_sum<LP>(a + b), p);
 }
 
 template <typename T>
@@ -397,7 +429,7 @@ __global__ void k_lin_forward(int K, int64_t n, const double *C1, const double *
 // the block that comes last (ticket) joins them in block order, so the result
 // does not depend on the order of arrival:
 //   scal[0] = m = max e, scal[1] = S^(1/q - 1) / n with S = sum (m_b / m)^q S_b,
-// and the loss (J, data term, penalty).  A block whose errors are all zero (or
+//   scal[2] = the loss's data term.  A block whose errors are all zero (or
 // NaN) has m_b = 0 and hands on their plain sum.  (One CTA over all errors, two
 // general powers a sample in a row, took 1815 us at 65,536 samples; the step
 // as a whole went from 6890 to 1837 us with this, the exact powers and the
@@ -424,8 +456,7 @@ __device__ __forceinline__ double block_sum(double x, double *red) {
   for (int w = 1; w < kLvlThreads / 32; ++w) x += red[w];
   return x;
 }
-__device__ void lin_reduce(int64_t n, double e, double q, double penalty, double *part, double *scal,
-                           double *loss) {
+__device__ void lin_reduce(int64_t n, double e, double q, double *part, double *scal) {
   __shared__ double red[kLvlThreads / 32];
   __shared__ bool last;
   const int t = threadIdx.x;
@@ -451,15 +482,10 @@ __device__ void lin_reduce(int64_t n, double e, double q, double penalty, double
     }
   const double S = block_sum(acc, red);
   if (t == 0) {
-    const double wsum = scal[5];
-    const double root = m > 0.0 ? root_p<0>(S, q) / double(n) : 0.0;
-    const double data = m * root;
-    const double pen = penalty * (wsum - 1.0) * (wsum - 1.0);
+    const double root = m > 0.0 ? root_q(S, q) / double(n) : 0.0;
     scal[0] = m;
     scal[1] = m > 0.0 ? root / S : 0.0;
-    loss[0] = data + pen;
-    loss[1] = data;
-    loss[2] = pen;
+    scal[2] = m * root;
   }
 }
 
@@ -511,10 +537,7 @@ __device__ __forceinline__ void tree_weights(int K, int t, double *Wt) {
 //  block 0   c1 of every node in the laminate precision (first half of the
 //            threads: the weights level by level, then all quotients at once)
 //            and the normalised normals (second half);
-//  block 1   zeroes the gradient sums and the scalars (nz doubles from acc),
-//            and adds up the weights, in leaf order, into scal[5] (one thread;
-//            the additions run beside block 0's levels: in the chain through
-//            the weights they would stand alone);
+//  block 1   zeroes the gradient sums and the scalars (nz doubles from acc);
 //  others    the phase stiffnesses of every sample, packed, in the laminate
 //            precision: PH[phase][21][sample] (converted once instead of by
 //            every bottom laminate).
@@ -524,10 +547,11 @@ constexpr int kSetupThreads = 2 << kLinMaxK;
 template <typename T>
 __global__ void __launch_bounds__(kSetupThreads)
     k_lvl_setup(int K, int64_t n, const double *normals, const double *v, const double *C1, const double *C2, T *nh,
-                T *c1s, T *PH, double *acc, int nz, double *scal) {
+                T *c1s, T *PH, double *acc, int nz) {
   __shared__ double Wt[2 * (1 << kLinMaxK)];
   const int N = (1 << K) - 1, L = 1 << K, t = threadIdx.x;
   constexpr int H = kSetupThreads / 2;
+  chain_begin();
   if (blockIdx.x > 1) {
     const int64_t i = int64_t(blockIdx.x - 2) * H + (t & (H - 1)), ph = t / H;  // one phase a thread
     if (i >= n) return;
@@ -536,18 +560,11 @@ __global__ void __launch_bounds__(kSetupThreads)
     lvl_store(PH, int(ph), n, i, a);
     return;
   }
-  if (t < L) Wt[t] = v[t] > 0.0 ? v[t] : 0.0;
   if (blockIdx.x == 1) {
     for (int i = t; i < nz; i += kSetupThreads) acc[i] = 0.0;
-    __syncthreads();
-    if (t == 0) {
-      double w = 0.0;
-#pragma unroll 8
-      for (int j = 0; j < L; ++j) w += Wt[j];
-      scal[5] = w;
-    }
     return;
   }
+  if (t < L) Wt[t] = v[t] > 0.0 ? v[t] : 0.0;
   if (t >= H && t - H < N) {
     const int pp = t - H;
     const double x = normals[3 * pp], y = normals[3 * pp + 1], z = normals[3 * pp + 2];
@@ -567,6 +584,7 @@ __global__ void __launch_bounds__(kSetupThreads)
 template <typename T>
 __global__ void __launch_bounds__(kLvlThreads) k_lvl_fwd(int K, int k, int64_t n, const T *PH, const T *nh,
                                                          const T *c1s, T *NS) {
+  chain_begin();
   const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
   if (s >= n) return;
   const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j;
@@ -584,58 +602,92 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_fwd(int K, int k, int64_t n
   lvl_store(NS, pp, n, s, out);
 }
 
-// per-sample error from the root column, and the batch reduction
-template <int MODE, typename T>
+// per-sample error e_s = |T - D|_p / |T|_p from the root column (FP64), and the
+// batch reduction
+template <int MODE, int LP, typename T>
 __global__ void __launch_bounds__(kLvlThreads) k_lvl_err(int K, int64_t n, const T *NS, const double *Ct, double p,
-                                                         double q, double penalty, double *err, double *part,
-                                                         double *scal, double *loss) {
-  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
+                                                         double q, double *err, double *part, double *scal) {
+  const int64_t s = (int64_t(blockIdx.x) * kLvlThreads + threadIdx.x) / LP;
+  const int row = LP == 1 ? 0 : threadIdx.x % LP;
+  chain_begin();
   double e = 0.0;
-  if (s < n) {
-    T D[21];
-    lvl_load(NS, (1 << K) - 2, n, s, D);
-    e = lin_error<MODE>(Ct + 36 * s, D, p);
-    err[s] = e;
-  }
-  lin_reduce(n, e, q, penalty, part, scal, loss);
+  const int64_t sc = s < n ? s : n - 1;  // lanes past the batch repeat its last sample
+  const double *Tg = Ct + 36 * sc;
+  const T *R = NS + (int64_t((1 << K) - 2) * 21) * n + sc;  // component q of the root: R[q n]
+  T D[21];
+  if (LP == 1) lvl_load(NS, (1 << K) - 2, n, sc, D);
+  const double nx = sample_norm<MODE, LP>(p, row, [&](int i, int j) {
+    return Tg[6 * i + j] - double(LP == 1 ? sget(D, i, j) : R[(i <= j ? sidx(i, j) : sidx(j, i)) * n]);
+  });
+  e = nx / sample_norm<MODE, LP>(p, row, [&](int i, int j) { return Tg[6 * i + j]; });
+  if (s >= n || row != 0) e = 0.0;
+  else err[s] = e;
+  lin_reduce(n, e, q, part, scal);
 }
 
 // dJ/dD at the root: (1/N) S^(1/q-1) (e_s/m)^(q-1) de_s/dD, with |T - D|_p =
 // e_s |T|_p; for p = 1 every component's is +-1 / |T|_1
-template <int MODE, typename T>
-__device__ __forceinline__ void lin_seed(const double *Tg, const T *D, double p, double q, double e,
-                                         const double *scal, T G[21]) {
+template <int MODE, int LP, typename T>
+__device__ __forceinline__ void lin_seed(int64_t n, int row, const double *Tg, const T *R, double p, double q,
+                                         double e, const double *scal, bool st, T *G) {
   const double m = scal[0];
   const double coef = (m > 0.0 && e > 0.0) ? scal[1] * pow_q(e / m, q - 1.0) : 0.0;
-  const double nt = lin_norm<MODE>(p, [&](int i, int j) { return Tg[6 * i + j]; });
+  const double nt = sample_norm<MODE, LP>(p, row, [&](int i, int j) { return Tg[6 * i + j]; });
   const double f = MODE == 1 ? 1.0 / nt : (MODE == 2 ? 1.0 / (e * nt) : pow(e * nt, 1.0 - p)) / nt;
+  auto put = [&](int i, int j) {
+    const int c = sidx(i, j);
+    const double x = Tg[6 * i + j] - double(R[c * n]);
+    const double sg = x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0);
+    const double xp = MODE == 1 ? 1.0 : (MODE == 2 ? fabs(x) : pow(fabs(x), p - 1.0));
+    const double de = e > 0.0 ? -sg * xp * f : 0.0;
+    if (st) G[c * n] = T(coef * de);
+  };
+  if (LP == 1) {
 #pragma unroll
-  for (int i = 0; i < 6; ++i)
+    for (int i = 0; i < 6; ++i)
 #pragma unroll
-    for (int j = i; j < 6; ++j) {
-      const double x = Tg[6 * i + j] - double(sget(D, i, j));
-      const double sg = x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0);
-      const double xp = MODE == 1 ? 1.0 : (MODE == 2 ? fabs(x) : pow(fabs(x), p - 1.0));
-      const double de = e > 0.0 ? -sg * xp * f : 0.0;
-      G[sidx(i, j)] = T(coef * de);
-    }
+      for (int j = i; j < 6; ++j) put(i, j);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 6; ++j)
+      if (row <= j) put(row, j);
+  }
 }
-template <int MODE, typename T>
+// Also, in the last block, the weights' sum in leaf order (into scal[5]: one
+// thread, 9 us at K = 8 beside the other blocks; the weights sum to about 1 and
+// 1 is taken off, so its order shows) and the loss (J, data term, penalty).
+template <int MODE, int LP, typename T>
 __global__ void __launch_bounds__(kLvlThreads) k_lvl_seed(int K, int64_t n, const T *NS, const double *Ct, double p,
-                                                          double q, const double *err, const double *scal, T *GA) {
-  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
-  if (s >= n) return;
-  const int root = (1 << K) - 2;
-  T D[21], G[21];
-  lvl_load(NS, root, n, s, D);
-  lin_seed<MODE>(Ct + 36 * s, D, p, q, err[s], scal, G);
-  lvl_store(GA, root, n, s, G);
+                                                          double q, const double *err, const double *v,
+                                                          double penalty, double *scal, double *loss, T *GA) {
+  __shared__ double wl[1 << kLinMaxK];
+  chain_begin();
+  if (blockIdx.x == gridDim.x - 1) {
+    for (int j = threadIdx.x; j < (1 << K); j += kLvlThreads) wl[j] = v[j] > 0.0 ? v[j] : 0.0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double w = 0.0;
+#pragma unroll 8
+      for (int j = 0; j < (1 << K); ++j) w += wl[j];
+      const double data = scal[2], pen = penalty * (w - 1.0) * (w - 1.0);
+      scal[5] = w;
+      loss[0] = data + pen;
+      loss[1] = data;
+      loss[2] = pen;
+    }
+    return;
+  }
+  const int64_t s = (int64_t(blockIdx.x) * kLvlThreads + threadIdx.x) / LP;
+  const int row = LP == 1 ? 0 : threadIdx.x % LP;
+  const int64_t sc = s < n ? s : n - 1, root = int64_t((1 << K) - 2) * 21 * n + sc;
+  lin_seed<MODE, LP>(n, row, Ct + 36 * sc, NS + root, p, q, err[sc], scal, s < n, GA + root);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kLvlThreads) k_lvl_bwd(int K, int k, int64_t n, const T *PH, const T *nh,
                                                          const T *c1s, const T *NS, T *GA, double *gnh,
                                                          double *gc1) {
+  chain_begin();
   __shared__ T red[4][kLvlThreads / 32];
   const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
   const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j;
@@ -691,6 +743,7 @@ __global__ void __launch_bounds__(kLvlThreads) k_lvl_bwd(int K, int k, int64_t n
 template <bool LEAF, typename T>
 __global__ void __launch_bounds__(kLvlThreads, LEAF ? 3 : 4) k_lvl_fwd2(int K, int k, int64_t n, const T *PH, const T *nh,
                                                           const T *c1s, T *NS) {
+  chain_begin();
   const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
   if (s >= n) return;
   const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j, pc = (1 << K) - (1 << (k + 1)) + 2 * j;
@@ -722,6 +775,7 @@ template <bool LEAF, typename T>
 __global__ void __launch_bounds__(kLvlThreads, 3) k_lvl_bwd2(int K, int k, int64_t n, const T *PH, const T *nh,
                                                           const T *c1s, const T *NS, T *GA, double *gnh,
                                                           double *gc1) {
+  chain_begin();
   __shared__ T red[3][4][kLvlThreads / 32];
   const int64_t s = int64_t(blockIdx.x) * kLvlThreads + threadIdx.x;
   const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j, pc = (1 << K) - (1 << (k + 1)) + 2 * j;
@@ -794,6 +848,7 @@ __global__ void __launch_bounds__(kLvlThreads, 3) k_lvl_bwd2(int K, int k, int64
 __global__ void __launch_bounds__(kSetupThreads)
     k_lin_finish(int K, const double *normals, const double *v, double penalty, const double *gnh,
                  const double *gc1, const double *scal, double *grad_n, double *grad_v) {
+  chain_begin();
   __shared__ double Wt[2 << kLinMaxK], gW[2 << kLinMaxK];  // leaves [0, L), nodes [L, L + N)
   const int N = (1 << K) - 1, L = 1 << K, t = threadIdx.x;
   constexpr int H = kSetupThreads / 2;
@@ -801,11 +856,11 @@ __global__ void __launch_bounds__(kSetupThreads)
   if (t >= H && t - H < N) {
     const int pp = t - H;
     const double x = normals[3 * pp], y = normals[3 * pp + 1], z = normals[3 * pp + 2];
-    const double len = sqrt(x * x + y * y + z * z);
-    const double nh[3] = {x / len, y / len, z / len};
+    const double il = 1.0 / sqrt(x * x + y * y + z * z);
+    const double nh[3] = {x * il, y * il, z * il};
     const double g[3] = {gnh[3 * pp], gnh[3 * pp + 1], gnh[3 * pp + 2]};
     const double gd = g[0] * nh[0] + g[1] * nh[1] + g[2] * nh[2];
-    for (int c = 0; c < 3; ++c) grad_n[3 * pp + c] = (g[c] - gd * nh[c]) / len;
+    for (int c = 0; c < 3; ++c) grad_n[3 * pp + c] = (g[c] - gd * nh[c]) * il;
   }
   __syncthreads();
   tree_weights(K, t, Wt);
@@ -894,49 +949,58 @@ template <typename T>
 dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, const double *C2,
                           const double *Ct, const double *normals, const double *v, double p, double q,
                           double penalty, double *err, double *scal, double *loss, T *consts, T *PH, T *NS, T *GA,
-                          double *gnh, double *gc1) {
+                          double *gnh, double *gc1, double *grad_n, double *grad_v) {
   const unsigned nb = unsigned((n + kLvlThreads - 1) / kLvlThreads);
   if (nb > 2147483647u) return lin_fail("dmn_linear_loss_grad: batch too large");
   const int N = (1 << K) - 1;
   T *nh = consts, *c1s = consts + 3 * N;
   const unsigned ns = unsigned((n + kSetupThreads / 2 - 1) / (kSetupThreads / 2));
-  k_lvl_setup<T><<<2 + ns, kSetupThreads, 0, st>>>(K, n, normals, v, C1, C2, nh, c1s, PH, gnh, 4 * N + 5, scal);
+  cudaError_t e = cudaSuccess;
+  // a small batch's launches overlap (its kernels last little longer than their
+  // launch: 32 samples, K = 8: 107 -> 93 us with the eight-lane kernels); a large
+  // one's do not (65,536 samples: early CTAs of the next level cost 4 %)
+  const bool small = n <= 2048;
+  auto go = [&](auto f, dim3 grid, unsigned threads, auto... args) {
+    if (e == cudaSuccess) e = launch_chained(small, f, grid, dim3(threads), 0, st, args...);
+  };
+  go(k_lvl_setup<T>, dim3(2 + ns), kSetupThreads, K, n, normals, v, C1, C2, nh, c1s, PH, gnh, 4 * N + 5);
   // FP32: pairs of levels from the bottom (FP64 laminates: 251 registers for one
   // level, and bound by the FP64 pipe, so one level a launch)
   int k = K;
   if constexpr (sizeof(T) == 4)
-    for (; k >= 2; k -= 2) {
-      const dim3 grid(nb, 1u << (k - 2));
-      if (k == K) k_lvl_fwd2<true><<<grid, kLvlThreads, 0, st>>>(K, k - 1, n, PH, nh, c1s, NS);
-      else k_lvl_fwd2<false><<<grid, kLvlThreads, 0, st>>>(K, k - 1, n, PH, nh, c1s, NS);
-    }
-  for (; k >= 1; --k) k_lvl_fwd<T><<<dim3(nb, 1u << (k - 1)), kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: forward level launch");
+    for (; k >= 2; k -= 2)
+      go(k == K ? k_lvl_fwd2<true, T> : k_lvl_fwd2<false, T>, dim3(nb, 1u << (k - 2)), kLvlThreads, K, k - 1, n, PH,
+         nh, c1s, NS);
+  for (; k >= 1; --k) go(k_lvl_fwd<T>, dim3(nb, 1u << (k - 1)), kLvlThreads, K, k, n, PH, nh, c1s, NS);
   // the blocks' partial sums: in the adjoints' array, free until the seed, from an 8-byte boundary
   double *part = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(GA) + 7) & ~uintptr_t(7));
   const int mode = pow_mode(p);
-  (mode == 1 ? k_lvl_err<1, T> : mode == 2 ? k_lvl_err<2, T> : k_lvl_err<0, T>)<<<nb, kLvlThreads, 0, st>>>(
-      K, n, NS, Ct, p, q, penalty, err, part, scal, loss);
-  (mode == 1 ? k_lvl_seed<1, T> : mode == 2 ? k_lvl_seed<2, T> : k_lvl_seed<0, T>)<<<nb, kLvlThreads, 0, st>>>(
-      K, n, NS, Ct, p, q, err, scal, GA);
-  if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: loss launch");
+  if (small) {  // eight lanes a sample: at most 128 CTAs
+    const unsigned nb8 = unsigned((8 * n + kLvlThreads - 1) / kLvlThreads);
+    go(mode == 1 ? k_lvl_err<1, 8, T> : mode == 2 ? k_lvl_err<2, 8, T> : k_lvl_err<0, 8, T>, dim3(nb8), kLvlThreads,
+       K, n, NS, Ct, p, q, err, part, scal);
+    go(mode == 1 ? k_lvl_seed<1, 8, T> : mode == 2 ? k_lvl_seed<2, 8, T> : k_lvl_seed<0, 8, T>, dim3(nb8 + 1),
+       kLvlThreads, K, n, NS, Ct, p, q, err, v, penalty, scal, loss, GA);
+  } else {
+    go(mode == 1 ? k_lvl_err<1, 1, T> : mode == 2 ? k_lvl_err<2, 1, T> : k_lvl_err<0, 1, T>, dim3(nb), kLvlThreads,
+       K, n, NS, Ct, p, q, err, part, scal);
+    go(mode == 1 ? k_lvl_seed<1, 1, T> : mode == 2 ? k_lvl_seed<2, 1, T> : k_lvl_seed<0, 1, T>, dim3(nb + 1),
+       kLvlThreads, K, n, NS, Ct, p, q, err, v, penalty, scal, loss, GA);
+  }
   // the same pairs, root first
   k = 1;
   if constexpr (sizeof(T) == 4) {
     if (K & 1) {
-      k_lvl_bwd<T><<<dim3(nb, 1), kLvlThreads, 0, st>>>(K, 1, n, PH, nh, c1s, NS, GA, gnh, gc1);
+      go(k_lvl_bwd<T>, dim3(nb, 1), kLvlThreads, K, 1, n, PH, nh, c1s, NS, GA, gnh, gc1);
       k = 2;
     }
-    for (; k < K; k += 2) {
-      const dim3 grid(nb, 1u << (k - 1));
-      if (k + 1 == K) k_lvl_bwd2<true><<<grid, kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
-      else k_lvl_bwd2<false><<<grid, kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
-    }
+    for (; k < K; k += 2)
+      go(k + 1 == K ? k_lvl_bwd2<true, T> : k_lvl_bwd2<false, T>, dim3(nb, 1u << (k - 1)), kLvlThreads, K, k, n, PH,
+         nh, c1s, NS, GA, gnh, gc1);
   }
-  for (; k <= K; ++k)
-    k_lvl_bwd<T><<<dim3(nb, 1u << (k - 1)), kLvlThreads, 0, st>>>(K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
-  if ((e = cudaGetLastError()) != cudaSuccess) return lin_cuda(e, "dmn_linear: backward level launch");
+  for (; k <= K; ++k) go(k_lvl_bwd<T>, dim3(nb, 1u << (k - 1)), kLvlThreads, K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
+  go(k_lin_finish, dim3(1), kSetupThreads, K, normals, v, penalty, gnh, gc1, scal, grad_n, grad_v);
+  if (e != cudaSuccess) return lin_cuda(e, "dmn_linear_loss_grad: launch");
   return DMN_OK;
 }
 
@@ -976,20 +1040,14 @@ extern "C" dmn_status dmn_linear_loss_grad(dmn_stream stream, int32_t K, int64_t
   double *err = d_work, *gnh = d_work + n_samples, *gc1 = gnh + 3 * N, *scal = gc1 + N;
   double *consts = scal + 8, *nodes = consts + 4 * N;
   const int64_t cells = int64_t(21) * N * n_samples, ph = int64_t(42) * n_samples;
-  dmn_status s;
   if (precision == DMN_LIN_FP64)
-    s = lin_train_pass<double>(st, K, n_samples, d_C1, d_C2, d_Ctarget, d_normals, d_v, p, q, penalty, err, scal,
-                               d_loss, consts, nodes, nodes + ph, nodes + ph + cells, gnh, gc1);
-  else {
-    float *f = reinterpret_cast<float *>(nodes);
-    s = lin_train_pass<float>(st, K, n_samples, d_C1, d_C2, d_Ctarget, d_normals, d_v, p, q, penalty, err, scal,
-                              d_loss, reinterpret_cast<float *>(consts), f, f + ph, f + ph + cells, gnh, gc1);
-  }
-  if (s != DMN_OK) return s;
-  k_lin_finish<<<1, kSetupThreads, 0, st>>>(K, d_normals, d_v, penalty, gnh, gc1, scal, d_grad_n, d_grad_v);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return lin_cuda(e, "dmn_linear: finish launch");
-  return DMN_OK;
+    return lin_train_pass<double>(st, K, n_samples, d_C1, d_C2, d_Ctarget, d_normals, d_v, p, q, penalty, err, scal,
+                                  d_loss, consts, nodes, nodes + ph, nodes + ph + cells, gnh, gc1, d_grad_n,
+                                  d_grad_v);
+  float *f = reinterpret_cast<float *>(nodes);
+  return lin_train_pass<float>(st, K, n_samples, d_C1, d_C2, d_Ctarget, d_normals, d_v, p, q, penalty, err, scal,
+                               d_loss, reinterpret_cast<float *>(consts), f, f + ph, f + ph + cells, gnh, gc1,
+                               d_grad_n, d_grad_v);
 }
 
 extern "C" dmn_status dmn_linear_amsgrad(dmn_stream stream, int64_t n_params, double *d_params,
