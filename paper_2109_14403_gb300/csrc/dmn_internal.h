@@ -55,7 +55,8 @@ size_t warp_scratch_bytes_per_cta(int K);
 KernelFn warp_kernel(int K, int minb);
 KernelFn warp_kernel8(int minb);
 // threads per CTA of the kernel a variant selects
-int solve_block_threads(int K, int variant, int law);
+int solve_block_threads(int K, bool mixed, int variant, int law);
+int compact_block_threads64(int K);  // ... of the compact kernel's FP64 instances
 cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
                           int *blocks_per_sm);
 cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, int blocks_per_sm,

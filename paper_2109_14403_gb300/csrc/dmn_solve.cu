@@ -479,9 +479,11 @@ bool solve_variant_valid(int variant) {
 static bool uses_warp_form(int K, bool mixed, int variant, int law) {
   return is_warp_variant(variant) && warp_form_supports(K, mixed, law);
 }
-int solve_block_threads(int K, int variant, int law) {
-  (void)law;
-  return is_warp_variant(variant) ? 32 * warp_form_warps() : (1 << (K - 1));
+static bool is_compact(int K, bool mixed, int variant, int law);
+int solve_block_threads(int K, bool mixed, int variant, int law) {
+  if (uses_warp_form(K, mixed, variant, law)) return 32 * warp_form_warps();
+  const int G = 1 << (K - 1);
+  return !mixed && is_compact(K, mixed, variant, law) ? compact_block_threads64(K) : G;
 }
 static bool is_compact(int K, bool mixed, int variant, int law) {
   return law >= 2 || !mixed ? K <= 9 : (K <= 8 && variant >= 11);
@@ -541,7 +543,7 @@ static int carveout_pct(size_t smem, int ctas) {
 cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
                           int *blocks_per_sm) {
   const size_t smem = solve_smem_bytes(K, zw, n_mats, mixed, variant, law);
-  const int threads = solve_block_threads(K, variant, law);
+  const int threads = solve_block_threads(K, mixed, variant, law);
   const KernelFn f = pick(K, mixed, variant, law, false), g = pick(K, mixed, variant, law, true);
   if (g != f) {  // the instance of small launches
     int b = 0;
@@ -554,7 +556,7 @@ cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, in
 cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, int blocks_per_sm,
                          cudaStream_t s) {
   const size_t smem = solve_smem_bytes(P.K, P.zw, P.n_mats, mixed, variant, P.law);
-  cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned long long), s);
+  const cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   const int per_sm = (grid + num_sms - 1) / num_sms;
   cudaLaunchAttribute at[1];
@@ -562,7 +564,7 @@ cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid
   at[0].val.sharedMemCarveout = unsigned(carveout_pct(smem, per_sm < blocks_per_sm ? per_sm : blocks_per_sm));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(grid));
-  cfg.blockDim = dim3(unsigned(solve_block_threads(P.K, variant, P.law)));
+  cfg.blockDim = dim3(unsigned(solve_block_threads(P.K, mixed, variant, P.law)));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = at;

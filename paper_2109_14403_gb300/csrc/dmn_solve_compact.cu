@@ -16,9 +16,11 @@ size_t compact_smem_bytes(int K, int zw, int n_mats, bool mixed) {
   return (b + 15) & ~size_t(15);
 }
 
+int compact_block_threads64(int K) { return K <= 5 ? 32 : 1 << (K - 1); }
+
 KernelFn compact_kernel(int K, bool mixed, int minb) {
-  (void)K;  // depth <= 8: at most 128 threads
-  if (!mixed) return dmn_solve_compact<double, double, 128, 1, 1>;
+  // depth <= 8: at most 128 threads
+  if (!mixed) return K <= 5 ? dmn_solve_compact<double, double, 32, 1, 1> : dmn_solve_compact<double, double, 128, 1, 1>;
   if (minb >= 4) return dmn_solve_compact<float, dfl, 128, 4, 1>;
   return minb == 3 ? dmn_solve_compact<float, dfl, 128, 3, 1> : dmn_solve_compact<float, dfl, 128, 2, 1>;
 }

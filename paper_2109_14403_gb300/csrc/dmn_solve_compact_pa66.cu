@@ -11,7 +11,7 @@ size_t compact_smem_bytes_pa(int K, int hw, int n_mats, bool mixed) {
 }
 
 KernelFn compact_kernel_pa66(int K, bool mixed) {
-  (void)K;  // depth <= 8: at most 128 threads
+  if (!mixed && K <= 5) return dmn_solve_compact<double, double, 32, 1, 3>;
   return mixed ? dmn_solve_compact<float, dfl, 128, 2, 3> : dmn_solve_compact<double, double, 128, 1, 3>;
 }
 

@@ -5,6 +5,7 @@
 namespace dmn {
 
 KernelFn compact_kernel_vp(int K, bool mixed) {
+  if (!mixed && K <= 5) return dmn_solve_compact<double, double, 32, 1, 2>;
   if (K <= 8)
     return mixed ? dmn_solve_compact<float, dfl, 128, 3, 2> : dmn_solve_compact<double, double, 128, 1, 2>;
   return mixed ? dmn_solve_compact<float, dfl, 256, 1, 2> : dmn_solve_compact<double, double, 256, 1, 2>;

@@ -599,7 +599,7 @@ struct Scratch {
 __host__ __device__ inline Scratch scratch_layout(int G, int tf_bytes) {
   Scratch c;
   c.GX = G >= 2 ? G / 2 : 1;  // level K-1 has G/2 nodes
-  c.GY = G >= 4 ? G / 4 : 1;  // level K-2
+  c.GY = tf_bytes == 8 && G < 32 ? G : (G >= 4 ? G / 4 : 1);  // level K-2 (small FP64 trees: level K)
   c.sx = 0;
   c.sy = 6 * c.GX;
   const int rx_tf = (6 * c.GX + 6 * c.GY) * (8 / tf_bytes);  // records start after the sums
@@ -617,6 +617,7 @@ __host__ __device__ inline Scratch scratch_layout(int G, int tf_bytes) {
 }  // namespace compact_detail
 using namespace compact_detail;
 
+// FP64 trees of fewer than 32 bottom laminates take the instances with MAXT = 32.
 // LAW: largest material kind the instance handles (1: thermoelastic and J2;
 // 2: also the Perzyna leaf; 3: also the PA66 leaf, whose per-point constants
 // (MatPA) follow the materials' and whose leaves keep their history, not
@@ -660,20 +661,27 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
   HP *anc = scr;  // strain sums: per non-bottom node c2 B x, c1 B x, c2 tr, c1 tr
   HP *redD = scr, *redX = scr + 32;  // epilogue: warp sums of D and Diss (32 each)
 
-  const unsigned mask = group_mask(G);
-  const int W = group_width(G);
-  const int lane = t & 31, warp = t >> 5, nwarp = (G + 31) >> 5;
+  constexpr bool D64 = sizeof(TF) == 8;
+  // SMALL: the FP64 instances for trees of fewer than 32 bottom laminates, one
+  // warp a CTA (the upper levels use it whole).  Else a thread per bottom laminate.
+  constexpr bool SMALL = D64 && MAXT == 32;
+  const int T = SMALL ? 32 : G;
+  const bool bot = !SMALL || t < G;  // this thread has a bottom laminate
+  const unsigned mask = group_mask(T);
+  const int W = group_width(T);
+  const int lane = t & 31, warp = t >> 5, nwarp = (T + 31) >> 5;
   // FP64 instances: an FP64 warp instruction takes 64 cycles of its
   // sub-partition (19 of the SM with all four busy) whatever the number of
   // active lanes (a probe of independent FMA chains), so their phases are laid
-  // out for few, full warps
-  constexpr bool D64 = sizeof(TF) == 8;
-  // this thread's bottom laminate.  FP64: the first half of the threads take
-  // the even ones, the second half the odd ones, so that the laminates of
-  // level K-1 find their left child in the registers of thread j < G/2 and
-  // fill whole warps (level K-1 below).  Mixed: in order (the packed level K-1
-  // cost it 2 to 4 %: one more barrier and more spills)
-  const int b = !D64 || K == 1 ? t : (t < G / 2 ? 2 * t : 2 * (t - G / 2) + 1);
+  // out for few, full warps.  PACK: the laminates of level K-1 on threads j <
+  // G/2, whole warps, with their left child's record in registers: the first
+  // half of the threads take the even bottom laminates, the second half the odd
+  // ones.  SMALL trees take level K-1 from shared memory like the levels above
+  // it (64 points at K = 4: 287 -> 219 us); mixed ones in order by shuffle (the
+  // packed level cost 2 to 4 %: one more barrier and more spills).
+  constexpr bool PACK = D64 && !SMALL;
+  // this thread's bottom laminate
+  const int b = !bot ? 0 : (!PACK ? t : (t < G / 2 ? 2 * t : 2 * (t - G / 2) + 1));
   if (t == 0) {
     // a warp slot's sub-partition is slot mod 4 and a CTA's warps take
     // consecutive slots: rotate the leader by the CTA's slot group
@@ -712,10 +720,10 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
     orec[33] = R.gg;
   };
 
-  for (int i = t; i < P.n_mats; i += G)
+  for (int i = t; i < P.n_mats; i += T)
     mat_static<TF, HP>(mp_s[i], *reinterpret_cast<const MatDev *>(P.mat + kMatWords * i), P.dt);
   if (LAW == 3)
-    for (int i = t; i < P.n_mats; i += G)
+    for (int i = t; i < P.n_mats; i += T)
       if (int(P.mat[kMatWords * i] + 0.5) == 3)
         mat_static_pa<TF, HP>(mpa_s[i], *reinterpret_cast<const MatDev *>(P.mat + kMatWords * i));
   if (t == 0) misc[0] = hp_from(1.0 / P.dt, tag);
@@ -743,7 +751,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
   // Ends with a barrier: eK is complete and the scratch region free again.
   enum { SW_PLAIN = 0, SW_WARM = 1, SW_STEP = 2 };
   auto sweep = [&](int mode, HP tr_root) -> HP {
-    for (int q = t; q < G - 1; q += G) {
+    for (int q = t; q < G - 1; q += T) {
       const int p = G + q;
       NodeHP<HP> nd;
       load_node(P, p, nd);
@@ -780,24 +788,27 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       }
     }
     __syncthreads();
-    HP e[6], tr = tr_root;
+    HP tr = tr_root;
+    if (bot) {
+      HP e[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) e[c] = mode == SW_STEP ? hp_zero(tag) : eb[c];
-    for (int k = 1; k <= K - 1; ++k) {
-      const int p = (1 << K) - (1 << k) + (b >> (K - k));
-      const HP *ent = anc + 14 * (p - G);
-      if ((b >> (K - k - 1)) & 1) {
+      for (int c = 0; c < 6; ++c) e[c] = mode == SW_STEP ? hp_zero(tag) : eb[c];
+      for (int k = 1; k <= K - 1; ++k) {
+        const int p = (1 << K) - (1 << k) + (b >> (K - k));
+        const HP *ent = anc + 14 * (p - G);
+        if ((b >> (K - k - 1)) & 1) {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) e[c] = e[c] - ent[6 + c];
-        if (mode == SW_WARM) tr = tr - ent[13];
-      } else {
+          for (int c = 0; c < 6; ++c) e[c] = e[c] - ent[6 + c];
+          if (mode == SW_WARM) tr = tr - ent[13];
+        } else {
 #pragma unroll
-        for (int c = 0; c < 6; ++c) e[c] = e[c] + ent[c];
-        if (mode == SW_WARM) tr = tr + ent[12];
+          for (int c = 0; c < 6; ++c) e[c] = e[c] + ent[c];
+          if (mode == SW_WARM) tr = tr + ent[12];
+        }
       }
-    }
 #pragma unroll
-    for (int c = 0; c < 6; ++c) eK[6 * t + c] = mode == SW_STEP ? eK[6 * t + c] + e[c] : e[c];
+      for (int c = 0; c < 6; ++c) eK[6 * t + c] = mode == SW_STEP ? eK[6 * t + c] + e[c] : e[c];
+    }
     __syncthreads();
     return tr;
   };
@@ -840,17 +851,17 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       const float *d0 = P.da0 ? P.da0 + pt * (3 * N) : nullptr;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int i = t + u * G;
+        const int i = t + u * T;
         vp[u] = d0 && i < 3 * N ? ld_stream(d0 + i) : 0.0f;
       }
-      if (G >= 8 && t < 6) {
+      if (T >= 8 && t < 6) {
         ve = ld_stream(sin + t);
         vd = ld_stream(P.deps + pt * 6 + t);
       }
       if (d0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int i = t + u * G;
+          const int i = t + u * T;
           if (i < 3 * N) da_s[i] = TF(vp[u]);
         }
       }
@@ -871,28 +882,28 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
           const double *ra = reinterpret_cast<const double *>(a_s);
           const double *rz = reinterpret_cast<const double *>(zn_s);
 #pragma unroll 1
-          for (int i = t; i < 3 * N; i += G) a_s[i] = hp_load(ra[i], tag);
+          for (int i = t; i < 3 * N; i += T) a_s[i] = hp_load(ra[i], tag);
           if (LAW < 3) {
 #pragma unroll 1
-            for (int i = t; i < ZW; i += G) zn_s[i] = hp_load(rz[i], tag);
+            for (int i = t; i < ZW; i += T) zn_s[i] = hp_load(rz[i], tag);
           }
         }
       } else {
 #pragma unroll 1
-        for (int i = t; i < 3 * N; i += G) a_s[i] = hp_load(ld_stream(sin + 8 + i), tag);
+        for (int i = t; i < 3 * N; i += T) a_s[i] = hp_load(ld_stream(sin + 8 + i), tag);
         if (LAW < 3) {
 #pragma unroll 1
-          for (int i = t; i < ZW; i += G) zn_s[i] = hp_load(ld_stream(sin + 8 + 3 * N + i), tag);
+          for (int i = t; i < ZW; i += T) zn_s[i] = hp_load(ld_stream(sin + 8 + 3 * N + i), tag);
         }
       }
-      if (G >= 8) {
+      if (T >= 8) {
         if (t < 6) {
           ebd[t] = ve + vd;  // eps_bar^{n+1} = eps_bar^n + deps exactly in FP64
           eb[t] = hp_load(ve + vd, tag);
           eb[6 + t] = hp_load(vd, tag);
         }
       } else {
-        for (int c = t; c < 6; c += G) {
+        for (int c = t; c < 6; c += T) {
           const double d = P.deps[pt * 6 + c], e1 = sin[c] + d;
           ebd[c] = e1;
           eb[c] = hp_load(e1, tag);
@@ -901,11 +912,11 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       }
     }
     __syncthreads();
-    for (int i = t; i < P.n_mats; i += G) mat_point<TF, HP, LAW>(mp_s[i], hp_load(theta, tag), misc[0], idt_f);
+    for (int i = t; i < P.n_mats; i += T) mat_point<TF, HP, LAW>(mp_s[i], hp_load(theta, tag), misc[0], idt_f);
     if (LAW == 3) {
       // PA66 constants at this temperature, then each thread's leaves: the
       // history of a PA66 leaf, the internal variables of a J2 leaf
-      for (int i = t; i < P.n_mats; i += G)
+      for (int i = t; i < P.n_mats; i += T)
         if (mp_s[i].kind == 3)
           mat_point_pa<TF, HP>(mpa_s[i], *reinterpret_cast<const MatDev *>(P.mat + kMatWords * i), theta,
                                P.dt);
@@ -913,7 +924,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
 #pragma unroll 1
       for (int sd = 0; sd < 2; ++sd) {
         const int zo = sd ? zo1 : zo0, ph = sd ? ph1 : ph0, hq = sd ? hq1 : hq0;
-        if (zo < 0) continue;
+        if (zo < 0 || !bot) continue;
         if (mp_s[ph].kind == 3) {
           pa_history<TF, HP>(mpa_s[ph], sin + zo, zn_s + hq);
         } else {
@@ -947,8 +958,10 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       const HP trj = an[0] * nd.n[0] + an[1] * nd.n[1] + an[2] * nd.n[2];
       trn0 = tre + nd.c2 * trj;
       trn1 = tre - nd.c1 * trj;
+      if (bot) {
 #pragma unroll
-      for (int r = 0; r < 3; ++r) a_s[3 * b + r] = hp_add_tf(an[r], da_s[3 * b + r]);
+        for (int r = 0; r < 3; ++r) a_s[3 * b + r] = hp_add_tf(an[r], da_s[3 * b + r]);
+      }
       first = false;  // this thread alone uses a_s[3b..] until the next barrier
     } else {
       sweep(SW_PLAIN, hp_zero(tag));  // strains of the bottom laminates at a^n
@@ -962,9 +975,9 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       // terms (coupling term, dissipation, thermal tangents)
       const bool full = !ctrl->first;
       // ---- R2: leaves and laminate b ----
-      TF r2;
+      TF r2 = TF(0);
       HP S[6];
-      {
+      if (bot) {
         NodeHP<HP> nd;
         load_node(P, b, nd);
         HP el[6], er[6];
@@ -1020,11 +1033,18 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
         else combine<TF>(rec, rr, n, c1, c2, rbv, gh_s + 21 * b, full);
         if (K == 1) put_root(rec, S);
       }
-      // ---- level K-1.  FP64: node j on thread j < G/2, which formed its left
+      // ---- level K-1.  PACK: node j on thread j < G/2, which formed its left
       //      child; the right child's record comes through shared memory, in
-      //      the slot that then takes the node's own.  Mixed: neighbouring
-      //      lanes (2j, 2j+1) ----
-      if (K >= 2) {
+      //      the slot that then takes the node's own.  Smaller FP64 trees: with
+      //      the levels above (the bottom laminates' records in Y).  Mixed:
+      //      neighbouring lanes (2j, 2j+1) ----
+      if constexpr (SMALL) {
+        if (bot && K >= 2) {
+          rec_put(recY + RS * b, rec);
+#pragma unroll
+          for (int c = 0; c < 6; ++c) Sy[6 * b + c] = S[c];
+        }
+      } else if (K >= 2) {
         Rec<TF> other;
         HP So[6];
         if constexpr (D64) {
@@ -1081,21 +1101,22 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       //      L, warp L goes on alone with warp barriers and the other warps
       //      move to the reduction barrier.  A CTA of fewer than 8 threads
       //      (K = 3) condenses its root on one thread. ----
-      if (G >= 8) {
+      if (T >= 8) {
         // lanes per node.  FP64: as many as keep the warps full: one on levels of
         // 64 and more nodes, two (combine_half) on 8 to 32, eight below
         // (K = 8: 9.9 k -> about 5.8 k FP64 warp instructions per pass)
         auto lanes_of = [&](int k) { return !D64 || k <= 3 ? 8 : (k <= 6 ? 2 : 1); };
-        for (int k = K - 2; k >= 1; --k) {
+        const int k_top = SMALL ? K - 1 : K - 2;
+        for (int k = k_top; k >= 1; --k) {
           const int lpn = lanes_of(k), ntask = lpn << (k - 1);
-          const bool wide = ntask > 32 && G > 32;
-          const bool prod_wide = k + 1 == K - 1 ? G > 32 : ((lanes_of(k + 1) << k) > 32 && G > 32);
+          const bool wide = ntask > 32 && T > 32;
+          const bool prod_wide = k == k_top ? T > 32 : ((lanes_of(k + 1) << k) > 32 && T > 32);
           if (prod_wide) __syncthreads();
           if (!wide) {  // this level and the ones above: warp L alone
             if (warp != L) break;
             if (!prod_wide) __syncwarp(mask);
           }
-          const int step = wide ? G : (G < 32 ? G : 32);
+          const int step = wide ? T : (T < 32 ? T : 32);
           const int q0 = wide ? t : lane;
           const int cnt = 1 << (k - 1);
           for (int qb = 0; qb < ntask; qb += step) {
@@ -1213,7 +1234,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
           // warm-started iteration failed: run Algorithm 1 again from a^n
           attempt = 1;
           it_total = ctrl->it;
-          for (int i = t; i < 3 * N; i += G) a_s[i] = hp_load(sin[8 + i], tag);
+          for (int i = t; i < 3 * N; i += T) a_s[i] = hp_load(sin[8 + i], tag);
           __syncthreads();  // every thread has read ctrl->status and ctrl->it
           if (t == 0) {
             ctrl->first = 1;
@@ -1283,7 +1304,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       } else {
         // ---- backtracking (rare): a -= f da, strains from a new sweep ----
         const TF f = ctrl->gi * (TF(1) - gamma);
-        for (int i = t; i < 3 * N; i += G) a_s[i] = hp_add_tf(a_s[i], -f * da_s[i]);
+        for (int i = t; i < 3 * N; i += T) a_s[i] = hp_add_tf(a_s[i], -f * da_s[i]);
         __syncthreads();
         sweep(SW_PLAIN, hp_zero(tag));  // its barriers also order the reads of ctrl->gi above
         if (t == 0) {
@@ -1314,7 +1335,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
     }
     __syncthreads();
     int bad = 0;
-    for (int c = t; c < kOutWords; c += G) {
+    for (int c = t; c < kOutWords; c += T) {
       double v;
       if (c < 6) v = hp_to(sroot[c]);
       else if (c < 42) v = double(sget(orec, (c - 6) / 6, (c - 6) % 6));
@@ -1332,13 +1353,13 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       P.status[pt] = (bad ? 2 : ctrl->status) | (attempt ? 4 : 0) | (bbad ? kPtBounds : 0);
       P.iters[pt] = ctrl->it + it_total;
     }
-    for (int c = t; c < 8; c += G) sout[c] = c < 6 ? ebd[c] : (c == 6 ? theta : 0.0);
-    for (int i = t; i < 3 * N; i += G) __stcs(sout + 8 + i, hp_to(a_s[i]));
+    for (int c = t; c < 8; c += T) sout[c] = c < 6 ? ebd[c] : (c == 6 ? theta : 0.0);
+    for (int i = t; i < 3 * N; i += T) __stcs(sout + 8 + i, hp_to(a_s[i]));
     if (LAW == 3) {  // each thread its own leaves (it parked their values itself)
 #pragma unroll 1
       for (int sd = 0; sd < 2; ++sd) {
         const int zo = sd ? zo1 : zo0, ph = sd ? ph1 : ph0;
-        if (zo < 0) continue;
+        if (zo < 0 || !bot) continue;
         if (mp_s[ph].kind == 3) {
           pa_finish<TF, HP>(mpa_s[ph], sin + zo, sout + zo);
         } else {
@@ -1351,16 +1372,16 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
         }
       }
     } else {
-      for (int i0 = t; i0 < ZW; i0 += 8 * G) {  // parked internal variables -> FP64 in place
+      for (int i0 = t; i0 < ZW; i0 += 8 * T) {  // parked internal variables -> FP64 in place
         HP v[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = i0 + u * G < ZW ? ld_once(zw + i0 + u * G) : hp_zero(tag);
+        for (int u = 0; u < 8; ++u) v[u] = i0 + u * T < ZW ? ld_once(zw + i0 + u * T) : hp_zero(tag);
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (i0 + u * G < ZW) __stcs(sout + 8 + 3 * N + i0 + u * G, hp_to(v[u]));
+          if (i0 + u * T < ZW) __stcs(sout + 8 + 3 * N + i0 + u * T, hp_to(v[u]));
       }
     }
-    for (int i = P.zend + t; i < P.SW; i += G) sout[i] = 0.0;  // padding word
+    for (int i = P.zend + t; i < P.SW; i += T) sout[i] = 0.0;  // padding word
     __syncthreads();
   }
 }
