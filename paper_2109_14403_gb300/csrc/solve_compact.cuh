@@ -966,6 +966,21 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
     } else {
       sweep(SW_PLAIN, hp_zero(tag));  // strains of the bottom laminates at a^n
     }
+    // jumps and (LAW < 3) internal variables of the pass to the output state, by
+    // `step` threads: FP64 from a_s and, in place, from the parked values
+    auto store_state = [&](int i0, int step) {
+      for (int i = i0; i < 3 * N; i += step) __stcs(sout + 8 + i, hp_to(a_s[i]));
+      if (LAW < 3)
+        for (int i = i0; i < ZW; i += 8 * step) {
+          HP v[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) v[u] = i + u * step < ZW ? ld_once(zw + i + u * step) : hp_zero(tag);
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (i + u * step < ZW) __stcs(sout + 8 + 3 * N + i + u * step, hp_to(v[u]));
+        }
+    };
+    bool stored = false;
     int attempt = 0, it_total = 0;
     HP Dsum = hp_zero(tag), Xsum = hp_zero(tag);
     Rec<TF> rec;
@@ -1183,6 +1198,20 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
           put_root(rec, S);
         }
       }
+      // ---- while warp L condenses the narrow levels, the others store the
+      //      state (10 k of a point's 140 k cycles stood alone at its end) if
+      //      this pass is likely the accepted one: a Newton step reduces the
+      //      residual by 1e4 and more where no leaf starts to yield, and most
+      //      warm starts need one step.  If it is not, the next pass parks its
+      //      values anew; storing after every pass that could end costs the
+      //      plastic ramp 2.5 %.  Behind the block barrier before the first
+      //      level, so the parked values are there.  (K = 7 uneven -3 %, one
+      //      element -3 %, K = 9 -1.5 %, warm K = 8 -1.6 %, ramp -0.8 %.  Not where
+      //      it lost: FP64, whose other warps share the FP64 pipe, +1.3 %;
+      //      Perzyna trees of K <= 8, +2 % of the cyclic workload.) ----
+      constexpr bool EARLY = !D64 && (LAW == 1 || (LAW == 2 && MAXT > 128));
+      stored = EARLY && full && nwarp > 1 && ctrl->res_old < tol * (P.da0 ? TF(1e7) : TF(1e4));
+      if (stored && warp != L) store_state(((warp - L - 1) & (nwarp - 1)) * 32 + lane, 32 * (nwarp - 1));
       // ---- residual norm, decision (Algorithm 1) ----
       r2 = warp_sum(r2, mask, W);
       if (lane == 0) red[warp] = r2;
@@ -1354,7 +1383,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       P.iters[pt] = ctrl->it + it_total;
     }
     for (int c = t; c < 8; c += T) sout[c] = c < 6 ? ebd[c] : (c == 6 ? theta : 0.0);
-    for (int i = t; i < 3 * N; i += T) __stcs(sout + 8 + i, hp_to(a_s[i]));
+    if (!stored) store_state(t, T);
     if (LAW == 3) {  // each thread its own leaves (it parked their values itself)
 #pragma unroll 1
       for (int sd = 0; sd < 2; ++sd) {
@@ -1370,15 +1399,6 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
             sout[zo + c] = hp_to(v);
           }
         }
-      }
-    } else {
-      for (int i0 = t; i0 < ZW; i0 += 8 * T) {  // parked internal variables -> FP64 in place
-        HP v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = i0 + u * T < ZW ? ld_once(zw + i0 + u * T) : hp_zero(tag);
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (i0 + u * T < ZW) __stcs(sout + 8 + 3 * N + i0 + u * T, hp_to(v[u]));
       }
     }
     for (int i = P.zend + t; i < P.SW; i += T) sout[i] = 0.0;  // padding word

@@ -69,3 +69,35 @@ def test_small_and_large_mixed_launches_agree_in_every_bit(K, variant):
             assert np.array_equal(out.cpu().numpy(), many[k][1][:n])
             assert np.array_equal(s.cpu().numpy(), many[k][0][:n])
         d.close()
+
+
+@pytest.mark.parametrize("K,maxit,tol,scale", [(7, 1, 1e-12, 8.0), (8, 2, 1e-12, 30.0), (8, 50, 1e-7, 30.0),
+                                               (7, 50, 1e-9, 20.0)])
+def test_states_of_passes_stored_early_or_late(K, maxit, tol, scale):
+    """The compact kernel stores the state beside the last pass's condensation
+    or after it, and again if the pass is not accepted: the state is that of
+    the owner-mapped kernel, which stores once, also where the iteration ends
+    by its limit.  Both stop with the same Newton steps in FP32: their jumps
+    differ by the residual the steps leave (tol, or the limit's) and rounding."""
+    from paper_2109_14403_gb300 import DMN
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev = torch.device("cuda:0")
+    n = 700
+    deps, theta = syn.random_walk_k8(n_points=n, n_incr=2)
+    res = {}
+    for variant in (3, 13):
+        d = DMN(K, *syn.tree(K), syn.materials(), tol=tol, maxit=maxit, precision="mixed", solve_variant=variant)
+        s = d.init_state(torch.full((n,), syn.THETA_START, dtype=torch.float64, device=dev))
+        s, out, st, it = d.eval(torch.tensor(scale * deps[0], device=dev), torch.tensor(theta[0], device=dev), 1.0, s)
+        res[variant] = (s.cpu().numpy(), out.cpu().numpy(), st.cpu().numpy(), it.cpu().numpy())
+        d.close()
+    a, b = res[3], res[13]
+    same = (a[3] == b[3]) & (a[2] == b[2])
+    assert same.mean() > 0.99
+    N3 = 3 * ((1 << K) - 1)
+    assert np.isfinite(b[0]).all()
+    assert np.array_equal(a[0][:, :7], b[0][:, :7])
+    for lo, hi in ((8, 8 + N3), (8 + N3, a[0].shape[1])):
+        x, y = a[0][same, lo:hi], b[0][same, lo:hi]
+        assert np.abs(x - y).max() <= 1e-5 * np.abs(x).max()
