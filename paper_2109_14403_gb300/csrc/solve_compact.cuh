@@ -422,6 +422,88 @@ __device__ __forceinline__ void combine_node(const SolveParams &P, int p, const 
   rec_put(dst, L);
 }
 
+// A node on eight lanes (combine_rows' mapping) with these formulas: 130 FP64
+// instructions, against 161
+__device__ __forceinline__ void combine_rows64(const SolveParams &P, int p, int r, bool st, unsigned mask,
+                                               const double *rcL, const double *rcR, const double *sL,
+                                               const double *sR, double *dst, double *sdst, double *gh, double &r2,
+                                               bool full, bool root) {
+  const int rw = r < 6 ? r : 5;
+  const int ra = rw == 2 ? 4 : 5, rb = rw == 0 ? 4 : 3;  // rows coupled with component e = rw < 3
+  const int ia = rw == 0 ? 1 : 0, ib = rw == 2 ? 1 : 2;
+  const bool own = st && r < 6;
+  auto sh = [&](double v, int src) { return __shfl_sync(mask, v, src, 8); };
+  NodeHP<double> nd;
+  load_node(P, p, nd);
+  const double iwcc = ld_keep(P.node + kNodeWords * DMN_IDX(p, P.N) + 7);
+  const double c1 = nd.c1, c2 = nd.c2, cc = c1 * c2;
+  const double ne = pick3(nd.n, rw), na = pick3(nd.ns, ia), nb = pick3(nd.ns, ib);
+  // traction component e = rw of a Mandel vector whose component rw is v
+  auto bt_e = [&](double v) { return fma(v, ne, fma(sh(v, ra), na, sh(v, rb) * nb)); };
+  const int rbase = rw * (11 - rw) / 2;  // packed index of (rw, rw) minus rw
+  double xr[6], dC[6], U[3], m[3], V[3], W[3], Ki[3][3];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int q = c >= rw ? rbase + c : c * (11 - c) / 2 + rw;
+    xr[c] = rcR[q];
+    dC[c] = rcL[q] - xr[c];
+  }
+  btvec_hp(nd, dC, U);
+  btvec_hp(nd, xr, m);
+#pragma unroll
+  for (int f = 0; f < 3; ++f) m[f] = bt_e(fma(c2, U[f], m[f]));  // row e of K on lane e
+  const double k6[6] = {sh(m[0], 0), sh(m[1], 0), sh(m[2], 0), sh(m[1], 1), sh(m[2], 1), sh(m[2], 2)};
+  inv_sym3(k6, Ki);
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    V[e] = dot3(Ki[e], U);
+    if (own) gh[6 * e + r] = V[e];
+    W[e] = cc * V[e];
+  }
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    double x = fma(c1, dC[c], xr[c]);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) x = fma(-U[e], sh(W[e], c), x);
+    if (own && c >= rw) dst[rbase + c] = x;
+  }
+  // residual r_p = w c1 c2 B^T (c2 S_L - c1 S_R), component e on lane e
+  const double SL = sL[rw], SR = sR[rw], re = bt_e(c2 * SL - c1 * SR);
+  if (own) sdst[r] = SL + SR;
+  if (st && r < 3) r2 = fma(re, re, r2);
+  // v <- c1 v_L + c2 v_R - c1 c2 U K^-1 (b + B^T (v_L - v_R)); t, h: the solve
+  auto vec = [&](int off, double b, double t[3], double h[3]) {
+    const double vr = rcR[off + rw], d = rcL[off + rw] - vr, te = bt_e(d) + b;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) t[e] = sh(te, e);
+    double x = fma(c1, d, vr);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      h[e] = dot3(Ki[e], t);
+      x = fma(U[e], -cc * h[e], x);
+    }
+    return x;
+  };
+  double t[3], h[3];
+  const double ds = vec(21, re * iwcc, t, h);
+  if (st && r == 0) {
+#pragma unroll
+    for (int e = 0; e < 3; ++e) gh[18 + e] = h[e];
+  }
+  if (own && !root) dst[21 + r] = ds;
+  if (full) {
+    double ht[3];
+    const int o = root ? 21 : 27;  // the output layout of orec: tau at 21, dd at 27, g at 33
+    const double tau = vec(27, 0.0, t, ht), dd = vec(33, 0.0, t, h);
+    const double gR = rcR[39], gg = fma(c1, rcL[39] - gR, gR) - cc * dot3(t, ht);
+    if (own) {
+      dst[o + r] = tau;
+      dst[o + 6 + r] = dd;
+      if (r == 0) dst[o + 12] = gg;
+    }
+  }
+}
+
 // A node on two lanes (2i, 2i + 1 of an aligned pair): lane h owns Mandel rows
 // 3h .. 3h + 2.  Sums over rows (K, the right-hand sides) are halves added by a
 // shuffle; of C_hat a lane forms its own 3 x 3 block's upper triangle and, of
@@ -554,6 +636,42 @@ __device__ __forceinline__ void combine_half(const SolveParams &P, int p, int h,
     vec(33, nullptr, t, hs);
     const double gR = rcR[39], gg = fma(c1, rcL[39] - gR, gR) - cc * dot3(t, ht);
     if (st && h == 0) dst[39] = gg;
+  }
+}
+
+// Back-substitution of level k <= 4 on one warp, eight lanes a node: da_p =
+// -(G_p de_p + h_p), children's de +- c B da into the next level's buffer, and at
+// the bottom level (k = K) a += da.
+__device__ __forceinline__ void step_rows64(const SolveParams &P, int k, int lane, unsigned mask, const double *src,
+                                            double *nxt, const double *gh, double *da, double *a) {
+  const int cnt = 1 << (k - 1), r = lane & 7, e = r < 3 ? r : 2, c = r < 6 ? r : 5;
+  for (int q = lane >> 3; q < ((cnt + 3) & ~3); q += 4) {
+    const bool st = q < cnt;
+    const int j = st ? q : cnt - 1, p = DMN_IDX((1 << P.K) - (1 << k) + j, P.N);
+    const double *g = gh + 21 * p;
+    double x = g[18 + e];
+    if (src) {
+#pragma unroll
+      for (int i = 0; i < 6; ++i) x = fma(g[6 * e + i], src[6 * j + i], x);
+    }
+    x = -x;
+    if (st && r < 3) {
+      da[3 * p + r] = x;
+      if (k == P.K) a[3 * p + r] += x;
+    }
+    if (k < P.K) {
+      NodeHP<double> nd;
+      load_node(P, p, nd);
+      const double d[3] = {__shfl_sync(mask, x, 0, 8), __shfl_sync(mask, x, 1, 8), __shfl_sync(mask, x, 2, 8)};
+      // J = u d[i] + v d[i']: c < 3: n_c d_c; the shear components two terms
+      const int i0 = c < 3 ? c : (c == 3 ? 1 : 0), i1 = c < 3 ? c : (c == 5 ? 1 : 2);
+      const double u = c < 3 ? pick3(nd.n, c) : pick3(nd.ns, i1), v = c < 3 ? 0.0 : pick3(nd.ns, i0);
+      const double J = fma(u, pick3(d, i0), v * pick3(d, i1)), de = src ? src[6 * j + c] : 0.0;
+      if (st && r < 6) {
+        nxt[12 * j + c] = fma(nd.c2, J, de);
+        nxt[12 * j + 6 + c] = fma(-nd.c1, J, de);
+      }
+    }
   }
 }
 
@@ -1162,9 +1280,13 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
                 combine_half(P, p, q & 1, st, mask, rc, rc + RS, sc, sc + 6, dst, sd, gh_s + 21 * p, r2, full);
                 continue;
               }
+              combine_rows64(P, p, q & 7, st, mask, rc, rc + RS, sc, sc + 6, dst, sd, gh_s + 21 * p, r2, full,
+                             k == 1);
+              continue;
             }
-            combine_rows<TF, HP>(P, p, q & 7, st, mask, rc, rc + RS, sc, sc + 6, dst, sd, gh_s + 21 * p, r2,
-                                 full, k == 1);
+            if constexpr (!D64)
+              combine_rows<TF, HP>(P, p, q & 7, st, mask, rc, rc + RS, sc, sc + 6, dst, sd, gh_s + 21 * p, r2,
+                                   full, k == 1);
           }
         }
       } else if (K == 3) {
@@ -1225,9 +1347,15 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
           const TF v = tf_of(sroot[c], (TF *)nullptr);
           sn += v * v;
         }
-        TF den = sqrt(sn);
-        if (den < res_floor) den = res_floor;
-        const TF res = sqrt(s) / (TF(N) * den);
+        TF res;
+        if constexpr (D64) {  // one square root: the other warps wait
+          const double f2 = res_floor * res_floor;
+          res = sqrt(s / ((double(N) * N) * (sn < f2 ? f2 : sn)));
+        } else {
+          TF den = sqrt(sn);
+          if (den < res_floor) den = res_floor;
+          res = sqrt(s) / (TF(N) * den);
+        }
         Ctrl<TF> &c = *ctrl;
         const bool accept = c.first || (res < c.res_old) || (c.bt >= P.maxbt);
         int action;
@@ -1285,7 +1413,16 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
         //      B da terms of their ancestors
         for (int k = 1; k <= K; ++k) {
           const int j = node_at(k);  // level K: j = t
-          if (j >= 0) {
+          bool on_rows = false;
+          if constexpr (D64) {
+            // a node on eight lanes: component e of da on lane e < 3, Mandel
+            // component c of B da and of the children on lane c < 6 (10 FP64
+            // instructions a round of four nodes, against 42)
+            on_rows = k <= 4;
+            if (on_rows && warp == L)
+              step_rows64(P, k, lane, mask, k == 1 ? nullptr : tbuf(k), tbuf(k + 1), gh_s, da_s, a_s);
+          }
+          if (!on_rows && j >= 0) {
             const int p = DMN_IDX((1 << K) - (1 << k) + j, N);
             TF de[6];
             if (k == 1) {
