@@ -72,6 +72,10 @@ bool gemm_args_ok(const void *A, const void *B, int M, int N, int K) {
          !((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15);
 }
 
+// a product whose tiles are all resident at once is short: its launch overlaps
+// the one before it (pdl.cuh)
+bool overlaps(int M, int N) { return (M / BM) * (N / BN) <= 2 * g_gemm_sms; }
+
 // C = A . B^T with the fused epilogue ep; A [M x K], B [N x K] bf16; rows of A
 // from a_rows on read as zero.  N a multiple of 256 and a 128 x 256 tile for
 // every SM: the persistent wide form (one CTA per SM), else (and with z_out or
@@ -93,8 +97,8 @@ cudaError_t gemm(cudaStream_t s, const void *A, const void *B, int M, int N, int
     return cudaGetLastError();
   }
   if (!make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
-  gemm_bf16_tile<false, false, BN, STAGES><<<dim3(N / BN, M / BM), 128, GEMM_SMEM, s>>>(ma, mb, K, ep);
-  return cudaGetLastError();
+  return launch_chained(overlaps(M, N), gemm_bf16_tile<false, false, BN, STAGES>, dim3(N / BN, M / BM), dim3(128),
+                        GEMM_SMEM, s, ma, mb, K, ep);
 }
 // input gradient: C [M x N] = A . B, A [M x K], B [K x N] as stored
 cudaError_t gemm_dgrad(cudaStream_t s, const void *A, const void *B, int M, int N, int K, EpiArgs ep) {
@@ -103,8 +107,8 @@ cudaError_t gemm_dgrad(cudaStream_t s, const void *A, const void *B, int M, int 
   if (e != cudaSuccess) return e;
   CUtensorMap ma, mb;
   if (!make_map(&ma, A, M, K) || !make_map(&mb, B, K, N, BK)) return cudaErrorInvalidValue;
-  gemm_bf16_tile<false, true, BN, STAGES><<<dim3(N / BN, M / BM), 128, GEMM_SMEM, s>>>(ma, mb, K, ep);
-  return cudaGetLastError();
+  return launch_chained(overlaps(M, N), gemm_bf16_tile<false, true, BN, STAGES>, dim3(N / BN, M / BM), dim3(128),
+                        GEMM_SMEM, s, ma, mb, K, ep);
 }
 // adds layer l's weight gradient to a launch: C [M x N] (fp32) = A^T . B, A [K x
 // M], B [K x N] (rows from b_rows on read as zero)
@@ -314,6 +318,7 @@ struct ColsumArgs {
 };
 __global__ void __launch_bounds__(1024) k_colsum(const ColsumArgs A) {
   __shared__ float2 red[32][32];
+  chain_begin();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (int(blockIdx.x) == A.blk0[A.layers]) {
     __shared__ double rl[32];
@@ -382,6 +387,7 @@ __global__ void __launch_bounds__(256)
     k_amsgrad_pack(int64_t count4, float4 *w, const float4 *g, float4 *m, float4 *v, float4 *vmax, AmsArgs a,
                    const PackArgs P) {
   const int64_t i = blockIdx.x * int64_t(256) + threadIdx.x;
+  chain_begin();
   if (i >= count4) return;
   const float4 gi = g[i];
   float4 wi = w[i], mi = m[i], vi = v[i], xi = vmax[i];
@@ -763,8 +769,10 @@ extern "C" dmn_status dmn_mlp_train_step(dmn_mlp m, dmn_stream stream, int64_t n
     if (!wgrad_add(wg, m->dz[l], l == 0 ? x : m->h[l - 1], m->dout[l], m->din[l], int(npad), m->grads + m->ow[l],
                    l == 0 ? n : npad))
       return cuda_fail(cudaErrorInvalidValue, "wgrad");
-  gemm_bf16_wgrad<<<wg.blk0[m->L], 128, tile_smem(WG_BN, WG_ST), s>>>(wg, int(npad));
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "wgrad");
+  const bool small = overlaps(int(npad), m->H);
+  if ((e = launch_chained(small, gemm_bf16_wgrad, dim3(wg.blk0[m->L]), dim3(128), tile_smem(WG_BN, WG_ST), s, wg,
+                          int(npad))) != cudaSuccess)
+    return cuda_fail(e, "wgrad");
   ColsumArgs C = {};
   PackArgs P = {};
   C.layers = P.layers = m->L;
@@ -782,14 +790,15 @@ extern "C" dmn_status dmn_mlp_train_step(dmn_mlp m, dmn_stream stream, int64_t n
   C.loss_part = m->lpart;
   C.loss = d_loss;
   C.lscale = 1.0f / (float(n) * float(m->n3));
-  k_colsum<<<C.blk0[m->L] + (d_loss ? 1 : 0), 1024, 0, s>>>(C);
+  e = launch_chained(small, k_colsum, dim3(C.blk0[m->L] + (d_loss ? 1 : 0)), dim3(1024), 0, s, C);
+  if (e != cudaSuccess) return cuda_fail(e, "bias gradients");
   m->step += 1;
   const int64_t n4 = m->nparam / 4;
-  k_amsgrad_pack<<<unsigned((n4 + 255) / 256), 256, 0, s>>>(
-      n4, reinterpret_cast<float4 *>(m->params), reinterpret_cast<const float4 *>(m->grads),
+  e = launch_chained(
+      small, k_amsgrad_pack, dim3(unsigned((n4 + 255) / 256)), dim3(256), 0, s, n4, reinterpret_cast<float4 *>(m->params), reinterpret_cast<const float4 *>(m->grads),
       reinterpret_cast<float4 *>(m->m), reinterpret_cast<float4 *>(m->v), reinterpret_cast<float4 *>(m->vmax),
       ams_args(lr, kBeta1, kBeta2, kEps, m->step), P);
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dmn_mlp_train_step");
+  if (e != cudaSuccess) return cuda_fail(e, "dmn_mlp_train_step");
   return DMN_OK;
 }
 

@@ -28,6 +28,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "pdl.cuh"
+
 namespace dmn {
 namespace mlp {
 
@@ -400,6 +402,7 @@ template <bool AMN, bool BMN, int BNT, int NST>
 __global__ void __launch_bounds__(128, 2)
     gemm_bf16_tile(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                    int K, const EpiArgs ep) {
+  chain_begin();
   gemm_tile_body<AMN, BMN, BNT, NST>(map_a, map_b, K, ep, blockIdx.x, blockIdx.y);
 }
 
@@ -417,6 +420,7 @@ struct WgradArgs {
 };
 static_assert(sizeof(WgradArgs) <= 4000, "kernel parameters");
 __global__ void __launch_bounds__(128, 2) gemm_bf16_wgrad(const __grid_constant__ WgradArgs A, int K) {
+  chain_begin();
   int l = 0;
   while (int(blockIdx.x) >= A.blk0[l + 1]) ++l;
   const int q = int(blockIdx.x) - A.blk0[l];
