@@ -177,8 +177,9 @@ __global__ void k_features(int64_t n, int n3, int sw, const double *deps, const 
 // warp per row, each lane two adjacent columns per step (one bf16x2 store;
 // ld = kin is a multiple of 128, so the pairs stay 4-byte aligned).  Bound by the
 // two states' jumps it reads (12 KB a row at K = 8).  VEC: a lane's pair of jumps
-// as one 16-byte load, four steps in flight (states 16-byte aligned, an even
-// number of words); else word by word.
+// as one 16-byte load, two steps in flight (states 16-byte aligned, an even
+// number of words; 65,536 rows 166 us, one step 173, four 178, seven 193); else
+// word by word (180).
 template <bool VEC>
 __global__ void __launch_bounds__(256)
     k_features_norm(int64_t n, int n3, int sw, int ld, const double *deps, const double *theta, const double *sin,
@@ -197,15 +198,15 @@ __global__ void __launch_bounds__(256)
       xr[c0 >> 1] = __floats2bfloat162_rn(v0, v1);
     };
     if (VEC && ap) {
-      constexpr int U = 4;
+      constexpr int U = 2;
       for (int c0 = 2 * lane; c0 < ld; c0 += 64 * U) {
         double2 q[U], p[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int c = c0 + 64 * u;
           const bool in = c >= 8 && c + 1 < sw && c < nin;  // c + 1 == nin: the word after the jumps
-          q[u] = in ? __ldcs(reinterpret_cast<const double2 *>(a + c)) : make_double2(0.0, 0.0);
-          p[u] = in ? __ldcs(reinterpret_cast<const double2 *>(ap + c)) : make_double2(0.0, 0.0);
+          q[u] = in ? *reinterpret_cast<const double2 *>(a + c) : make_double2(0.0, 0.0);
+          p[u] = in ? *reinterpret_cast<const double2 *>(ap + c) : make_double2(0.0, 0.0);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
