@@ -839,6 +839,108 @@ __global__ void __launch_bounds__(kLvlThreads, 3) k_lvl_bwd2(int K, int k, int64
   }
 }
 
+// The same for a small batch, where a launch is as long as one thread's chain:
+// the two children on two threads (warps w and w + 4 of 8), so a chain of two
+// laminates, not three.  Forward: the second child's stiffness to the first's
+// thread through shared memory.  Reverse: both threads take the parent, each its
+// own child.  (K = 8, 32 samples: 93 -> 84 us.)
+template <bool LEAF, typename T>
+__global__ void __launch_bounds__(2 * kLvlThreads, 1)
+    k_lvl_fwd2s(int K, int k, int64_t n, const T *PH, const T *nh, const T *c1s, T *NS) {
+  __shared__ T ys[21][kLvlThreads];
+  chain_begin();
+  const int t = threadIdx.x % kLvlThreads, c = threadIdx.x / kLvlThreads;
+  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + t;
+  const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j, pc = (1 << K) - (1 << (k + 1)) + 2 * j + c;
+  const int pg = (1 << K) - (1 << (k + 2)) + 4 * j + 2 * c;  // grandchildren of this child
+  T X[21];
+  if (s < n) {
+    T CL[21], CR[21];
+    lvl_load(LEAF ? PH : NS, LEAF ? 0 : pg, n, s, CL);
+    lvl_load(LEAF ? PH : NS, LEAF ? 1 : pg + 1, n, s, CR);
+    const T nn[3] = {nh[3 * pc], nh[3 * pc + 1], nh[3 * pc + 2]};
+    lam_forward(CL, CR, nn, c1s[pc], X);
+    if (c == 1)
+#pragma unroll
+      for (int q = 0; q < 21; ++q) ys[q][t] = X[q];
+    lvl_store(NS, pc, n, s, X);
+  }
+  __syncthreads();
+  if (c == 0 && s < n) {
+    T Y[21], out[21];
+#pragma unroll
+    for (int q = 0; q < 21; ++q) Y[q] = ys[q][t];
+    const T nn[3] = {nh[3 * pp], nh[3 * pp + 1], nh[3 * pp + 2]};
+    lam_forward(X, Y, nn, c1s[pp], out);
+    lvl_store(NS, pp, n, s, out);
+  }
+}
+
+template <bool LEAF, typename T>
+__global__ void __launch_bounds__(2 * kLvlThreads, 1)
+    k_lvl_bwd2s(int K, int k, int64_t n, const T *PH, const T *nh, const T *c1s, const T *NS, T *GA, double *gnh,
+                double *gc1) {
+  __shared__ T red[3][4][kLvlThreads / 32];
+  chain_begin();
+  const int t = threadIdx.x % kLvlThreads, c = threadIdx.x / kLvlThreads;
+  const int64_t s = int64_t(blockIdx.x) * kLvlThreads + t;
+  const int j = blockIdx.y, pp = (1 << K) - (1 << k) + j, pc = (1 << K) - (1 << (k + 1)) + 2 * j;
+  const int pg = (1 << K) - (1 << (k + 2)) + 4 * j + 2 * c;
+  const int lane = t & 31, warp = t >> 5;
+  auto warp_sums = [&](int node, const T gn[3], T g1) {
+    T r[4] = {gn[0], gn[1], gn[2], g1};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) r[i] += __shfl_down_sync(0xffffffffu, r[i], o);
+    if (lane == 0)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) red[node][i][warp] = r[i];
+  };
+  T G[21];
+  {
+    T gn[3] = {T(0), T(0), T(0)}, g1 = T(0);
+    if (s < n) {
+      T CL[21], CR[21], GL[21], GR[21];
+      lvl_load(NS, pc, n, s, CL);
+      lvl_load(NS, pc + 1, n, s, CR);
+      lvl_load(GA, pp, n, s, G);
+      const T nn[3] = {nh[3 * pp], nh[3 * pp + 1], nh[3 * pp + 2]};
+      lam_backward<true>(CL, CR, nn, c1s[pp], G, GL, GR, gn, g1);
+#pragma unroll
+      for (int q = 0; q < 21; ++q) G[q] = c ? GR[q] : GL[q];
+    }
+    if (c == 0) warp_sums(0, gn, g1);
+  }
+  {
+    T gn[3] = {T(0), T(0), T(0)}, g1 = T(0);
+    if (s < n) {
+      T CL[21], CR[21];
+      lvl_load(LEAF ? PH : NS, LEAF ? 0 : pg, n, s, CL);
+      lvl_load(LEAF ? PH : NS, LEAF ? 1 : pg + 1, n, s, CR);
+      const int p = pc + c;
+      const T nn[3] = {nh[3 * p], nh[3 * p + 1], nh[3 * p + 2]};
+      if (LEAF) {
+        T *none = nullptr;
+        lam_backward<false>(CL, CR, nn, c1s[p], G, none, none, gn, g1);
+      } else {
+        T HL[21], HR[21];
+        lam_backward<true>(CL, CR, nn, c1s[p], G, HL, HR, gn, g1);
+        lvl_store(GA, pg, n, s, HL);
+        lvl_store(GA, pg + 1, n, s, HR);
+      }
+    }
+    warp_sums(1 + c, gn, g1);
+  }
+  __syncthreads();
+  if (threadIdx.x < 12) {
+    const int node = threadIdx.x >> 2, i = threadIdx.x & 3, p = node == 0 ? pp : pc + node - 1;
+    T acc = T(0);
+    for (int w = 0; w < kLvlThreads / 32; ++w) acc += red[node][i][w];
+    atomicAdd(i < 3 ? gnh + 3 * p + i : gc1 + p, double(acc));
+  }
+}
+
 // The chain through the weights (c1 = W_1 / W, w = <v>_+, penalty) and the
 // normalisation of the normals: one CTA.  Its second half takes the normals;
 // the first the weights level by level, then every node's two quotients at
@@ -960,6 +1062,7 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   // launch: 32 samples, K = 8: 107 -> 93 us with the eight-lane kernels); a large
   // one's do not (65,536 samples: early CTAs of the next level cost 4 %)
   const bool small = n <= 2048;
+  const bool split = n <= kLvlThreads;  // a block of samples: at most 2^(K-2) CTAs a launch
   auto go = [&](auto f, dim3 grid, unsigned threads, auto... args) {
     if (e == cudaSuccess) e = launch_chained(small, f, grid, dim3(threads), 0, st, args...);
   };
@@ -968,9 +1071,11 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   // level, and bound by the FP64 pipe, so one level a launch)
   int k = K;
   if constexpr (sizeof(T) == 4)
-    for (; k >= 2; k -= 2)
-      go(k == K ? k_lvl_fwd2<true, T> : k_lvl_fwd2<false, T>, dim3(nb, 1u << (k - 2)), kLvlThreads, K, k - 1, n, PH,
-         nh, c1s, NS);
+    for (; k >= 2; k -= 2) {
+      const auto f = split ? (k == K ? k_lvl_fwd2s<true, T> : k_lvl_fwd2s<false, T>)
+                           : (k == K ? k_lvl_fwd2<true, T> : k_lvl_fwd2<false, T>);
+      go(f, dim3(nb, 1u << (k - 2)), split ? 2 * kLvlThreads : kLvlThreads, K, k - 1, n, PH, nh, c1s, NS);
+    }
   for (; k >= 1; --k) go(k_lvl_fwd<T>, dim3(nb, 1u << (k - 1)), kLvlThreads, K, k, n, PH, nh, c1s, NS);
   // the blocks' partial sums: in the adjoints' array, free until the seed, from an 8-byte boundary
   double *part = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(GA) + 7) & ~uintptr_t(7));
@@ -994,9 +1099,11 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
       go(k_lvl_bwd<T>, dim3(nb, 1), kLvlThreads, K, 1, n, PH, nh, c1s, NS, GA, gnh, gc1);
       k = 2;
     }
-    for (; k < K; k += 2)
-      go(k + 1 == K ? k_lvl_bwd2<true, T> : k_lvl_bwd2<false, T>, dim3(nb, 1u << (k - 1)), kLvlThreads, K, k, n, PH,
-         nh, c1s, NS, GA, gnh, gc1);
+    for (; k < K; k += 2) {
+      const auto f = split ? (k + 1 == K ? k_lvl_bwd2s<true, T> : k_lvl_bwd2s<false, T>)
+                           : (k + 1 == K ? k_lvl_bwd2<true, T> : k_lvl_bwd2<false, T>);
+      go(f, dim3(nb, 1u << (k - 1)), split ? 2 * kLvlThreads : kLvlThreads, K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
+    }
   }
   for (; k <= K; ++k) go(k_lvl_bwd<T>, dim3(nb, 1u << (k - 1)), kLvlThreads, K, k, n, PH, nh, c1s, NS, GA, gnh, gc1);
   go(k_lin_finish, dim3(1), kSetupThreads, K, normals, v, penalty, gnh, gc1, scal, grad_n, grad_v);
