@@ -181,12 +181,10 @@ def solve_kernel_name(variant, precision, law=1):
                 else "dmn_solve_compact<float, dfl, 128, 3, 2>")
     if 22 <= variant <= 24 and precision == "mixed":
         return f"dmn_solve_warp<8, 4, {variant - 20}, 1>"
-    if variant >= 11:
-        if precision == "fp64":
-            return "dmn_solve_compact<double, double, 128, 1, 1>"
-        return f"dmn_solve_compact<float, dfl, 128, {max(2, variant - 10)}, 1>"
     if precision == "fp64":
-        return "dmn_solve_kernel<double, double, 128, 1>"
+        return "dmn_solve_compact<double, double, 128, 1, 1>"
+    if variant >= 11:
+        return f"dmn_solve_compact<float, dfl, 128, {max(2, variant - 10)}, 1>"
     return f"dmn_solve_kernel<float, dfl, 128, {variant if variant in (2, 4) else 3}>"
 
 
@@ -664,7 +662,7 @@ def run_cyclic(args):
                          "passes_per_eval": passes,
                          "hbm": {"achieved": hbm, "peak": peak, "unit": "GB/s", "frac": hbm / peak,
                                  "peak_source": how, "bytes_per_eval": bpe}},
-            "clocks": clk.summary(), "gpu_launches": 2 * evals + 2 * steps}
+            "clocks": clk.summary(), "gpu_launches": 3 * evals + 2 * steps}
     if not args.no_cpu_baseline and world == 1:
         line["cpu_baseline"] = cpu_baseline_cyclic(n_points=32 if pa66 else 256, pa66=pa66)
     print(json.dumps(line), flush=True)
@@ -673,13 +671,13 @@ def run_cyclic(args):
 
 
 def lin_flops_per_sample(K):
-    """Algorithmic FLOPs of one training step per sample: one forward sweep at
-    ~975 per laminate (U = D B, M B, B^T M B, its inverse, U K^-1, the 21
-    outputs) and one reverse sweep at ~2350 per laminate (the forward
-    intermediates again, A, Q, the three inner products, dJ/dB, B Q and the
-    two child adjoints)."""
+    """Algorithmic FLOPs of one training step per sample, the zeros of B left
+    out: one forward sweep at ~650 per laminate (D, M, U = D B, M B, B^T M B, its
+    inverse, U K^-1: 435; the 21 outputs) and one reverse sweep at ~1070 (the
+    435 again, A, Q, the three inner products, dJ/dB) plus ~414 for B Q and the
+    two children's adjoints where the children are laminates."""
     N = (1 << K) - 1
-    return N * (975 + 2350)
+    return N * (650 + 1070) + (N >> 1) * 414
 
 
 def run_linear(args):
@@ -746,8 +744,8 @@ def run_linear(args):
             "roofline": {"bound": "alu", "achieved": fl, "peak": FP32_PEAK if prec == "fp32" else FP64_PEAK,
                          "unit": "TFLOP/s", "frac": fl / (FP32_PEAK if prec == "fp32" else FP64_PEAK),
                          "traffic": None,
-                         "kernel": f"k_lvl_bwd<{'float' if prec == 'fp32' else 'double'}> + "
-                                   "k_lvl_fwd (whole step)", "flops_per_sample": lin_flops_per_sample(K)},
+                         "kernel": ("k_lvl_bwd2<float> + k_lvl_fwd2<float> (whole step)" if prec == "fp32"
+                                    else "k_lvl_bwd<double> + k_lvl_fwd<double> (whole step)"), "flops_per_sample": lin_flops_per_sample(K)},
             "clocks": clk.summary(), "gpu_launches": ((K + 6 + (K & 1)) if prec == "fp32" else 2 * K + 6) * steps}
     if not args.no_cpu_baseline and world == 1:
         import oracle.linear as olin

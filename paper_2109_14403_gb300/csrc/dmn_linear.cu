@@ -7,11 +7,11 @@
 // over the batch; the laminates of a level run one per thread, the levels one
 // after another with a barrier, the node stiffnesses in shared memory.
 // dmn_linear_loss_grad: level-synchronous over the whole batch, one launch
-// per level and direction, every (sample, node) pair a thread, the node
-// stiffnesses and their adjoints in the caller's workspace; the backward pass
-// walks the tree top-down: per node it turns the adjoint G of its stiffness
-// into the adjoints of its two children and into dJ/dn and dJ/dc1, which each
-// block sums over its samples before one FP64 atomic add.
+// per level (FP32: two levels) and direction, every (sample, node) pair a
+// thread, the node stiffnesses and their adjoints in the caller's workspace;
+// the backward pass walks the tree top-down: per node it turns the adjoint G of
+// its stiffness into the adjoints of its two children and into dJ/dn and
+// dJ/dc1, which each block sums over its samples before one FP64 atomic add.
 // A laminate is computed in condensed form: with D = C_L - C_R, M = c2 C_L +
 // c1 C_R, U = D B, K = B^T M B,
 //   C = c1 C_L + c2 C_R - c1 c2 U K^-1 U^T,

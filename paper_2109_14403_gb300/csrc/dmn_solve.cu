@@ -460,10 +460,10 @@ static size_t owner_smem_bytes(int K, int zw, int n_mats, bool mixed) {
 // FP64, K <= 9: the compact kernel, whatever the variant (the owner-mapped form
 // has each level's nodes on one lane per warp or less, and an FP64 warp
 // instruction costs the same however few lanes are active: 1.4 to 2.0 times
-// the time at every K = 3..8, from 32 to 65,536 points).  Mixed: 0 = default;
-// 2..4 = owner-mapped kernel for that many CTAs per SM; 10 + m = compact kernel
-// (dmn_solve_compact.cu) compiled for m = 2, 3 or 4 CTAs per SM (11 runs as
-// 12).  Deeper trees take the owner-mapped 512-thread kernel.  A tree with
+// the time at every K = 3..8, from 32 to 65,536 points; 2.8 times at K = 9, 64 to
+// 8,192 points).  Mixed: 0 = default; 2..4 = owner-mapped kernel for that many
+// CTAs per SM; 10 + m = compact kernel (dmn_solve_compact.cu) compiled for m =
+// 2, 3 or 4 CTAs per SM (11 runs as 12).  Deeper trees take the owner-mapped 512-thread kernel.  A tree with
 // Perzyna leaves (law 2) always takes the compact instances that include that
 // leaf law (dmn_solve_compact_vp.cu, K <= 9), whatever the variant; one with
 // PA66 leaves (law 3) the instances of dmn_solve_compact_pa66.cu (K <= 8).
