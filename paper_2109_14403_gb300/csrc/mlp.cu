@@ -306,58 +306,6 @@ __global__ void k_norm_t(int64_t n, int nout, int ld, const float *tgt, const fl
   }
 }
 
-// Bias gradients of every layer in one launch: the column sums of dZ_l [npad x
-// C_l], 64 columns a CTA, 32 warps over the rows; the last block adds up the
-// loss (the warps' sums of squares, FP64, fixed order).
-struct ColsumArgs {
-  int layers, npad, nloss, blk0[kMaxLayers + 1];  // first block of each layer
-  const bf16 *dz[kMaxLayers];
-  float *db[kMaxLayers];
-  int cols[kMaxLayers];
-  const float *loss_part;
-  float *loss, lscale;
-};
-__global__ void __launch_bounds__(1024) k_colsum(const ColsumArgs A) {
-  __shared__ float2 red[32][32];
-  chain_begin();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (int(blockIdx.x) == A.blk0[A.layers]) {
-    __shared__ double rl[32];
-    double s = 0.0;
-    for (int i = threadIdx.x; i < A.nloss; i += 1024) s += double(A.loss_part[i]);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) rl[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < 32; ++w) s += rl[w];
-      *A.loss = float(s * double(A.lscale));
-    }
-    return;
-  }
-  int l = 0;
-  while (int(blockIdx.x) >= A.blk0[l + 1]) ++l;
-  const int c = (int(blockIdx.x) - A.blk0[l]) * 64 + 2 * lane, C = A.cols[l];
-  const bf16 *p = A.dz[l] + c;
-  float2 s = {0.0f, 0.0f};
-#pragma unroll 32
-  for (int r = warp; r < A.npad; r += 32) {
-    const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p + size_t(r) * C));
-    s.x += v.x;
-    s.y += v.y;
-  }
-  red[warp][lane] = s;
-  __syncthreads();
-  // pairwise over the warps (the tree of a warp's shuffle reduction)
-  for (int o = 16; o > 0; o >>= 1) {
-    if (warp < o) {
-      red[warp][lane].x += red[warp + o][lane].x;
-      red[warp][lane].y += red[warp + o][lane].y;
-    }
-    __syncthreads();
-  }
-  if (warp == 0) *reinterpret_cast<float2 *>(A.db[l] + c) = red[0][lane];
-}
-
 // AMSGrad with bias correction (Reddi, Kale, Kumar 2018; the maximum of the
 // second-moment estimates replaces it in the step size)
 struct AmsArgs {
@@ -770,29 +718,25 @@ extern "C" dmn_status dmn_mlp_train_step(dmn_mlp m, dmn_stream stream, int64_t n
     if (!wgrad_add(wg, m->dz[l], l == 0 ? x : m->h[l - 1], m->dout[l], m->din[l], int(npad), m->grads + m->ow[l],
                    l == 0 ? n : npad))
       return cuda_fail(cudaErrorInvalidValue, "wgrad");
-  const bool small = overlaps(int(npad), m->H);
-  if ((e = launch_chained(small, gemm_bf16_wgrad, dim3(wg.blk0[m->L]), dim3(128), tile_smem(WG_BN, WG_ST), s, wg,
-                          int(npad))) != cudaSuccess)
-    return cuda_fail(e, "wgrad");
-  ColsumArgs C = {};
   PackArgs P = {};
-  C.layers = P.layers = m->L;
-  C.npad = int(npad);
+  P.layers = m->L;
   for (int l = 0; l < m->L; ++l) {
-    C.dz[l] = m->dz[l];
-    C.db[l] = m->grads + m->ob[l];
-    C.cols[l] = m->dout[l];
-    C.blk0[l + 1] = C.blk0[l] + m->dout[l] / 64;
+    wg.dz[l] = m->dz[l];
+    wg.db[l] = m->grads + m->ob[l];
+    wg.cols[l] = m->dout[l];
+    wg.cblk0[l + 1] = wg.cblk0[l] + m->dout[l] / CS_COLS;
     P.ow[l] = m->ow[l];
     P.ob[l] = m->ob[l];
     P.w[l] = m->w[l];
   }
-  C.nloss = int(npad / BM) * (m->nout_pad / BN) * 4;
-  C.loss_part = m->lpart;
-  C.loss = d_loss;
-  C.lscale = 1.0f / (float(n) * float(m->n3));
-  e = launch_chained(small, k_colsum, dim3(C.blk0[m->L] + (d_loss ? 1 : 0)), dim3(1024), 0, s, C);
-  if (e != cudaSuccess) return cuda_fail(e, "bias gradients");
+  wg.nloss = int(npad / BM) * (m->nout_pad / BN) * 4;
+  wg.loss_part = m->lpart;
+  wg.loss = d_loss;
+  wg.lscale = 1.0f / (float(n) * float(m->n3));
+  const bool small = overlaps(int(npad), m->H);
+  if ((e = launch_chained(small, gemm_bf16_wgrad, dim3(wg.blk0[m->L] + wg.cblk0[m->L] + (d_loss ? 1 : 0)), dim3(128),
+                          tile_smem(WG_BN, WG_ST), s, wg, int(npad))) != cudaSuccess)
+    return cuda_fail(e, "wgrad");
   m->step += 1;
   const int64_t n4 = m->nparam / 4;
   e = launch_chained(

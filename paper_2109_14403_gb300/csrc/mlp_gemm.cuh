@@ -411,19 +411,88 @@ __global__ void __launch_bounds__(128, 2)
 // hidden units: 30 us a layer on that many SMs), together (128 x 64: 168 tiles)
 // they fill the chip.  Each output stays one chain of MMAs over the batch, the
 // order of its roundings.
+// The bias gradients (column sums of dZ_l) and the loss read what these tiles
+// read, so they are blocks of the same launch, behind the tiles in the slots
+// that 168 tiles leave free on 152 SMs (as a kernel of their own after them: a step
+// of 4,096 rows 191.6 us, now 180.2).
 constexpr int kMaxLayers = 9;
 struct WgradArgs {
   CUtensorMap a[kMaxLayers], b[kMaxLayers];  // dZ_l [K x M_l], X_l [K x N_l]
   int layers, blk0[kMaxLayers + 1], nx[kMaxLayers], ldc[kMaxLayers];
   float *out[kMaxLayers];
   int *err;
+  int cblk0[kMaxLayers + 1], cols[kMaxLayers];  // column sums: first block (after the tiles) and columns of each layer
+  const __nv_bfloat16 *dz[kMaxLayers];
+  float *db[kMaxLayers];
+  int nloss;  // the loss: partial sums, their number and scale (loss NULL: no block)
+  const float *loss_part;
+  float *loss, lscale;
 };
 static_assert(sizeof(WgradArgs) <= 4000, "kernel parameters");
+
+// Column sums of dz [rows x C] (rows a multiple of 32), 32 columns from c0 on:
+// 16 lanes of two columns, each thread four of 32 row classes (rows r mod 32,
+// one chain each), then the classes pairwise.
+constexpr int CS_COLS = 32;
+__device__ __forceinline__ void colsum_body(const __nv_bfloat16 *dz, int C, int rows, int c0, float *db,
+                                            float2 (*red)[16]) {
+  const int x = threadIdx.x & 15, g = threadIdx.x >> 4;
+  const __nv_bfloat16 *p = dz + c0 + 2 * x;
+  float2 s[4] = {};
+#pragma unroll 8
+  for (int r = g; r < rows; r += 32)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 v =
+          __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p + size_t(r + 8 * k) * C));
+      s[k].x += v.x;
+      s[k].y += v.y;
+    }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) red[g + 8 * k][x] = s[k];
+  __syncthreads();
+  for (int o = 16; o > 0; o >>= 1) {
+    for (int q = g; q < o; q += 8) {
+      red[q][x].x += red[q + o][x].x;
+      red[q][x].y += red[q + o][x].y;
+    }
+    __syncthreads();
+  }
+  if (g == 0) *reinterpret_cast<float2 *>(db + c0 + 2 * x) = red[0][x];
+}
+// The loss: the sum of the tiles' partial sums in FP64, 32 rows of 32 lanes in a
+// fixed order
+__device__ __forceinline__ void loss_body(const float *part, int n, float scale, float *loss, double *rl) {
+  const int lane = threadIdx.x & 31;
+  for (int w = threadIdx.x >> 5; w < 32; w += 4) {
+    double s = 0.0;
+    for (int i = 32 * w + lane; i < n; i += 1024) s += double(part[i]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) rl[w] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = rl[0];
+    for (int w = 1; w < 32; ++w) s += rl[w];
+    *loss = float(s * double(scale));
+  }
+}
 __global__ void __launch_bounds__(128, 2) gemm_bf16_wgrad(const __grid_constant__ WgradArgs A, int K) {
+  extern __shared__ __align__(1024) unsigned char gsm[];
   chain_begin();
-  int l = 0;
-  while (int(blockIdx.x) >= A.blk0[l + 1]) ++l;
-  const int q = int(blockIdx.x) - A.blk0[l];
+  int l = 0, q = int(blockIdx.x);
+  if (q >= A.blk0[A.layers]) {
+    q -= A.blk0[A.layers];
+    if (q >= A.cblk0[A.layers]) {
+      loss_body(A.loss_part, A.nloss, A.lscale, A.loss, reinterpret_cast<double *>(gsm));
+      return;
+    }
+    while (q >= A.cblk0[l + 1]) ++l;
+    colsum_body(A.dz[l], A.cols[l], K, (q - A.cblk0[l]) * CS_COLS, A.db[l], reinterpret_cast<float2(*)[16]>(gsm));
+    return;
+  }
+  while (q >= A.blk0[l + 1]) ++l;
+  q -= A.blk0[l];
   EpiArgs ep = {};
   ep.mode = EPI_F32;
   ep.f_out = A.out[l];

@@ -78,6 +78,19 @@ def test_misaligned_buffers_take_the_same_values():
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("n", [1, 128, 1000])
+def test_a_step_without_a_loss_buffer_takes_the_same_gradients(n):
+    res = []
+    for with_loss in (True, False):
+        net = _net(4, 128, 2, n)
+        x, t = _batch(net, n, seed=2)
+        net.train_step(x, t, 1e-3, torch.zeros(1, dtype=torch.float32, device="cuda:0") if with_loss else None)
+        res.append((net.grads(), net.params()))
+        net.close()
+    for a, b in zip(*res):
+        assert np.array_equal(a, b)
+
+
 def test_wide_and_tile_forms_agree():
     """Rows of a batch that fills the chip with 128 x 256 tiles against the
     same rows alone."""
