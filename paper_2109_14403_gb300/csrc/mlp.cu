@@ -60,6 +60,10 @@ cudaError_t gemm_setup() {
   e = cudaFuncSetAttribute(gemm_bf16_tile<false, false, BN, STAGES>, smem, GEMM_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tile<false, true, BN, STAGES>, smem, GEMM_SMEM);
   if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_bf16_tile<false, false, WG_BN, WG_ST>, smem, tile_smem(WG_BN, WG_ST));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(gemm_bf16_tile<false, true, WG_BN, WG_ST>, smem, tile_smem(WG_BN, WG_ST));
+  if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_bf16_wgrad, smem, tile_smem(WG_BN, WG_ST));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tn_wide, smem, WGEMM_SMEM);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_gemm_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -75,6 +79,15 @@ bool gemm_args_ok(const void *A, const void *B, int M, int N, int K) {
 // a product whose tiles are all resident at once is short: its launch overlaps
 // the one before it (pdl.cuh)
 bool overlaps(int M, int N) { return (M / BM) * (N / BN) <= 2 * g_gemm_sms; }
+
+// ... with at most one 128 x 128 tile an SM: tiles of 64 columns, up to two CTAs
+// an SM.  Such a product lasts as long as one tile, and half of the columns are
+// half of its epilogue (a step of 4,096 pairs 180 -> 172 us, of 64 142 -> 126;
+// inference of 64 to 4,096 rows 47..57 -> 42..52).  The hidden layers and their
+// input gradients; the same chain of MMAs for every output.
+bool narrow(int M, int N, const EpiArgs &ep) {
+  return (M / BM) * (N / BN) <= g_gemm_sms && (ep.mode == EPI_BIAS_SILU || ep.mode == EPI_DSILU);
+}
 
 // C = A . B^T with the fused epilogue ep; A [M x K], B [N x K] bf16; rows of A
 // from a_rows on read as zero.  N a multiple of 256 and a 128 x 256 tile for
@@ -96,6 +109,11 @@ cudaError_t gemm(cudaStream_t s, const void *A, const void *B, int M, int N, int
                                                                                               K, ep);
     return cudaGetLastError();
   }
+  if (narrow(M, N, ep)) {
+    if (!make_map(&mb, B, N, K, WG_BN)) return cudaErrorInvalidValue;
+    return launch_chained(true, gemm_bf16_tile<false, false, WG_BN, WG_ST>, dim3(N / WG_BN, M / BM), dim3(128),
+                          tile_smem(WG_BN, WG_ST), s, ma, mb, K, ep);
+  }
   if (!make_map(&mb, B, N, K)) return cudaErrorInvalidValue;
   return launch_chained(overlaps(M, N), gemm_bf16_tile<false, false, BN, STAGES>, dim3(N / BN, M / BM), dim3(128),
                         GEMM_SMEM, s, ma, mb, K, ep);
@@ -107,6 +125,9 @@ cudaError_t gemm_dgrad(cudaStream_t s, const void *A, const void *B, int M, int 
   if (e != cudaSuccess) return e;
   CUtensorMap ma, mb;
   if (!make_map(&ma, A, M, K) || !make_map(&mb, B, K, N, BK)) return cudaErrorInvalidValue;
+  if (narrow(M, N, ep))
+    return launch_chained(true, gemm_bf16_tile<false, true, WG_BN, WG_ST>, dim3(N / WG_BN, M / BM), dim3(128),
+                          tile_smem(WG_BN, WG_ST), s, ma, mb, K, ep);
   return launch_chained(overlaps(M, N), gemm_bf16_tile<false, true, BN, STAGES>, dim3(N / BN, M / BM), dim3(128),
                         GEMM_SMEM, s, ma, mb, K, ep);
 }

@@ -246,8 +246,9 @@ __device__ __forceinline__ uint64_t sdesc_mn_sw128(const void *tile) {
 // ([K x N]); the tensor core takes it that way, so that the backward pass
 // needs no transposed copies: dW = dZ^T . X with both operands as the batch's
 // rows, dX = dZ . W with W as stored.  BNT columns and NST stages: 128 and 3, or 64
-// and 4 for the weight gradients (gemm_bf16_wgrad), two CTAs per SM.
-constexpr int WG_BN = 64, WG_ST = 4;  // weight gradients
+// and 4 for short products and the weight gradients (gemm_bf16_wgrad), two CTAs
+// per SM.
+constexpr int WG_BN = 64, WG_ST = 4;  // the narrow tile
 __host__ __device__ constexpr int tile_smem(int bnt, int nst) { return nst * (TILE_A + bnt * BK * 2) + 1024 + 256; }
 static_assert(tile_smem(BN, STAGES) == GEMM_SMEM && 2 * (tile_smem(WG_BN, WG_ST) + 1024) <= 228 * 1024, "shared memory");
 template <bool AMN, bool BMN, int BNT, int NST>

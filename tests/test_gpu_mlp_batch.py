@@ -91,6 +91,17 @@ def test_a_step_without_a_loss_buffer_takes_the_same_gradients(n):
         assert np.array_equal(a, b)
 
 
+def test_narrow_and_square_tiles_agree():
+    """Hidden layers of two 128-column tiles: a row panel for every two SMs runs
+    64 columns a tile, one panel more 128."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 2
+    n = 128 * (sms // 2) + 1
+    net = _net(3, 256, 2, n)
+    x, _ = _batch(net, n, seed=4)
+    assert torch.equal(net.predict(x)[:n - 1], net.predict(x[:n - 1].contiguous()))
+    net.close()
+
+
 def test_wide_and_tile_forms_agree():
     """Rows of a batch that fills the chip with 128 x 256 tiles against the
     same rows alone."""
