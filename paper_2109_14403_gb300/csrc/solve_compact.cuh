@@ -1352,10 +1352,20 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
           sn += v * v;
         }
         TF res;
-        if constexpr (D64) {  // one square root: the other warps wait
-          const double f2 = res_floor * res_floor;
-          res = sqrt(s / ((double(N) * N) * (sn < f2 ? f2 : sn)));
-        } else {
+        bool two_roots = true;
+        if constexpr (D64) {
+          // One square root (the other warps wait), where numerator and
+          // denominator are far inside the range of a double, by their
+          // exponents: a floor below 1.5e-162 squares to zero, and a point
+          // without stress was 0/0.
+          const double f2 = res_floor * res_floor, d2 = (double(N) * N) * (sn < f2 ? f2 : sn);
+          const unsigned es = unsigned(__double2hiint(s)) >> 20, ed = unsigned(__double2hiint(d2)) >> 20;
+          if (es < 1423u && ed - 623u < 800u) {  // s < 2^400, 2^-400 <= d2 < 2^400
+            res = sqrt(s / d2);
+            two_roots = false;
+          }
+        }
+        if (two_roots) {
           TF den = sqrt(sn);
           if (den < res_floor) den = res_floor;
           res = sqrt(s) / (TF(N) * den);
