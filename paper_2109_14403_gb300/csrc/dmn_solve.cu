@@ -528,17 +528,21 @@ static cudaError_t prepare_kernel(KernelFn f, size_t smem, int threads, int *blo
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }
 
-// The smallest shared memory configuration that holds the resident CTAs (1 KB
-// per CTA for the system); the rest stays L1 for the node tables and spills.
+// The smallest shared memory configuration that holds `ctas` CTAs (each its
+// dynamic and at most 128 static bytes in units of 128, and 1 KB for the
+// system); the rest stays L1 for the node tables and spills.
+constexpr size_t cta_smem(size_t dyn) { return ((dyn + 128 + 127) & ~size_t(127)) + 1024; }
+constexpr int carveout_kb(size_t smem, int ctas) {
+  constexpr int kConfigKB[] = {8, 16, 32, 64, 100, 132, 164, 196};
+  for (int kb : kConfigKB)
+    if (size_t(kb) * 1024 >= size_t(ctas) * cta_smem(smem)) return kb;
+  return 228;
+}
+static_assert(carveout_kb(9888, 3) == 64 && carveout_kb(65456, 3) == 196 && carveout_kb(71600, 3) == 228,
+              "CTAs of 9,904 bytes take 11,008 each: 32 KB hold two, not three");
 // The driver rounds a requested percentage up to the next configuration, so
 // request the largest percentage below the chosen one.
-static int carveout_pct(size_t smem, int ctas) {
-  static const int kConfigKB[] = {8, 16, 32, 64, 100, 132, 164, 196};
-  const size_t need = size_t(ctas) * (smem + 1024);
-  for (int kb : kConfigKB)
-    if (size_t(kb) * 1024 >= need) return kb * 100 / 228;
-  return 100;
-}
+static int carveout_pct(size_t smem, int ctas) { return carveout_kb(smem, ctas) * 100 / 228; }
 
 cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
                           int *blocks_per_sm) {
@@ -558,10 +562,15 @@ cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid
   const size_t smem = solve_smem_bytes(P.K, P.zw, P.n_mats, mixed, variant, P.law);
   const cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  const int per_sm = (grid + num_sms - 1) / num_sms;
+  // room for every CTA the SM could hold, not only for this launch's: with less,
+  // evaluations on other streams waited for each other's SMs (eight streams of 150
+  // points, K = 6: FP64 1252 us became 2856 with the launch's own CTAs alone and is
+  // 965 now; mixed 354, 667, 341; K = 8 mixed 597, 928, 626).  One launch alone on
+  // the chip gains little from the larger L1 (K = 9 mixed J2 up to 152 points -13 %,
+  // 16 Perzyna points at K = 8 -6 %, others 0 to 1 %).
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-  at[0].val.sharedMemCarveout = unsigned(carveout_pct(smem, per_sm < blocks_per_sm ? per_sm : blocks_per_sm));
+  at[0].val.sharedMemCarveout = unsigned(carveout_pct(smem, blocks_per_sm));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(grid));
   cfg.blockDim = dim3(unsigned(solve_block_threads(P.K, mixed, variant, P.law)));
