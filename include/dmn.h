@@ -151,8 +151,9 @@ typedef struct {
                            compact kernel (upper tree levels on one warp,
                            strains updated by the Newton step), as 12; 12, 13,
                            14 = compact kernel for 2, 3 or 4 CTAs per SM.
-                           Launches of at most two CTAs per SM run the
-                           instance for two.  22, 23, 24 =
+                           Launches of at most two CTAs per SM that fill
+                           half of the SMs' room at most run the instance
+                           for two.  22, 23, 24 =
                            one warp per Gauss point (lane l condenses the
                            subtree under level-6 node l in registers, levels
                            5..1 by shuffles; four points per CTA, register

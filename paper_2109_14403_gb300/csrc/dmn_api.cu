@@ -18,7 +18,7 @@ struct dmn_handle_s {
   int K, N, nleaf, SW, zend, n_mats;
   dmn_options opt;
   int device, num_sms;
-  int blocks_per_sm;     // resident CTAs per SM of the selected kernel variant
+  Residency res;         // resident CTAs per SM of the selected kernel variant
   unsigned long long *d_queue;  // work-queue counter (one per handle)
   unsigned long long *d_open;   // dmn_eval_mixed: points still iterating
   double *d_node;        // [N][kNodeWords]
@@ -318,11 +318,11 @@ extern "C" dmn_status dmn_create(dmn_handle *out, int32_t K, const double *leaf_
       free_handle(h);
       return fail(DMN_ERR_ARG, "dmn_create: K=%d does not fit one SM in the requested precision", K);
     }
-    if ((e = prepare_solve(K, zw, n_mats, mixed, o.solve_variant, law, &h->blocks_per_sm)) != cudaSuccess) {
+    if ((e = prepare_solve(K, zw, n_mats, mixed, o.solve_variant, law, &h->res)) != cudaSuccess) {
       free_handle(h);
       return cuda_fail(e, "prepare_solve");
     }
-    if (h->blocks_per_sm < 1) {
+    if (h->res.ctas < 1) {
       free_handle(h);
       return fail(DMN_ERR_ARG, "dmn_create: K=%d does not fit one SM in the requested precision", K);
     }
@@ -338,7 +338,7 @@ extern "C" dmn_status dmn_create(dmn_handle *out, int32_t K, const double *leaf_
       (e = cudaMalloc(&h->d_open, sizeof(unsigned long long))) != cudaSuccess ||
       (is_warp_variant(o.solve_variant) &&
        (e = cudaMalloc(&h->d_gh, warp_scratch_bytes_per_cta(K) * size_t(h->num_sms) *
-                                     size_t(h->blocks_per_sm))) != cudaSuccess)) {
+                                     size_t(h->res.ctas))) != cudaSuccess)) {
     free_handle(h);
     return cuda_fail(e, "cudaMalloc");
   }
@@ -446,10 +446,10 @@ static dmn_status eval_impl(dmn_handle h, dmn_stream stream, int64_t n_points,
   P.da0 = d_da;
   P.skip = d_skip;
   P.gh = h->d_gh;
-  int64_t grid = (int64_t)h->num_sms * h->blocks_per_sm;  // the scratch holds this many CTAs
+  int64_t grid = (int64_t)h->num_sms * h->res.ctas;  // the scratch holds this many CTAs
   const int64_t per_cta = is_warp_variant(h->opt.solve_variant) ? warp_form_warps() : 1;
   if (grid > (n_points + per_cta - 1) / per_cta) grid = (n_points + per_cta - 1) / per_cta;
-  cudaError_t e = launch_solve(P, mixed, h->opt.solve_variant, (int)grid, h->num_sms, h->blocks_per_sm,
+  cudaError_t e = launch_solve(P, mixed, h->opt.solve_variant, (int)grid, h->num_sms, h->res,
                                (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "dmn_eval launch");
   return DMN_OK;

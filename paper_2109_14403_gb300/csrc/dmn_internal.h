@@ -57,9 +57,13 @@ KernelFn warp_kernel8(int minb);
 // threads per CTA of the kernel a variant selects
 int solve_block_threads(int K, bool mixed, int variant, int law);
 int compact_block_threads64(int K);  // ... of the compact kernel's FP64 instances
-cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
-                          int *blocks_per_sm);
-cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, int blocks_per_sm,
+// resident CTAs per SM of the kernel a variant selects, and of its instance for
+// small launches (0: there is none)
+struct Residency {
+  int ctas, few;
+};
+cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law, Residency *res);
+cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, Residency res,
                          cudaStream_t s);
 // dmn_eval_mixed (dmn_drive.cu): prescribed strain components, outer = 0 and
 // optionally the tangent predictor; one outer Newton update after an

@@ -146,14 +146,15 @@ extern "C" dmn_status dmn_eval_noalloc(int32_t K, const double *leaf_w, const do
   }
   unsigned char *base = static_cast<unsigned char *>(addr);
   const bool mixed = o.precision == DMN_PREC_MIXED;
-  int num_sms = 0, smem_optin = 0, blocks_per_sm = 0;
+  int num_sms = 0, smem_optin = 0;
+  Residency res = {};
   cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (solve_smem_bytes(K, zw, n_mats, mixed, o.solve_variant, law) > (size_t)smem_optin)
     return na_fail(DMN_ERR_ARG, "dmn_eval_noalloc: K=%d does not fit one SM in this precision", K);
-  e = prepare_solve(K, zw, n_mats, mixed, o.solve_variant, law, &blocks_per_sm);
+  e = prepare_solve(K, zw, n_mats, mixed, o.solve_variant, law, &res);
   if (e != cudaSuccess) return na_fail(DMN_ERR_CUDA, "prepare_solve: %s", cudaGetErrorString(e));
-  if (blocks_per_sm < 1) return na_fail(DMN_ERR_ARG, "dmn_eval_noalloc: kernel does not fit one SM");
+  if (res.ctas < 1) return na_fail(DMN_ERR_ARG, "dmn_eval_noalloc: kernel does not fit one SM");
 
   // ---- upload the tables (stream-ordered copies from the call-local
   //      arrays above, which are pageable memory: the copy is staged before
@@ -205,9 +206,9 @@ extern "C" dmn_status dmn_eval_noalloc(int32_t K, const double *leaf_w, const do
   P.out = d_out;
   P.status = d_status;
   P.iters = d_iters;
-  int64_t grid = (int64_t)num_sms * blocks_per_sm;
+  int64_t grid = (int64_t)num_sms * res.ctas;
   if (grid > n_points) grid = n_points;
-  e = launch_solve(P, mixed, o.solve_variant, (int)grid, num_sms, blocks_per_sm, s);
+  e = launch_solve(P, mixed, o.solve_variant, (int)grid, num_sms, res, s);
   if (e != cudaSuccess) return na_fail(DMN_ERR_CUDA, "dmn_eval_noalloc launch: %s", cudaGetErrorString(e));
   return DMN_OK;
 }

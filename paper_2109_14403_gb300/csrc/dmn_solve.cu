@@ -467,10 +467,14 @@ static size_t owner_smem_bytes(int K, int zw, int n_mats, bool mixed) {
 // Perzyna leaves (law 2) always takes the compact instances that include that
 // leaf law (dmn_solve_compact_vp.cu, K <= 9), whatever the variant; one with
 // PA66 leaves (law 3) the instances of dmn_solve_compact_pa66.cu (K <= 8).
-// A mixed launch of at most two CTAs per SM (`few`) takes its form's instance
-// for two: the same operations with more registers (compact 232 against 168,
-// no spills), where the smaller budget gains no residency (27 points at K = 8
-// 66.2 -> 63.6 us, 32 at K = 3 62.5 -> 59.4).
+// A mixed launch of at most two CTAs per SM that fills at most half of what the
+// SMs hold of it (`few`) takes its form's instance for two: the same operations
+// with more registers (compact 254 against 168 with 80 bytes of spills, owner 245
+// against 168 with 192), where the smaller budget gains no residency (27 points at
+// K = 8 66.2 -> 63.6 us, 32 at K = 3 62.5 -> 59.4; up to 304 points at K = 3..5 4 to
+// 7 %).  Half, so that another stream's launch still fits: at K = 8, two of these CTAs
+// an SM for three, launches of 300 points on three to eight streams took 3 to 8 %
+// longer than on the other instance, which costs one launch alone 2 %.
 bool is_warp_variant(int variant) { return variant >= 22 && variant <= 24; }
 bool solve_variant_valid(int variant) {
   return variant == 0 || (variant >= 2 && variant <= 4) || (variant >= 11 && variant <= 14) ||
@@ -544,20 +548,19 @@ static_assert(carveout_kb(9888, 3) == 64 && carveout_kb(65456, 3) == 196 && carv
 // request the largest percentage below the chosen one.
 static int carveout_pct(size_t smem, int ctas) { return carveout_kb(smem, ctas) * 100 / 228; }
 
-cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law,
-                          int *blocks_per_sm) {
+cudaError_t prepare_solve(int K, int zw, int n_mats, bool mixed, int variant, int law, Residency *res) {
   const size_t smem = solve_smem_bytes(K, zw, n_mats, mixed, variant, law);
   const int threads = solve_block_threads(K, mixed, variant, law);
   const KernelFn f = pick(K, mixed, variant, law, false), g = pick(K, mixed, variant, law, true);
-  if (g != f) {  // the instance of small launches
-    int b = 0;
-    const cudaError_t e = prepare_kernel(g, smem, threads, &b);
+  res->few = 0;
+  if (g != f) {
+    const cudaError_t e = prepare_kernel(g, smem, threads, &res->few);
     if (e != cudaSuccess) return e;
   }
-  return prepare_kernel(f, smem, threads, blocks_per_sm);
+  return prepare_kernel(f, smem, threads, &res->ctas);
 }
 
-cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, int blocks_per_sm,
+cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid, int num_sms, Residency res,
                          cudaStream_t s) {
   const size_t smem = solve_smem_bytes(P.K, P.zw, P.n_mats, mixed, variant, P.law);
   const cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned long long), s);
@@ -570,7 +573,7 @@ cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid
   // 16 Perzyna points at K = 8 -6 %, others 0 to 1 %).
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-  at[0].val.sharedMemCarveout = unsigned(carveout_pct(smem, blocks_per_sm));
+  at[0].val.sharedMemCarveout = unsigned(carveout_pct(smem, res.ctas));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(grid));
   cfg.blockDim = dim3(unsigned(solve_block_threads(P.K, mixed, variant, P.law)));
@@ -578,7 +581,8 @@ cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, pick(P.K, mixed, variant, P.law, grid <= 2 * num_sms), P);
+  const bool few = grid <= 2 * num_sms && 2 * grid <= res.few * num_sms;
+  return cudaLaunchKernelEx(&cfg, pick(P.K, mixed, variant, P.law, few), P);
 }
 
 // the index-check log of this translation unit (debug build; dmn_check.cuh)

@@ -52,3 +52,24 @@ def test_eight_fp64_evaluations_of_a_point_an_sm_overlap():
         pytest.skip("no CUDA device")
     n = torch.cuda.get_device_properties(0).multi_processor_count - 2
     assert _graph_us(8, 6, n, "fp64") < 3.0 * _graph_us(1, 6, n, "fp64")
+
+
+@pytest.mark.parametrize("K,variant", [(5, 0), (7, 13), (8, 13)])
+def test_instances_on_either_side_of_the_small_launch_rule_agree(K, variant):
+    """The instance with the larger register budget serves launches that fill at
+    most half of what the SMs hold of it (K = 8: one CTA an SM): the same points
+    with the same bits in launches on either side of one and of two an SM."""
+    from paper_2109_14403_gb300 import DMN
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    dev, sms = torch.device("cuda:0"), torch.cuda.get_device_properties(0).multi_processor_count
+    d = DMN(K, *syn.tree(K), syn.materials(), tol=1e-12, precision="mixed", solve_variant=variant)
+    deps, theta = syn.random_walk_k8(n_points=2 * sms + 1, n_incr=1)
+    ref = None
+    for n in (2 * sms + 1, 2 * sms, sms + 1, sms):
+        s = d.init_state(torch.full((n,), syn.THETA_START, dtype=torch.float64, device=dev))
+        s, out, st, it = d.eval(torch.tensor(8.0 * deps[0, :n], device=dev), torch.tensor(theta[0, :n], device=dev),
+                                0.7, s)
+        ref = ref or (s, out, it)
+        assert torch.equal(s, ref[0][:n]) and torch.equal(out, ref[1][:n]) and torch.equal(it, ref[2][:n])
+    d.close()
