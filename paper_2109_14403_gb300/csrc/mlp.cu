@@ -65,7 +65,8 @@ cudaError_t gemm_setup() {
     e = cudaFuncSetAttribute(gemm_bf16_tile<false, true, WG_BN, WG_ST>, smem, tile_smem(WG_BN, WG_ST));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(gemm_bf16_wgrad, smem, tile_smem(WG_BN, WG_ST));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tn_wide, smem, WGEMM_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tn_wide<false>, smem, wide_smem(false));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_bf16_tn_wide<true>, smem, wide_smem(true));
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_gemm_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) g_gemm_configured_dev = dev;
   return e;
@@ -90,23 +91,29 @@ bool narrow(int M, int N, const EpiArgs &ep) {
 }
 
 // C = A . B^T with the fused epilogue ep; A [M x K], B [N x K] bf16; rows of A
-// from a_rows on read as zero.  N a multiple of 256 and a 128 x 256 tile for
-// every SM: the persistent wide form (one CTA per SM), else (and with z_out or
-// the loss, the training step's) the tile form, whose 128 x 128 tiles spread a
-// product over twice the SMs (4,096 rows, a hidden layer: 18 -> 12 us).
+// from a_rows on read as zero.  N a multiple of 256 and enough 128 x 256 tiles: the
+// persistent wide form (one CTA per SM), else (and with z_out or the loss, the
+// training step's) the tile form, whose 128 x 128 tiles spread a product over
+// twice the SMs (4,096 rows, a hidden layer: 18 -> 12 us).  Enough is a tile for
+// every SM, or for plain FP32 output for more than half of them: with fewer the tile
+// form has an SM for every half tile (64 tiles, K = 512 to 4,096: 0.85 to 0.9 of the
+// wide form's time; 128 tiles, K = 4,096: 1.10).
 cudaError_t gemm(cudaStream_t s, const void *A, const void *B, int M, int N, int K, EpiArgs ep, int64_t a_rows) {
   if (!gemm_args_ok(A, B, M, N, K)) return cudaErrorInvalidValue;
   cudaError_t e = gemm_setup();
   if (e != cudaSuccess) return e;
   CUtensorMap ma, mb;
   if (!make_map(&ma, A, a_rows, K)) return cudaErrorInvalidValue;
-  if (N % WBN == 0 && (M / BM) * (N / WBN) >= g_gemm_sms && !ep.z_out && ep.mode != EPI_LOSS) {
+  const bool plain = ep.mode == EPI_F32;
+  const int64_t tiles = int64_t(M / BM) * (N / WBN);
+  if (N % WBN == 0 && tiles * (plain ? 2 : 1) >= g_gemm_sms + (plain ? 1 : 0) && !ep.z_out && ep.mode != EPI_LOSS) {
     CUtensorMap mh = ma;  // unused unless the activation leaves by TMA
     if (!make_map(&mb, B, N, K, WBN) || (ep.mode == EPI_BIAS_SILU && !make_map(&mh, ep.h_out, M, N, 32)))
       return cudaErrorInvalidValue;
-    const int tiles = (M / BM) * (N / WBN);
-    gemm_bf16_tn_wide<<<tiles < g_gemm_sms ? tiles : g_gemm_sms, 64 + 32 * WEPI, WGEMM_SMEM, s>>>(ma, mb, mh, M, N,
-                                                                                              K, ep);
+    const int ctas = int(tiles < g_gemm_sms ? tiles : g_gemm_sms);
+    const bool lng = plain || K >= 2048;
+    (lng ? gemm_bf16_tn_wide<true> : gemm_bf16_tn_wide<false>)<<<ctas, wide_threads(lng), wide_smem(lng), s>>>(
+        ma, mb, mh, M, N, K, ep);
     return cudaGetLastError();
   }
   if (narrow(M, N, ep)) {

@@ -530,12 +530,26 @@ __global__ void __launch_bounds__(128, 2) gemm_bf16_wgrad(const __grid_constant_
 // FP32 prediction (rows of an odd length: no TMA) is staged as 32 rows x 32
 // columns and written a row at a time, the lanes on consecutive columns.  Every
 // wait is bounded as in the form above.
-constexpr int WBN = 256, WST = 3, WEPI = 16;  // stages, epilogue warps
+// LONG, for long reductions (K >= 2048: a tile's MMAs take four times its
+// epilogue) and plain FP32 output: the staging's memory is a fourth stage instead,
+// and eight warps of 128 columns store directly (the prediction through 32 x 17
+// floats a warp, two rows at a time).  8,192^3: 876 -> 772 us; inference of 65,536
+// rows with 4,096 hidden units 3,449 -> 3,285 (1,024 units, which stay: 470, 460 this
+// way; 16,384 rows of them 157, 166).  FP32 rows leave as whole 32-byte sectors: half
+// a sector an instruction, merged or not as the warps happen to run, took 217 to
+// 247 us at 65,536 x 2,048 x 512; now 190.
+constexpr int WBN = 256;
 constexpr int WTILE_B = WBN * BK * 2;
 constexpr int WSTAGE = TILE_A + WTILE_B;  // 48 KB, a multiple of 1024
-constexpr int WSTAGE_EPI = WEPI * 4096;   // staging: per warp 32 rows of 128 bytes
-constexpr int WGEMM_SMEM = WST * WSTAGE + WSTAGE_EPI + 1024 + 256;
-static_assert(WGEMM_SMEM <= 232448, "opt-in shared memory per CTA");
+__host__ __device__ constexpr int wide_stages(bool lng) { return lng ? 4 : 3; }
+__host__ __device__ constexpr int wide_epi(bool lng) { return lng ? 8 : 16; }  // epilogue warps
+__host__ __device__ constexpr int wide_threads(bool lng) { return 64 + 32 * wide_epi(lng); }
+// staging per epilogue warp: 32 rows of 128 bytes, or of 17 floats
+__host__ __device__ constexpr int wide_stage_epi(bool lng) { return wide_epi(lng) * (lng ? 32 * 17 * 4 : 4096); }
+__host__ __device__ constexpr int wide_smem(bool lng) {
+  return wide_stages(lng) * WSTAGE + wide_stage_epi(lng) + 1024 + 256;
+}
+static_assert(wide_smem(false) <= 232448 && wide_smem(true) <= 232448, "opt-in shared memory per CTA");
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -572,16 +586,26 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void 
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+// eight floats to a 32-byte boundary: one whole sector a lane
+__device__ __forceinline__ void st_sector(float *p, const float v[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+
 // Modes EPI_BIAS_SILU without z_out (map_h: its bf16 output, [M x N], boxes of
-// 32 rows x 64 columns; unused in the others), EPI_BIAS_F32, EPI_F32.
-__global__ void __launch_bounds__(64 + 32 * WEPI, 1)
+// 32 rows x 64 columns; unused in the others) and EPI_BIAS_F32; LONG: the same and
+// EPI_F32, map_h unused.
+template <bool LONG>
+__global__ void __launch_bounds__(wide_threads(LONG), 1)
     gemm_bf16_tn_wide(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                       const __grid_constant__ CUtensorMap map_h, int M, int N, int K, const EpiArgs ep) {
   extern __shared__ __align__(1024) unsigned char gsm[];
   unsigned char *base = reinterpret_cast<unsigned char *>(
       (reinterpret_cast<uintptr_t>(gsm) + 1023) & ~uintptr_t(1023));
+  constexpr int WST = wide_stages(LONG), WEPI = wide_epi(LONG);
   unsigned char *stage_epi = base + WST * WSTAGE;
-  uint64_t *full = reinterpret_cast<uint64_t *>(base + WST * WSTAGE + WSTAGE_EPI);
+  uint64_t *full = reinterpret_cast<uint64_t *>(stage_epi + wide_stage_epi(LONG));
   uint64_t *empty = full + WST;
   uint64_t *accf = empty + WST;  // 2: accumulator full (MMA -> epilogue)
   uint64_t *acce = accf + 2;     // 2: accumulator empty (epilogue -> MMA)
@@ -664,14 +688,68 @@ __global__ void __launch_bounds__(64 + 32 * WEPI, 1)
         umma_commit(&accf[b]);  // arrives once this tile's MMAs have completed
       }
     }
-  } else {  // ---- epilogue: warps 2..17 ----
+  } else if constexpr (LONG) {  // ---- epilogue: warps 2..9 ----
     const int qd = warp & 3;  // TMEM lane quarter = tile rows 32 qd ..
     constexpr int CW = WBN / (WEPI / 4);  // this warp's columns ch0 .. ch0 + CW - 1
+    const int ch0 = ((warp - 2) >> 2) * CW;
+    float *stg = reinterpret_cast<float *>(stage_epi) + (warp - 2) * 32 * 17;
+    const bool row32 = !(reinterpret_cast<uintptr_t>(ep.f_out) & 31);
+    int j = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++j) {
+      const int b = j & 1;
+      const bool ok = mbar_wait(&accf[b], (j >> 1) & 1);
+      if (!__all_sync(0xffffffffu, ok) || *(volatile int *)fail) {
+        if (lane == 0) atomicExch(fail, 1);
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int m0 = (t / ntn) * BM + qd * 32, n0 = (t % ntn) * WBN;
+      const uint32_t trow = tmem + (uint32_t(qd * 32) << 16) + uint32_t(b * WBN);
+      if (ep.mode == EPI_F32 && row32) {
+        float *fo = ep.f_out + size_t(m0 + lane) * ep.ldc + n0 + ch0;
+#pragma unroll
+        for (int h = 0; h < CW; h += 16) {
+          float v[16];
+          tmem_ld16(trow + ch0 + h, v);
+#pragma unroll
+          for (int q = 0; q < 2; ++q) st_sector(fo + h + 8 * q, v + 8 * q);
+        }
+      } else if (ep.mode == EPI_BIAS_F32) {
+        for (int c0 = ch0; c0 < ch0 + CW; c0 += 16) {
+          float v[16];
+          tmem_ld16(trow + c0, v);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) stg[lane * 17 + i] = v[i];
+          __syncwarp();
+          // lanes 0..15 on row rr, 16..31 on row rr + 1, consecutive columns
+          const int cl = lane & 15, n = n0 + c0 + cl;
+          const bool cv = n < ep.n_valid;
+          const float bb = cv ? ep.bias[n] : 0.0f, sc = cv ? ep.scale[n] : 0.0f, sh = cv ? ep.shift[n] : 0.0f;
+          for (int rr = lane >> 4; rr < 32; rr += 2)
+            if (cv && m0 + rr < ep.m_valid)
+              ep.f_out[size_t(m0 + rr) * ep.ld_f + n] = (stg[rr * 17 + cl] + bb) * sc + sh;
+          __syncwarp();
+        }
+      } else {
+        for (int c0 = ch0; c0 < ch0 + CW; c0 += 32) {
+          float v[32];
+          tmem_ld32(trow + c0, v);
+          epi_chunk16(ep, m0 + lane, n0 + c0, v);
+          epi_chunk16(ep, m0 + lane, n0 + c0 + 16, v + 16);
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acce[b]);
+    }
+  } else {  // ---- epilogue: warps 2..17 ----
+    const int qd = warp & 3;
+    constexpr int CW = WBN / (WEPI / 4);
     static_assert(CW == 64, "two 32-column chunks, one 128-byte row of bf16");
     const int ch0 = ((warp - 2) >> 2) * CW;
     unsigned char *stg = stage_epi + (warp - 2) * 4096;
     float *stf = reinterpret_cast<float *>(stg);
-    const bool pred = ep.mode == EPI_BIAS_F32, act = ep.mode == EPI_BIAS_SILU;
+    const bool act = ep.mode == EPI_BIAS_SILU;  // else EPI_BIAS_F32
     int j = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++j) {
       const int b = j & 1;
@@ -719,7 +797,7 @@ __global__ void __launch_bounds__(64 + 32 * WEPI, 1)
             *reinterpret_cast<uint4 *>(stg + lane * 128 + (((4 * h + q) ^ (lane & 7)) << 4)) =
                 *reinterpret_cast<uint4 *>(hb);
           }
-        } else if (pred) {
+        } else {
           // de-normalised prediction on valid rows and columns; column c of row
           // r in slot c ^ r of the row
           __syncwarp();
@@ -737,9 +815,6 @@ __global__ void __launch_bounds__(64 + 32 * WEPI, 1)
           } else if (cv) {
             for (int rr = 0; rr < rows; ++rr) dst[size_t(rr) * ep.ld_f] = (stf[rr * 32 + (lane ^ rr)] + bb) * sc + sh;
           }
-        } else {
-          epi_chunk16(ep, m0 + lane, n, v);
-          epi_chunk16(ep, m0 + lane, n + 16, v + 16);
         }
       }
       if (act) {
