@@ -2,6 +2,7 @@
 // for one Gauss point per CTA.  See dmn_kernels.cuh for the mapping and the
 // condensation.
 #include "dmn_internal.h"
+#include "pdl.cuh"
 #include "solve_common.cuh"
 
 namespace dmn {
@@ -564,7 +565,7 @@ cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid
                          cudaStream_t s) {
   const size_t smem = solve_smem_bytes(P.K, P.zw, P.n_mats, mixed, variant, P.law);
   const cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess) return launch_status(e);
   // room for every CTA the SM could hold, not only for this launch's: with less,
   // evaluations on other streams waited for each other's SMs (eight streams of 150
   // points, K = 6: FP64 1252 us became 2856 with the launch's own CTAs alone and is
@@ -582,7 +583,7 @@ cudaError_t launch_solve(const SolveParams &P, bool mixed, int variant, int grid
   cfg.attrs = at;
   cfg.numAttrs = 1;
   const bool few = grid <= 2 * num_sms && 2 * grid <= res.few * num_sms;
-  return cudaLaunchKernelEx(&cfg, pick(P.K, mixed, variant, P.law, few), P);
+  return launch_status(cudaLaunchKernelEx(&cfg, pick(P.K, mixed, variant, P.law, few), P));
 }
 
 // the index-check log of this translation unit (debug build; dmn_check.cuh)

@@ -20,6 +20,14 @@ __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// The result of a launch; a failed one is taken off the thread's error state too,
+// as cudaGetLastError after <<<>>> does: it has been reported, and left there it
+// would be found by the next launch check, the caller's own included.
+inline cudaError_t launch_status(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // overlap = false: an ordinary launch of such a kernel
 template <typename... P, typename... A>
 cudaError_t launch_chained(bool overlap, void (*f)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
@@ -34,7 +42,7 @@ cudaError_t launch_chained(bool overlap, void (*f)(P...), dim3 grid, dim3 block,
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, f, P(std::forward<A>(args))...);
+  return launch_status(cudaLaunchKernelEx(&cfg, f, P(std::forward<A>(args))...));
 }
 
 }  // namespace dmn
