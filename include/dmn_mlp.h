@@ -116,8 +116,8 @@ dmn_status dmn_mlp_get_normalization(dmn_mlp m, float *h_fmean, float *h_finv, f
                                      float *h_tstd);
 
 /* Building block: C = A B^T with A bf16 [M x K], B bf16 [N x K] (K
-   contiguous), C fp32 [M x N]; M, N multiples of 128, K of 64.  Runs the
-   tcgen05 GEMM the network uses. */
+   contiguous), C fp32 [M x N]; M, N multiples of 128, K of 64; the buffers
+   16-byte aligned.  Runs the tcgen05 GEMM the network uses. */
 dmn_status dmn_gemm_bf16_tn(dmn_stream stream, int32_t M, int32_t N, int32_t K, const void *d_a,
                             const void *d_b, float *d_c);
 

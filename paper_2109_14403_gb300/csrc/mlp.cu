@@ -852,6 +852,8 @@ extern "C" dmn_status dmn_gemm_bf16_tn(dmn_stream stream, int32_t M, int32_t N, 
   set_error_message("");
   if (!d_a || !d_b || !d_c || M <= 0 || N <= 0 || K <= 0 || M % 128 || N % 128 || K % 64)
     return fail(DMN_ERR_ARG, "dmn_gemm_bf16_tn: M, N must be multiples of 128 and K of 64");
+  if (reinterpret_cast<uintptr_t>(d_c) & 15)  // rows leave as 16- or 32-byte stores
+    return fail(DMN_ERR_ARG, "dmn_gemm_bf16_tn: d_c must be 16-byte aligned");
   EpiArgs ep;
   memset(&ep, 0, sizeof(ep));
   ep.mode = EPI_F32;
