@@ -17,8 +17,9 @@ uniaxial ramp that drives the matrix into plastic flow ("plastic") and the
 lognormal increment magnitudes of the uneven batch ("uneven").  Variant
 numbers are those of ``dmn_options.solve_variant``: 2, 3, 4 owner-mapped
 mixed; 12, 13, 14 compact mixed; 22, 23, 24 warp form (mixed, K = 6..8).
-FP64 has one form, the compact one (11, and 0).  A variant the library rejects for a
-configuration is left out of that run.
+FP64 has one form, the compact one (11; 0 selects it too), so its entries only
+record a time.  A variant the library rejects for a configuration is left out
+of that run.
 
 Usage (on a GPU):  python -m paper_2109_14403_gb300.autotune [--K 8] [--points 65536]
                    [--workload random_walk|plastic|uneven]
@@ -30,7 +31,7 @@ import json
 import os
 
 TABLE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "tuning.json")
-VARIANTS = {"mixed": (2, 3, 4, 12, 13, 14, 22, 23, 24), "fp64": (0, 11)}
+VARIANTS = {"mixed": (2, 3, 4, 12, 13, 14, 22, 23, 24), "fp64": (11,)}  # one number a kernel
 WORKLOADS = ("random_walk", "plastic", "uneven")
 # the mapping each variant selects (points per CTA, warps per point at K = 8)
 MAPPING = {0: "owner-mapped, 1 point per CTA", 2: "owner-mapped, 1 point per CTA",
@@ -40,6 +41,11 @@ MAPPING = {0: "owner-mapped, 1 point per CTA", 2: "owner-mapped, 1 point per CTA
            22: "warp form, 4 points per CTA, 1 warp per point",
            23: "warp form, 4 points per CTA, 1 warp per point",
            24: "warp form, 4 points per CTA, 1 warp per point"}
+
+
+def mapping(variant: int, precision: str) -> str:
+    """The mapping a variant selects; FP64 runs the compact form whatever it is."""
+    return MAPPING[11] if precision == "fp64" else MAPPING.get(variant, "")
 
 
 def key(K: int, precision: str, workload: str = "random_walk") -> str:
@@ -123,7 +129,7 @@ def tune(K: int = 8, n_points: int = 65536, n_steps: int = 4, warmup: int = 2,
         d.close()
     best = choose(times)
     table = load_table(path)
-    table[key(K, precision, workload)] = {"variant": best, "mapping": MAPPING.get(best, ""),
+    table[key(K, precision, workload)] = {"variant": best, "mapping": mapping(best, precision),
                                           "ms_per_step": times, "points": n_points,
                                           "workload": workload}
     with open(path, "w") as f:

@@ -75,3 +75,15 @@ def test_warp_variants_rejected_for_unsupported_trees():
         rc = L.dmn_create(ctypes.byref(h), K, w.ctypes.data_as(P), n.ctypes.data_as(P),
                           ph.ctypes.data_as(P), ctypes.cast(mats, P), 2, ctypes.byref(o))
         assert rc == dmn.DMN_ERR_ARG and b"one warp per point" in L.dmn_last_error()
+
+
+def test_fp64_has_one_kernel_to_time():
+    """FP64 runs the compact form whatever the variant, so the tuner has one
+    number for it, and the table's entries hold no other kernel's time."""
+    assert autotune.VARIANTS["fp64"] == (11,)
+    assert autotune.mapping(0, "fp64") == autotune.mapping(11, "fp64") == autotune.MAPPING[11]
+    assert autotune.mapping(0, "mixed") != autotune.mapping(13, "mixed")
+    for k, e in autotune.load_table().items():
+        if ",fp64" in k:
+            assert set(e["ms_per_step"]) == {"11"} and e["variant"] == 11, k
+            assert e["mapping"] == autotune.MAPPING[11]
