@@ -346,21 +346,24 @@ __device__ __forceinline__ double root_p(double x, double p) {
   return MODE == 1 ? x : (MODE == 2 ? sqrt(x) : pow(x, 1.0 / p));
 }
 
-// x^q for x >= 0; a small whole q by repeated squaring (within a few ulp).
-// One FP64 pow() is a serial chain of some 8 us here, and a 32-sample step had
-// six of them in a row.
+// x^q for x >= 0; a whole q up to 16 by repeated squaring: the relative error
+// of x^k is at most (k - 1) 2^-53 however the products are paired (seen: 11 2^-53 at
+// q = 16; 45 at 64, so larger q take pow()).  One FP64 pow() is a serial chain of some 8 us here,
+// and a 32-sample step had six of them in a row.
+constexpr double kSquaringMaxQ = 16.0;
 __device__ __forceinline__ double pow_q(double x, double q) {
-  if (!(q >= 0.0 && q <= 64.0) || q != floor(q)) return pow(x, q);
+  if (!(q >= 0.0 && q <= kSquaringMaxQ) || q != floor(q)) return pow(x, q);
   double r = 1.0;
   for (int k = int(q); k; k >>= 1, x *= x)
     if (k & 1) r *= x;
   return r;
 }
 
-// S^(1/q): a small whole q from the FP32 root by two Newton steps (relative
-// error 1e-6 -> 5e-12 -> rounding), a fifth of the FP64 pow()'s chain
+// S^(1/q): a whole q up to 16 from the FP32 root by two Newton steps (a relative
+// error e becomes (q - 1) / 2 e^2: 1e-6 -> 7.5e-12 at most -> rounding, 1/q of pow_q's
+// error among it), a fifth of the FP64 pow()'s chain
 __device__ __forceinline__ double root_q(double S, double q) {
-  if (!(q >= 1.0 && q <= 64.0) || q != floor(q) || !(S > 1e-30 && S < 1e30)) return pow(S, 1.0 / q);
+  if (!(q >= 1.0 && q <= kSquaringMaxQ) || q != floor(q) || !(S > 1e-30 && S < 1e30)) return pow(S, 1.0 / q);
   double x = double(powf(float(S), float(1.0 / q)));
 #pragma unroll 1
   for (int k = 0; k < 2; ++k) {
