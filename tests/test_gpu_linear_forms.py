@@ -34,6 +34,26 @@ def _problem(K, n, seed=0):
     return normals, v * 1.01, C1, C2
 
 
+def _grad(K, normals, v, C1, C2, Ct, **kw):
+    from paper_2109_14403_gb300.linear import DMNLinear
+    d = DMNLinear(K, normals, v, device=torch.device("cuda:0"))
+    loss = d.loss_grad(C1, C2, Ct, penalty=10.0, **kw).clone()
+    return float(loss[1].item()), d.grad.clone(), d
+
+
+@pytest.mark.parametrize("K,n", [(2, 129), (3, 300), (4, 1), (4, 128), (4, 129), (5, 127), (5, 2048), (5, 2049), (6, 2049),
+                                 (7, 128), (7, 129), (7, 300), (8, 127), (8, 129), (8, 2048), (8, 2049)])
+def test_fp32_levels_against_fp64(K, n):
+    from paper_2109_14403_gb300.linear import DMNLinear
+    normals, v, C1, C2 = _problem(K, n)
+    C1, C2 = _t(C1), _t(C2)
+    Ct = DMNLinear(K, *syn.linear_params(K, seed=400 + K), device=C1.device).forward(C1, C2)
+    J, g, _ = _grad(K, normals, v, C1, C2, Ct, precision="fp64")
+    J32, g32, _ = _grad(K, normals, v, C1, C2, Ct, precision="fp32")
+    assert abs(J32 - J) <= TOL["fp32"][0] * J
+    assert float((g32 - g).abs().max()) <= TOL["fp32"][1] * float(g.abs().max())
+
+
 @functools.lru_cache(maxsize=None)
 def _oracle(K, n, p, q):
     normals, v, C1, C2 = _problem(K, n, seed=1)
