@@ -36,7 +36,6 @@ namespace mlp {
 constexpr int BM = 128, BN = 128, BK = 64, STAGES = 3;
 constexpr int TILE_A = BM * BK * 2, TILE_B = BN * BK * 2;  // bytes per stage
 constexpr int GEMM_SMEM = STAGES * (TILE_A + TILE_B) + 1024 + 256;
-static_assert(BM * (BN + 1) * 4 <= STAGES * (TILE_A + TILE_B), "staged FP32 tile fits the ring");
 constexpr long long kWaitCycles = 4000000000ll;  // ~2 s at 2 GHz
 
 enum Epi {
@@ -368,13 +367,15 @@ __device__ __forceinline__ void gemm_tile_body(const CUtensorMap &map_a, const C
     }
     if (ep.mode == EPI_BIAS_F32) {
       // de-normalised prediction on valid rows and columns: the warp writes
-      // its 32 staged rows, lane l on columns l, l+32, l+64, l+96
+      // its 32 staged rows, lane l on columns l, l + 32, ..
+      static_assert(BM * (BNT + 1) * 4 <= NST * (TILE_A + TB), "staged FP32 tile fits the ring");
+      constexpr int NC = BNT / 32;
       __syncwarp();
       const float *tile = reinterpret_cast<const float *>(base);
-      float bb[4], sc[4], sh[4];
-      bool cv[4];
+      float bb[NC], sc[NC], sh[NC];
+      bool cv[NC];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < NC; ++q) {
         const int n = n0 + lane + 32 * q;
         cv[q] = n < ep.n_valid;
         bb[q] = cv[q] ? ep.bias[n] : 0.0f;
@@ -386,8 +387,8 @@ __device__ __forceinline__ void gemm_tile_body(const CUtensorMap &map_a, const C
         if (rg >= ep.m_valid) break;
         float *dst = ep.f_out + size_t(rg) * ep.ld_f + n0 + lane;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (cv[q]) dst[32 * q] = (tile[row * (BN + 1) + lane + 32 * q] + bb[q]) * sc[q] + sh[q];
+        for (int q = 0; q < NC; ++q)
+          if (cv[q]) dst[32 * q] = (tile[row * (BNT + 1) + lane + 32 * q] + bb[q]) * sc[q] + sh[q];
       }
     }
   }
