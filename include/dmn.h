@@ -173,7 +173,8 @@ void dmn_default_options(dmn_options *opt);
 
 /*
  * Create a DMN handle (Sec. 3.1 tree; Sec. 4 phase laws).
- *   K          tree depth, 1..10 (2^K leaves, 2^K - 1 laminates).
+ *   K          tree depth, 1..10 (2^K leaves, 2^K - 1 laminates); 10 in mixed
+ *              precision only.
  *   leaf_w     host, 2^K weights w_{K+1}^i, each > 0, summing to 1 within
  *              1e-12 (Sec. 3.1 constraint; zero weights are rejected).
  *   normals    host, (2^K - 1) x 3 lamination directions in the paper's

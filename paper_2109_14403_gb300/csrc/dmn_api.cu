@@ -287,6 +287,8 @@ extern "C" dmn_status dmn_create(dmn_handle *out, int32_t K, const double *leaf_
   int zw = lay.zw;
   if (law == 2 && K > 9) return fail(DMN_ERR_ARG, "dmn_create: Perzyna leaves need K <= 9 (K=%d)", K);
   if (law == 3 && K > 8) return fail(DMN_ERR_ARG, "dmn_create: PA66 leaves need K <= 8 (K=%d)", K);
+  if (K > 9 && o.precision != DMN_PREC_MIXED)
+    return fail(DMN_ERR_ARG, "dmn_create: K=%d does not fit one SM in the requested precision", K);
   if (law == 3) zw = lay.hw;  // the solve keeps the leaves' history, not z, in shared memory
   if (is_warp_variant(o.solve_variant) && !warp_form_supports(K, o.precision == DMN_PREC_MIXED, law))
     return fail(DMN_ERR_ARG,

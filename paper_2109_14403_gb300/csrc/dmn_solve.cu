@@ -445,29 +445,30 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_kernel(const SolveParams
   }
 }
 
-static size_t owner_smem_bytes(int K, int zw, int n_mats, bool mixed) {
+static size_t owner_smem_bytes(int K, int zw, int n_mats) {  // mixed
   const int N = (1 << K) - 1, G = 1 << (K - 1);
   const int nslot = G >= 64 ? G / 64 : 1;
-  const size_t hp = 8;  // double or float-float
+  const size_t hp = 8;  // float-float
   size_t b = hp * (3 * N + 9 * G + 2 * zw + 12 + 64 + 4) + sizeof(double) * (nslot * kRecWords);
-  b += (mixed ? sizeof(MatPt<float, dfl>) : sizeof(MatPt<double, double>)) * n_mats;
+  b += sizeof(MatPt<float, dfl>) * n_mats;
   b = (b + 15) & ~size_t(15);
-  b += mixed ? sizeof(Ctrl<float>) : sizeof(Ctrl<double>);
-  b += (mixed ? sizeof(float) : sizeof(double)) * (32 + 40 + 24 * N + 3 * (G >= 2 ? G / 2 : 1));
+  b += sizeof(Ctrl<float>);
+  b += sizeof(float) * (32 + 40 + 24 * N + 3 * (G >= 2 ? G / 2 : 1));
   return (b + 15) & ~size_t(15);
 }
 
 // kernel variants: (form, precision, threads bound, CTAs per SM requested).
 // FP64, K <= 9: the compact kernel, whatever the variant (the owner-mapped form
 // has each level's nodes on one lane per warp or less, and an FP64 warp
-// instruction costs the same however few lanes are active: 1.4 to 2.0 times
-// the time at every K = 3..8, from 32 to 65,536 points; 2.8 times at K = 9, 64 to
-// 8,192 points).  Mixed: 0 = default; 2..4 = owner-mapped kernel for that many
-// CTAs per SM; 10 + m = compact kernel (dmn_solve_compact.cu) compiled for m =
-// 2, 3 or 4 CTAs per SM (11 runs as 12).  Deeper trees take the owner-mapped 512-thread kernel.  A tree with
-// Perzyna leaves (law 2) always takes the compact instances that include that
-// leaf law (dmn_solve_compact_vp.cu, K <= 9), whatever the variant; one with
-// PA66 leaves (law 3) the instances of dmn_solve_compact_pa66.cu (K <= 8).
+// instruction costs the same however few lanes are active: 1.4 to 2.6 times
+// the time at every K = 1..8, from 16 to 65,536 points; 2.8 times at K = 9, 16 to
+// 8,192 points); K = 10 fits no SM.  Mixed: 0 = default; 2..4 = owner-mapped kernel
+// for that many CTAs per SM; 10 + m = compact kernel (dmn_solve_compact.cu)
+// compiled for m = 2, 3 or 4 CTAs per SM (11 runs as 12); deeper trees take the
+// owner-mapped 512-thread kernel.  A tree with Perzyna leaves (law 2) always
+// takes the compact instances that include that leaf law
+// (dmn_solve_compact_vp.cu, K <= 9), whatever the variant; one with PA66 leaves
+// (law 3) the instances of dmn_solve_compact_pa66.cu (K <= 8).
 // A mixed launch of at most two CTAs per SM that fills at most half of what the
 // SMs hold of it (`few`) takes its form's instance for two: the same operations
 // with more registers (compact 254 against 168 with 80 bytes of spills, owner 245
@@ -499,7 +500,7 @@ static KernelFn pick(int K, bool mixed, int variant, int law, bool few) {
   if (law == 3) return compact_kernel_pa66(K, mixed);
   if (law >= 2 || (!mixed && K == 9)) return compact_kernel_vp(K, mixed);
   if (is_compact(K, mixed, variant, law)) return compact_kernel(K, mixed, few ? 2 : variant - 10);
-  if (K > 8) return mixed ? dmn_solve_kernel<float, dfl, 512, 1> : dmn_solve_kernel<double, double, 512, 1>;
+  if (K > 8) return dmn_solve_kernel<float, dfl, 512, 1>;
   switch (few ? 2 : variant) {
     case 2: return dmn_solve_kernel<float, dfl, 128, 2>;
     case 4: return dmn_solve_kernel<float, dfl, 128, 4>;
@@ -511,7 +512,7 @@ size_t solve_smem_bytes(int K, int zw, int n_mats, bool mixed, int variant, int 
   if (uses_warp_form(K, mixed, variant, law)) return warp_smem_bytes(K, n_mats);
   if (law == 3) return compact_smem_bytes_pa(K, zw, n_mats, mixed);
   return is_compact(K, mixed, variant, law) ? compact_smem_bytes(K, zw, n_mats, mixed)
-                                     : owner_smem_bytes(K, zw, n_mats, mixed);
+                                            : owner_smem_bytes(K, zw, n_mats);
 }
 
 // One kernel instance serves every tree of a depth range (the compact instances

@@ -1293,7 +1293,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
                                    full, k == 1);
           }
         }
-      } else if (K == 3) {
+      } else if (!D64 && K == 3) {
         __syncwarp(mask);
         if (t == 0) {
           const int p = (1 << K) - 2;
@@ -1319,8 +1319,7 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
                             tf_of(rh[2], (TF *)nullptr)};
           r2 += rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
           const TF rbv[3] = {rv[0] * iwcc, rv[1] * iwcc, rv[2] * iwcc};
-          if constexpr (D64) combine_d(rec, other, nd, rbv, gh_s + 21 * p, full);
-          else combine<TF>(rec, other, n, c1, c2, rbv, gh_s + 21 * p, full);
+          combine<TF>(rec, other, n, c1, c2, rbv, gh_s + 21 * p, full);
           put_root(rec, S);
         }
       }
