@@ -176,18 +176,33 @@ __device__ __forceinline__ float f32_rn(double d) {
   r += (lo & 0x1fffffffu) + (r & 1u) > 0x10000000u ? 1u : 0u;  // to nearest, ties to even; a carry moves into the exponent
   return __uint_as_float(sign | r);
 }
+// The same result without a call and by branches, for the rows read word by word:
+// bound by their half-sector loads, they lose more to the call's registers than to
+// the FP64 pipe (65,536 rows at K = 8, states 8 bytes off: 208 us, 225 with the call)
+__device__ __forceinline__ float f32_rn_inline(double d) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(d));
+  const unsigned E = unsigned(b >> 52) & 0x7ffu, sign = unsigned(b >> 32) & 0x80000000u;
+  if (E == 0u) return __uint_as_float(sign);
+  if (E < 897u || E > 1150u) return __double2float_rn(d);
+  const unsigned long long mant = b & ((1ull << 52) - 1);
+  unsigned r = sign | ((E - 896u) << 23) | unsigned(mant >> 29);
+  const unsigned rem = unsigned(mant & ((1ull << 29) - 1)), half = 1u << 28;
+  if (rem > half || (rem == half && (r & 1u))) r += 1u;  // a carry moves into the exponent
+  return __uint_as_float(r);
+}
 
 // feature c of a row: deps (6), theta^{n+1}, theta^{n+1} - theta^n,
 // a^n - a^{n-1} (n3) as the difference of the two words rounded to float;
 // a = the state block at t^n, ap = at t^{n-1} or NULL (its columns 0)
 constexpr int kExtraFeatures = 0;
+template <float (*RN)(double) = f32_rn>
 __device__ __forceinline__ float feature(int c, int n3, const double *dep, double th, const double *a,
                                          const double *ap) {
   (void)n3;
-  if (c < 6) return f32_rn(dep[c]);
-  if (c == 6) return f32_rn(th);
+  if (c < 6) return RN(dep[c]);
+  if (c == 6) return RN(th);
   if (c == 7) return float(th - a[6]);
-  return ap ? f32_rn(a[c]) - f32_rn(ap[c]) : 0.0f;  // a^n - a^{n-1}: state words 8..
+  return ap ? RN(a[c]) - RN(ap[c]) : 0.0f;  // a^n - a^{n-1}: state words 8..
 }
 
 __global__ void k_features(int64_t n, int n3, int sw, const double *deps, const double *theta,
@@ -204,11 +219,14 @@ __global__ void k_features(int64_t n, int n3, int sw, const double *deps, const 
 // features of k_features, normalised and rounded to bf16 in one pass: one
 // warp per row, each lane two adjacent columns per step (one bf16x2 store;
 // ld = kin is a multiple of 128, so the pairs stay 4-byte aligned).  Bound by the
-// two states' jumps it reads (12 KB a row at K = 8).  VEC: a lane's pair of jumps
-// as one 16-byte load, two steps in flight (states 16-byte aligned, an even
-// number of words; 65,536 rows 166 us, one step 173, four 178, seven 193); else
-// word by word (180).
-template <bool VEC>
+// two states' jumps it reads (12 KB a row at K = 8).  Three instances, chosen by
+// the call: 16-byte loads of a lane's pair of jumps, two steps in flight (states
+// 16-byte aligned, an even number of words; 65,536 rows 166 us, one step 173, four
+// 178, seven 193); word by word (aligned 180, 8 bytes off 208); no previous state
+// (65,536 rows at K = 8 a call 76 us, 86 inside the instance for two states, whose
+// registers keep half of the warps out).
+enum { ROWS_FIRST, ROWS_WORDS, ROWS_VEC };  // no previous state; word by word; 16-byte loads
+template <int MODE>
 __global__ void __launch_bounds__(256)
     k_features_norm(int64_t n, int n3, int sw, int ld, const double *deps, const double *theta, const double *sin,
                     const double *sprev, const float *mean, const float *inv, bf16 *x) {
@@ -217,7 +235,7 @@ __global__ void __launch_bounds__(256)
   const int64_t nwarp = (int64_t(gridDim.x) * blockDim.x) >> 5;
   for (int64_t r = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; r < n; r += nwarp) {
     const double *a = sin + r * sw;
-    const double *ap = sprev ? sprev + r * sw : nullptr;
+    const double *ap = MODE == ROWS_FIRST ? nullptr : sprev + r * sw;
     __nv_bfloat162 *xr = reinterpret_cast<__nv_bfloat162 *>(x + r * ld);
     auto put = [&](int c0, float f0, float f1) {  // features of columns c0, c0 + 1
       float v0 = 0.0f, v1 = 0.0f;
@@ -225,7 +243,7 @@ __global__ void __launch_bounds__(256)
       if (c0 + 1 < nin) v1 = (f1 - __ldg(mean + c0 + 1)) * __ldg(inv + c0 + 1);
       xr[c0 >> 1] = __floats2bfloat162_rn(v0, v1);
     };
-    if (VEC && ap) {
+    if constexpr (MODE == ROWS_VEC) {
       constexpr int U = 2;
       for (int c0 = 2 * lane; c0 < ld; c0 += 64 * U) {
         double2 q[U], p[U];
@@ -250,6 +268,15 @@ __global__ void __launch_bounds__(256)
             put(c, f32_rn(q[u].x) - f32_rn(p[u].x), f32_rn(q[u].y) - f32_rn(p[u].y));
           }
         }
+      }
+    } else if constexpr (MODE == ROWS_WORDS) {
+      for (int c0 = 2 * lane; c0 < ld; c0 += 64) {
+        float v[2] = {0.0f, 0.0f};
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (c0 + u < nin)
+            v[u] = (feature<f32_rn_inline>(c0 + u, n3, deps + r * 6, theta[r], a, ap) - mean[c0 + u]) * inv[c0 + u];
+        xr[c0 >> 1] = __floats2bfloat162_rn(v[0], v[1]);
       }
     } else {
       for (int c0 = 2 * lane; c0 < ld; c0 += 64) {
@@ -651,7 +678,9 @@ extern "C" dmn_status dmn_mlp_input(dmn_mlp m, dmn_stream stream, int64_t n, con
   if (n == 0) return DMN_OK;
   const bool vec = ((reinterpret_cast<uintptr_t>(d_state_in) | reinterpret_cast<uintptr_t>(d_state_prev)) & 15) == 0 &&
                    (state_words & 1) == 0;
-  (vec ? k_features_norm<true> : k_features_norm<false>)<<<blocks_for(n * 32), 256, 0, (cudaStream_t)stream>>>(
+  const auto f = !d_state_prev ? k_features_norm<ROWS_FIRST>
+                               : (vec ? k_features_norm<ROWS_VEC> : k_features_norm<ROWS_WORDS>);
+  f<<<blocks_for(n * 32), 256, 0, (cudaStream_t)stream>>>(
       n, m->n3, int(state_words), m->kin, d_deps, d_theta, d_state_in, d_state_prev, m->fmean,
       m->finv, static_cast<bf16 *>(d_x_bf16));
   cudaError_t e = cudaGetLastError();
