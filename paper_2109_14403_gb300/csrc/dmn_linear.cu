@@ -1061,13 +1061,27 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   T *nh = consts, *c1s = consts + 3 * N;
   const unsigned ns = unsigned((n + kSetupThreads / 2 - 1) / (kSetupThreads / 2));
   cudaError_t e = cudaSuccess;
-  // a small batch's launches overlap (its kernels last little longer than their
-  // launch: 32 samples, K = 8: 107 -> 93 us with the eight-lane kernels); a large
-  // one's do not (65,536 samples: early CTAs of the next level cost 4 %)
-  const bool small = n <= 2048;
+  // Up to 2,048 samples the error and seed kernels take eight lanes a sample
+  // (general powers, K = 5, 2,048 samples: 205 us a step, 560 with one), and a small
+  // batch's launches overlap: its kernels last little longer than their launch (with
+  // the lanes 107 -> 93 us at K = 8, 32 samples).  Where a batch fills the chip, early
+  // CTAs of the next launch keep out those of the one that runs.  Steps that overlap
+  // against steps that do not, us:
+  //   FP32, p = 1, 2: 512 samples at K = 3, 5, 8 84, 107, 131 to 105, 119, 142; 2,048
+  //     95, 114, 165 to 106, 123, 167; 4,096 101, 135, 205 to 105, 122, 204
+  //   FP64: 512 at K = 3, 5 209, 316 to 223, 332, 64 at K = 8 438 to 462; but 1,024 at K = 5
+  //     394 to 331, 512 at K = 6 416 to 384, 256 at K = 8 613 to 539
+  //   general powers, FP32: 768 at K = 3 181 to 191, 512 at K = 5 201 to 207, 64 at K = 8
+  //     197 to 206; but 2,048 at K = 3 273 to 191, 256 and 2,048 at K = 8 314 to 228, 616 to 251
+  // So by the bottom laminates (256 warps of them), and for exact powers in FP32 up
+  // to 2,048 samples whatever the depth.
+  const bool lanes8 = n <= 2048;
+  const int mode = pow_mode(p);
+  const bool few = (n << (K - 1)) <= 8192;
+  const bool overlap = mode == 0 ? few && n < 1024 : (sizeof(T) == 4 ? n <= 2048 : few && n <= 2048);
   const bool split = n <= kLvlThreads;  // a block of samples: at most 2^(K-2) CTAs a launch
   auto go = [&](auto f, dim3 grid, unsigned threads, auto... args) {
-    if (e == cudaSuccess) e = launch_chained(small, f, grid, dim3(threads), 0, st, args...);
+    if (e == cudaSuccess) e = launch_chained(overlap, f, grid, dim3(threads), 0, st, args...);
   };
   go(k_lvl_setup<T>, dim3(2 + ns), kSetupThreads, K, n, normals, v, C1, C2, nh, c1s, PH, gnh, 4 * N + 5);
   // FP32: pairs of levels from the bottom (FP64 laminates: 251 registers for one
@@ -1082,8 +1096,7 @@ dmn_status lin_train_pass(cudaStream_t st, int K, int64_t n, const double *C1, c
   for (; k >= 1; --k) go(k_lvl_fwd<T>, dim3(nb, 1u << (k - 1)), kLvlThreads, K, k, n, PH, nh, c1s, NS);
   // the blocks' partial sums: in the adjoints' array, free until the seed, from an 8-byte boundary
   double *part = reinterpret_cast<double *>((reinterpret_cast<uintptr_t>(GA) + 7) & ~uintptr_t(7));
-  const int mode = pow_mode(p);
-  if (small) {  // eight lanes a sample: at most 128 CTAs
+  if (lanes8) {  // at most 128 CTAs
     const unsigned nb8 = unsigned((8 * n + kLvlThreads - 1) / kLvlThreads);
     go(mode == 1 ? k_lvl_err<1, 8, T> : mode == 2 ? k_lvl_err<2, 8, T> : k_lvl_err<0, 8, T>, dim3(nb8), kLvlThreads,
        K, n, NS, Ct, p, q, err, part, scal);

@@ -77,3 +77,23 @@ def test_exponents_in_small_and_large_batches(p, q, r, prec):
     g = d.grad.cpu().numpy()
     ref = f * np.concatenate([gn.reshape(-1), gv])
     assert np.abs(g - ref).max() <= tg * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("p", [1.0, 1.5])
+@pytest.mark.parametrize("K,n", [(5, 512), (3, 1023), (8, 64)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_overlapped_and_ordinary_launches_agree(K, n, p, prec):
+    """n samples fill what overlaps, twice as many do not (FP64, or a general
+    power): the batch twice over scales J and its gradient by 2^(1/q - 1)."""
+    from paper_2109_14403_gb300.linear import DMNLinear
+    q = 3.0
+    normals, v, C1, C2 = _problem(K, n, seed=2)
+    C1, C2 = _t(C1), _t(C2)
+    Ct = DMNLinear(K, *syn.linear_params(K, seed=402), device=C1.device).forward(C1, C2)
+    d = DMNLinear(K, normals, v, device=C1.device)
+    J = d.loss_grad(C1, C2, Ct, p=p, q=q, penalty=0.0, precision=prec).clone()
+    g, f = d.grad.clone(), 2.0 ** (1.0 / q - 1.0)
+    J2 = d.loss_grad(*[torch.cat([x, x]).contiguous() for x in (C1, C2, Ct)], p=p, q=q, penalty=0.0, precision=prec)
+    tl, tg = TOL[prec]
+    assert abs(float(J2[0]) - f * float(J[0])) <= tl * f * float(J[0])
+    assert float((d.grad - f * g).abs().max()) <= tg * f * float(g.abs().max())
