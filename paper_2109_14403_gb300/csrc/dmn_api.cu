@@ -282,7 +282,7 @@ extern "C" dmn_status dmn_create(dmn_handle *out, int32_t K, const double *leaf_
   if (build_tree_tables(K, leaf_w, normals, phase_map, mats, n_mats, mat.data(), node.data(),
                         node_df.data(), zoff.data(), hoff.data(), wscr.data(), &lay, why, sizeof(why)))
     return fail(DMN_ERR_ARG, "dmn_create: %s", why);
-  if (!(o.res_floor > 0.0)) o.res_floor = 1e-8 * lay.Emax;
+  o.res_floor = residual_floor(o, lay.Emax);
   const int law = lay.law, zend = lay.zend, off = lay.SW;
   int zw = lay.zw;
   if (law == 2 && K > 9) return fail(DMN_ERR_ARG, "dmn_create: Perzyna leaves need K <= 9 (K=%d)", K);

@@ -1,6 +1,7 @@
 // dmn_internal.h -- declarations shared by the library's translation units.
 #pragma once
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stddef.h>
 
 #include "../../include/dmn.h"
@@ -57,6 +58,12 @@ KernelFn warp_kernel8(int minb);
 // threads per CTA of the kernel a variant selects
 int solve_block_threads(int K, bool mixed, int variant, int law);
 int compact_block_threads64(int K);  // ... of the compact kernel's FP64 instances
+// the floor of |sigma_bar| the solve uses: the caller's, or the default; mixed forms
+// hold it in FP32, where a smaller one would be no floor (0 / 0 without stress)
+inline double residual_floor(const dmn_options &o, double Emax) {
+  const double f = o.res_floor > 0.0 ? o.res_floor : 1e-8 * Emax;
+  return o.precision == DMN_PREC_MIXED && f < double(FLT_MIN) ? double(FLT_MIN) : f;
+}
 // resident CTAs per SM of the kernel a variant selects, and of its instance for
 // small launches (0: there is none)
 struct Residency {

@@ -111,7 +111,7 @@ extern "C" dmn_status dmn_eval_noalloc(int32_t K, const double *leaf_w, const do
     return na_fail(DMN_ERR_ARG, "dmn_eval_noalloc: %s", why);
   if (lay.law == 3)
     return na_fail(DMN_ERR_ARG, "dmn_eval_noalloc: PA66 leaves (kind 3) need a dmn_handle");
-  if (!(o.res_floor > 0.0)) o.res_floor = 1e-8 * lay.Emax;
+  o.res_floor = residual_floor(o, lay.Emax);
   const int law = lay.law, zend = lay.zend, zw = lay.zw, SW = lay.SW;
   const size_t sbytes = sizeof(double) * (size_t)SW * (size_t)n_points;
   const char *sa = (const char *)d_state_in, *sb = (const char *)d_state_out;

@@ -37,3 +37,17 @@ def test_points_without_stress_converge_whatever_the_floor_fp64(K, floor):
     assert (it[:n // 2] == 1).all() and (out[:n // 2, :6] == 0.0).all()
     for a, b in ((s, s0), (out, out0), (it, it0)):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("K", [1, 3, 4, 6, 8, 9])
+@pytest.mark.parametrize("floor", [1e-30, 1e-50, 1e-300])
+def test_points_without_stress_converge_whatever_the_floor_mixed(K, floor):
+    """The mixed forms hold the floor in FP32: below its range it was zero."""
+    n = 12
+    s, out, st, it = _eval(K, "mixed", floor, n)
+    s0, out0, st0, it0 = _eval(K, "mixed", 0.0, n)
+    assert (st0 == 0).all()
+    assert (st == 0).all(), st
+    assert (it[:n // 2] == 1).all() and (out[:n // 2, :6] == 0.0).all()
+    for a, b in ((s, s0), (out, out0), (it, it0)):
+        assert np.array_equal(a, b)
