@@ -13,7 +13,7 @@ constexpr int kUpdThreads = 32, kWorkThreads = 128;
 // constant after unrolling; rows are exchanged by selects); false when a pivot
 // vanishes.  Pivots by the leading 32 bits of the magnitudes (integer
 // comparisons; an FP64 instruction takes 64 cycles of a warp here), one
-// reciprocal per column: about 300 FP64 instructions a point.  (With the
+// reciprocal per column: 161 operations and seven divisions a point.  (With the
 // system in local memory and a division per row the 4,096-point predictor took
 // 44 us.)
 template <int k>

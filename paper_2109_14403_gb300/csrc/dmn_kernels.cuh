@@ -252,7 +252,7 @@ struct LeafTan {
 // quantities (D, X and the record's tau, dd, gg) are left at zero.  PARTS
 // (FP64): the tangent goes to *tan by its parts, not into the record (whose ds
 // is not set either), and the plastic step takes one rsqrt in place of two
-// square roots and two divisions, each some 25 FP64 instructions.
+// square roots and two divisions.
 template <typename TF, typename HP, int LAW, bool PARTS = false>
 __device__ __forceinline__ void leaf_eval(const MatPt<TF, HP> &m, const HP eps[6], const HP *zn,
                                           HP trn, HP sig[6], HP &D, HP &X, Rec<TF> &R, HP *znew,

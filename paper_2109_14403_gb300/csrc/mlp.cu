@@ -1,7 +1,7 @@
-// mlp.cu -- the warm-start network of include/dmn_mlp.h: tensor maps, the
-// tcgen05 GEMM launches of the forward and backward passes, and the small
-// memory-bound kernels around them (features, normalisation, loss, bias
-// gradients, AMSGrad, weight packing, transposes).
+// mlp.cu -- the warm-start network of include/dmn_mlp.h: tensor maps, the choice
+// and launch of the tcgen05 GEMMs of the forward and backward passes (the bias
+// gradients and the loss ride with them), and the memory-bound kernels around
+// them (features, normalisation, AMSGrad with the weight packing).
 #include <cudaTypedefs.h>
 #include <math.h>
 #include <stdarg.h>

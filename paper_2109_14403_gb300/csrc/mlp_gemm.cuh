@@ -1,18 +1,22 @@
-// mlp_gemm.cuh -- BF16 tensor-core GEMM for the warm-start MLP on sm_103a:
-//   C[M x N] = A[M x K] . B[N x K]^T   (A, B bf16 with K contiguous; FP32
-//   accumulation in tensor memory), followed by a fused epilogue.
+// mlp_gemm.cuh -- BF16 tensor-core GEMMs for the warm-start MLP on sm_103a: FP32
+// accumulation in tensor memory, a fused epilogue.  C[M x N] = A[M x K] . B[N x K]^T
+// with K contiguous; the tile form also takes an operand with M or N contiguous
+// (the backward pass's, as stored).
 //
-// Two forms.  The persistent wide form (below, gemm_bf16_tn_wide) serves N a
-// multiple of 256; the tile form serves every other shape (N a multiple of
-// 128).  Tile form: one CTA of 128 threads computes a 128 x 128 tile (grid:
-// column tiles fastest); two CTAs share an SM, so one's epilogue overlaps the
-// other's MMAs:
+// Two forms, chosen by gemm() in mlp.cu.  The persistent wide form (below,
+// gemm_bf16_tn_wide: 128 x 256 tiles) serves inference and plain products of N a
+// multiple of 256 with tiles enough for the SMs; the tile form serves everything
+// else: other N (a multiple of 128), small products, and all of a training step.
+// Tile form: one CTA of 128 threads computes a tile of 128 rows and 128 columns from
+// a ring of three stages, or of 64 columns from four (short products and the
+// weight gradients); grid: column tiles fastest; two CTAs share an SM, so one's
+// epilogue overlaps the other's MMAs:
 //   warp 0, lane 0  loads A and B tiles (64 wide in K) with TMA bulk tensor
-//                   copies into a 3-stage ring of 128-byte-swizzled shared
-//                   memory, signalled by mbarriers with transaction counts;
-//   warp 1          allocates 128 TMEM columns; its lane 0 issues
-//                   tcgen05.mma (kind::f16, BF16 x BF16 -> F32, M=128,
-//                   N=128, K=16 per instruction) and releases each stage with
+//                   copies into the ring of 128-byte-swizzled shared memory,
+//                   signalled by mbarriers with transaction counts;
+//   warp 1          allocates a TMEM column per tile column; its lane 0 issues
+//                   tcgen05.mma (kind::f16, BF16 x BF16 -> F32, M = 128, the
+//                   tile's N, K = 16 per instruction) and releases each stage with
 //                   tcgen05.commit on that stage's "empty" mbarrier;
 //   all 4 warps     wait for the final commit, read the accumulator with
 //                   tcgen05.ld (warp w owns TMEM lanes 32w..32w+31 = tile rows)
@@ -504,8 +508,8 @@ __global__ void __launch_bounds__(128, 2) gemm_bf16_wgrad(const __grid_constant_
 }
 
 // ---------------------------------------------------------------- wide form
-// Persistent form for N a multiple of 256 (the network's forward layers: N =
-// 512 or 768): one CTA per SM loops over 128 x 256 tiles (column tiles
+// Persistent form for N a multiple of 256 (inference: the network's layers have N
+// = 512 or 768): one CTA per SM loops over 128 x 256 tiles (column tiles
 // fastest, so the CTAs sharing an A panel run together and read it from L2).
 // Warps with fixed roles:
 //   warp 0, lane 0  TMA producer: A (128 x 64) and B (256 x 64) of each K step

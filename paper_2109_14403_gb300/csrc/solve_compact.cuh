@@ -200,7 +200,9 @@ __device__ __forceinline__ void combine_rows(const SolveParams &P, int p, int r,
 // ---- the condensation in FP64 (combine() of dmn_kernels.cuh with fewer
 // operations): with dC = C_L - C_R, U = dC B and c1 + c2 = 1,
 //   K = B^T C_R B + c2 B^T U,  C_hat = C_R + c1 dC - U (c1 c2 G),
-// and B's zeros left out.  About 400 FP64 instructions per node, against 500.
+// and B's zeros left out.  Operations of a node, counted in the source (a fused
+// multiply-add as one, the output terms left out, and a division each): combine_d
+// 397, combine() 500; combine_leaves 216 with elastic leaves, 285 with a plastic one.
 
 // K^-1 of the symmetric K = (k00, k01, k02, k11, k12, k22)
 __device__ __forceinline__ void inv_sym3(const double k[6], double Ki[3][3]) {
@@ -422,8 +424,8 @@ __device__ __forceinline__ void combine_node(const SolveParams &P, int p, const 
   rec_put(dst, L);
 }
 
-// A node on eight lanes (combine_rows' mapping) with these formulas: 130 FP64
-// instructions, against 161
+// A node on eight lanes (combine_rows' mapping) with these formulas: 123
+// operations a lane, 154 with combine_rows' (counted as above)
 __device__ __forceinline__ void combine_rows64(const SolveParams &P, int p, int r, bool st, unsigned mask,
                                                const double *rcL, const double *rcR, const double *sL,
                                                const double *sR, double *dst, double *sdst, double *gh, double &r2,
@@ -508,7 +510,7 @@ __device__ __forceinline__ void combine_rows64(const SolveParams &P, int p, int 
 // 3h .. 3h + 2.  Sums over rows (K, the right-hand sides) are halves added by a
 // shuffle; of C_hat a lane forms its own 3 x 3 block's upper triangle and, of
 // the 3 x 3 block between the lanes, the pairs (own r, other o) with r <= o (both
-// form the diagonal).  About 300 FP64 instructions a lane.
+// form the diagonal).  290 operations a lane, counted as above.
 __device__ __forceinline__ void combine_half(const SolveParams &P, int p, int h, bool st, unsigned mask,
                                              const double *rcL, const double *rcR, const double *sL,
                                              const double *sR, double *dst, double *sdst, double *gh, double &r2,
@@ -1333,7 +1335,9 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
       //      level, so the parked values are there.  (K = 7 uneven -3 %, one
       //      element -3 %, K = 9 -1.5 %, warm K = 8 -1.6 %, ramp -0.8 %.  Not where
       //      it lost: FP64, whose other warps share the FP64 pipe, +1.3 %;
-      //      Perzyna trees of K <= 8, +2 % of the cyclic workload.) ----
+      //      Perzyna trees of K <= 8, +2 % of the cyclic workload, with an instance
+      //      that spills 360 bytes.  The thresholds and these exceptions are a fit
+      //      to the workloads named, not a model.) ----
       constexpr bool EARLY = !D64 && (LAW == 1 || (LAW == 2 && MAXT > 128));
       stored = EARLY && full && nwarp > 1 && ctrl->res_old < tol * (P.da0 ? TF(1e7) : TF(1e4));
       if (stored && warp != L) store_state(((warp - L - 1) & (nwarp - 1)) * 32 + lane, 32 * (nwarp - 1));
@@ -1429,8 +1433,8 @@ __global__ void __launch_bounds__(MAXT, MINB) dmn_solve_compact(const SolveParam
           bool on_rows = false;
           if constexpr (D64) {
             // a node on eight lanes: component e of da on lane e < 3, Mandel
-            // component c of B da and of the children on lane c < 6 (10 FP64
-            // instructions a round of four nodes, against 42)
+            // component c of B da and of the children on lane c < 6 (10
+            // operations a round of four nodes; a node on one lane takes 42)
             on_rows = k <= 4;
             if (on_rows && warp == L)
               step_rows64(P, k, lane, mask, k == 1 ? nullptr : tbuf(k), tbuf(k + 1), gh_s, da_s, a_s);
